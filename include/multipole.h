@@ -80,7 +80,9 @@ typedef enum {
 } mp_status;
 
 typedef enum {
-    MP_PREC_FP64 = 0,   /* every step in float64 on CUDA cores                       */
+    MP_PREC_FP64 = 0,   /* every step to float64 accuracy: the contractions as exact */
+                        /* integer slices on the tensor cores (l_max <= 71) or in    */
+                        /* float64 on CUDA cores, the rest in float64                */
     MP_PREC_BF16X3 = 1, /* angular contractions as split-bf16 tensor-core GEMMs,     */
                         /* density deviations in 2 bf16 terms, tables in 3           */
     MP_PREC_BF16X6 = 2  /* as BF16X3 with 3 bf16 terms on both operands              */

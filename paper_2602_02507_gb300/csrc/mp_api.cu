@@ -180,7 +180,7 @@ static void free_mesh_buffers(mp_mesh *m)
                     m->d_tabB, m->d_tabT, m->d_Aop, m->d_G0, m->phi_own, m->h_rho[0], m->h_rho[1],
                     m->h_phi[0], m->h_phi[1], m->d_err, m->d_gst, m->d_cwork, m->d_cweights, m->d_cgroups,
                     m->d_cchunks, m->d_cscratch, m->d_ccount, m->d_tabTh, m->d_tabGs, m->d_Cb, m->d_th_off,
-                    m->d_gs_off, m->d_cb_off, m->d_slab_off};
+                    m->d_gs_off, m->d_cb_off, m->d_slab_off, m->fp.arena};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &pe : m->prof_pending) {
@@ -474,6 +474,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
 
     const size_t nedges = (size_t)(n_r + 1) + (n_theta + 1) + (n_phi + 1);
     mp_status st;
+    if (m->eff_prec == MP_PREC_FP64) plan_fp64_tc(m);
 #define ALLOC(ptr, count)                             \
     st = dalloc(m, &(ptr), (size_t)(count));          \
     if (st != MP_OK) return fail(st);
@@ -490,12 +491,19 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
     ALLOC(m->d_A, (size_t)n_r * m->KL);
     ALLOC(m->d_MR, (size_t)(n_r + 1) * m->KL);
     ALLOC(m->d_MI, (size_t)(n_r + 1) * m->KL);
-    ALLOC(m->d_C, (size_t)n_r * m->KL);
+    ALLOC(m->d_C, (size_t)(m->fp.on ? m->fp.ldI : n_r) * m->KL);
     ALLOC(m->d_err, 4);
     ALLOC(m->d_slab_off, (size_t)2 * m->KL);  // radial sums of the other slabs (slab meshes)  // [0] error word, [2..3] budget of the pipeline waits (int64, 0: default)
     if (m->eff_prec == MP_PREC_FP64) {
-        ALLOC(m->d_F64, (size_t)m->R * m->P);
-        ALLOC(m->d_G64, (size_t)m->R * m->P);
+        if (m->fp.on) {
+            ALLOC(m->d_F64, (size_t)n_r * m->P * m->fp.ldJ);
+            ALLOC(m->d_G64, (size_t)n_r * m->P * m->fp.ldJ);
+            m->fp.arena_bytes = fp64_tc_arena(m);
+            ALLOC(m->fp.arena, m->fp.arena_bytes);
+        } else {
+            ALLOC(m->d_F64, (size_t)m->R * m->P);
+            ALLOC(m->d_G64, (size_t)m->R * m->P);
+        }
     } else {
         st = plan_split(m);
         if (st != MP_OK) return fail(st);
@@ -568,6 +576,10 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         if (st != MP_OK) return fail(st);
         st = cuda_status(launch_tables(m), "build tables");
         if (st != MP_OK) return fail(st);
+        if (m->fp.on) {
+            st = cuda_status(launch_fp64_tc_tables(m), "build float64 digit tables");
+            if (st != MP_OK) return fail(st);
+        }
         if (m->eff_prec != MP_PREC_FP64) {
             st = cuda_status(launch_split_tables(m), "build split tables");
             if (st != MP_OK) return fail(st);

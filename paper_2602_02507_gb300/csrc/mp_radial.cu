@@ -75,6 +75,7 @@ __device__ __forceinline__ void write_cb(const CbOut &o, int i, int l, int p, fl
     if (o.terms == 3) *reinterpret_cast<__nv_bfloat16 *>(base + 2 * c_term) = __float2bfloat16_rn(r1 - __bfloat162float(h1));
 }
 
+// ldC: the coefficients C go out as [n_r][K_L] (0) or as [K_L][ldC], one moment's shells together.
 // One block per moment column q; thread t owns shells [t*chunk, (t+1)*chunk).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const double *__restrict__ WR,
@@ -82,7 +83,7 @@ __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const
                                              const double *__restrict__ GI, double *__restrict__ MR,
                                              double *__restrict__ MI, double *__restrict__ C,
                                              float *__restrict__ C32, float2 *__restrict__ C0, int n_r, int KL,
-                                             const CbOut cbo, const double *__restrict__ off)
+                                             const CbOut cbo, const double *__restrict__ off, size_t ldC)
 {
     __shared__ double wt[2][NT / 32];
     // the next kernel's blocks may start (and copy their tables) while this one runs
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const
         const double mr_hi = fma(wr[i], a, mr_lo);
         double c = fma(GI[(size_t)l * n_r + i], mr_lo + mr_hi, GR[(size_t)l * n_r + i] * (mi + mi_hi));
         if (m > 0) c += c;
-        if (C) C[(size_t)i * KL + q] = c;
+        if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = c;
         const float c32 = f64_to_f32_alu(c);
         if (C32) C32[(size_t)i * KL + q] = c32;
         if (C0 && p == 0) C0[(size_t)i * Lp1 + l] = f32_pair(c);
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(NT) k_scan_reg(const double *__restrict__ A, c
                                                  const double *__restrict__ GI, double *__restrict__ MR,
                                                  double *__restrict__ MI, double *__restrict__ C,
                                                  float *__restrict__ C32, float2 *__restrict__ C0, int n_r, int KL,
-                                                 const CbOut cbo, const double *__restrict__ off)
+                                                 const CbOut cbo, const double *__restrict__ off, size_t ldC)
 {
     __shared__ double wt[2][NT / 32];
     // the next kernel's blocks may start (and copy their tables) while this one runs
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(NT) k_scan_reg(const double *__restrict__ A, c
             MI[(size_t)i * KL + q] = ei[k];
             double c = fma(g2[k], er[k] + er[k + 1], g1[k] * (ei[k] + ei[k + 1]));
             if (m > 0) c += c;
-            if (C) C[(size_t)i * KL + q] = c;
+            if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = c;
             const float c32 = f64_to_f32_alu(c);
             if (C32) C32[(size_t)i * KL + q] = c32;
             if (C0 && p == 0) C0[(size_t)i * Lp1 + l] = f32_pair(c);
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
                                                     const double *__restrict__ GI, double *__restrict__ MR,
                                                     double *__restrict__ MI, double *__restrict__ C,
                                                     float *__restrict__ C32, float2 *__restrict__ C0, int n_r, int KL,
-                                                    const CbOut cbo, const double *__restrict__ off)
+                                                    const CbOut cbo, const double *__restrict__ off, size_t ldC)
 {
     constexpr int NW = 4 * NT / 32;
     __shared__ double wt[2][NW][4];
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
             MI[(size_t)i * KL + q] = ei[k];
             double cv = fma(__ldg(gi + i), er + er1, __ldg(gr + i) * (ei[k] + ei[k + 1]));
             if (m > 0) cv += cv;
-            if (C) C[(size_t)i * KL + q] = cv;
+            if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = cv;
             const float c32 = f64_to_f32_alu(cv);
             if (C32) C32[(size_t)i * KL + q] = c32;
             if (C0 && p == 0) C0[(size_t)i * Lp1 + l] = f32_pair(cv);
@@ -647,7 +648,7 @@ static void scan_reg_launch(mp_mesh *m, int want_f32)
 {
     launch_pdl(k_scan_reg<NT, CH>, dim3(m->KL), dim3(NT), 0, m->stream, m->d_A, m->d_WR, m->d_WI, m->d_GR, m->d_GI,
                m->d_MR, m->d_MI, scan_c(m, want_f32), scan_c32(m, want_f32), want_f32 ? m->d_C0 : nullptr, m->n_r,
-               m->KL, cb_out(m, want_f32), m->use_slab_off ? (const double *)m->d_slab_off : nullptr);
+               m->KL, cb_out(m, want_f32), m->use_slab_off ? (const double *)m->d_slab_off : nullptr, (size_t)m->fp.ldI);
 }
 
 // Shells per thread CH for NT threads per moment column; false when n_r > 16 NT.
@@ -700,7 +701,7 @@ static bool scan_q4_dispatch(mp_mesh *m, int want_f32)
     auto go = [&](auto kern) {
         launch_pdl(kern, dim3((m->KL + 3) / 4), dim3(512), 0, m->stream, m->d_A, m->d_WR, m->d_WI, m->d_GR, m->d_GI,
                    m->d_MR, m->d_MI, scan_c(m, want_f32), scan_c32(m, want_f32), want_f32 ? m->d_C0 : nullptr,
-                   m->n_r, m->KL, cb_out(m, want_f32), m->use_slab_off ? (const double *)m->d_slab_off : nullptr);
+                   m->n_r, m->KL, cb_out(m, want_f32), m->use_slab_off ? (const double *)m->d_slab_off : nullptr, (size_t)m->fp.ldI);
     };
     if (ch <= 4)
         go(k_scan_q4<128, 4>);
@@ -729,7 +730,7 @@ cudaError_t launch_scan(mp_mesh *m, int want_f32)
                                                                     scan_c32(m, want_f32),
                                                                     want_f32 ? m->d_C0 : nullptr, m->n_r, m->KL,
                                                                     cb_out(m, want_f32),
-                                                                    m->use_slab_off ? (const double *)m->d_slab_off : nullptr);
+                                                                    m->use_slab_off ? (const double *)m->d_slab_off : nullptr, (size_t)m->fp.ldI);
     prof_end(m, "radial_scan", ev);
     return cudaGetLastError();
 }

@@ -273,7 +273,8 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate, one thread issues.
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 or fp16 inputs (as idesc says), fp32 accumulate, one
+// thread issues.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate)
 {
@@ -292,8 +293,16 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
                  : "memory");
 }
 
-// 32 lanes x 8 / 16 consecutive 32-bit columns; thread t of the warp gets lane
+// 32 lanes x 4 / 8 / 16 consecutive 32-bit columns; thread t of the warp gets lane
 // (32 * (warp % 4) + t) of the addressed lane quarter.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr)
+                 : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -336,6 +345,12 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
            | (1u << 10)                              // B format bf16
            | (static_cast<uint32_t>(N >> 3) << 17)   // N / 8
            | (static_cast<uint32_t>(M >> 4) << 24);  // M / 16
+}
+
+// The same with fp16 x fp16 inputs (format code 0 for A and B).
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N)
+{
+    return (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
 
 // ---------------------------------------------------------------- bit conversions
