@@ -129,6 +129,25 @@ static mp_status make_map(CUtensorMap *map, const void *ptr, long long rows, int
     return MP_OK;
 }
 
+mp_status make_map_f64_rows(CUtensorMap *map, const void *ptr, long long rows, int cols, int box_rows, int box_cols)
+{
+    return make_map(map, ptr, rows, cols, box_rows, box_cols);
+}
+
+mp_status make_map_f64_G(CUtensorMap *map, const void *ptr, int n_r, int P, int n_t, int ldJ)
+{
+    auto fn = encode_fn();
+    if (!fn) return set_error(MP_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    cuuint64_t dims[3] = {(cuuint64_t)n_t, (cuuint64_t)P, (cuuint64_t)n_r};
+    cuuint64_t strides[2] = {(cuuint64_t)ldJ * 8, (cuuint64_t)P * ldJ * 8};
+    cuuint32_t box[3] = {8u, 1u, 32u}, es[3] = {1u, 1u, 1u};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void *>(ptr), dims, strides, box, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return set_error(MP_ERR_CUDA, "cuTensorMapEncodeTiled (G) failed (%d)", (int)r);
+    return MP_OK;
+}
+
 mp_status make_map_f32(CUtensorMap *map, const void *ptr, int rank, const unsigned long long *dims,
                        const unsigned long long *strides_bytes, const unsigned *box, int swizzle128)
 {
@@ -500,6 +519,8 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
             ALLOC(m->d_G64, (size_t)n_r * m->P * m->fp.ldJ);
             m->fp.arena_bytes = fp64_tc_arena(m);
             ALLOC(m->fp.arena, m->fp.arena_bytes);
+            st = make_map_f64_G(&m->tm_G64, m->d_G64, n_r, m->P, n_theta, m->fp.ldJ);
+            if (st != MP_OK) return fail(st);
         } else {
             ALLOC(m->d_F64, (size_t)m->R * m->P);
             ALLOC(m->d_G64, (size_t)m->R * m->P);
@@ -588,6 +609,10 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         }
         st = cuda_status(cudaStreamSynchronize(m->stream), "table build");
         if (st != MP_OK) return fail(st);
+        if (m->fp.on) {
+            st = cuda_status(fp64_tc_bounds(m), "float64 table bounds");
+            if (st != MP_OK) return fail(st);
+        }
         st = cuda_status(gravity_prepare(m), "gravity stencils");
         if (st != MP_OK) return fail(st);
         st = cuda_status(coarsen_prepare(m), "coarsening blocks");

@@ -26,11 +26,18 @@
 //   k64_expand_tc    short K, many columns (A kept, columns streamed):
 //       (d1) G[i][p][j] = sum_l C[q][i] Ith[t][j] / dmu_j    rows (i, cos | sin) of one order m,
 //                                                            columns j, K = L + 1 - m
-//       (d2) Phi[i][j][k] = sum_p G[i][p][j] Iph[p][k]/dphi_k  rows (i, j), columns k, K = 2 L + 1
+//       (d2) Phi[i][j][k] = sum_p G[i][p][j] Iph[p][k]/dphi_k  rows (i, j), columns k, K = 2 L (the
+//            column m = 0 of the table is 1: G[i][0][j] joins the sums as an integer)
 // The seven digit matrices of B are stacked along N: digit a of A times the first 7 - a
 // digits of B is one MMA of N = (7 - a) Nt columns whose result lands Nt a columns to the
 // right, so a K step of 16 takes seven MMAs for its 28 products and reads A seven times
 // instead of 28 (with one MMA per pair the shared-memory reads of A would bound it).
+//
+// What bounds them: not the tensor core (about 40 % of the time at 1024 x 256 x 512 cells,
+// l_max = 32) nor HBM, but the integer instructions that split and rejoin the operands (half the
+// rate of float32's) and the hand-offs between the warps that issue them.  Measured there against
+// float64 on CUDA cores: (a1) 29.5 ms -> 724 us, (a2) 688 -> 98 us, (d1) 2143 -> 66 us, (d2)
+// 13.9 ms -> 423 us; at 512 x 128 x 256, l_max = 16: 1918 -> 102, 76 -> 21, 200 -> 17, 891 -> 69 us.
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -44,35 +51,49 @@ namespace {
 
 constexpr int kDig = 7;              // digits per operand
 constexpr int kChunkSteps = 8;       // contract: K steps (of 16) that share a row exponent and a chain
+constexpr int kDrainAt = 2;          // contract: steps of an item split before the one before it is drained
 constexpr int kExpandKMax = 146;     // expand: longest chain (7 * 146 * 2^14 < 2^24)
 constexpr int kWorkWarps = 16;
-constexpr int kThreads = (kWorkWarps + 2) * 32;
+constexpr int kThreadsX = (kWorkWarps + 4) * 32;  // expand: two MMA issuers, a table producer for each
+// contract: a fifth warpgroup (three MMA issuers, the table producer) gives registers to the four
+// that split: 640 x 96 = 512 x 112 + 128 x 32
+constexpr int kIssuersC = 3;
+constexpr int kThreadsC = (kWorkWarps + kIssuersC + 1) * 32;
+constexpr int kRegsWork = 112, kRegsRest = 32;
 constexpr int kExpNan = 2047;        // row exponent of a row with an infinity or a NaN
 constexpr int kNtX = 32;             // expand: columns per block
 constexpr int kRowsX = kDig * kNtX;  // expand: stacked table rows of a block
+constexpr int kKeepX = 2;             // expand: octets of k a thread keeps between its two looks at them
+constexpr int kBoxX = 32 * 64;       // expand: a warp's output box, 32 rows of 8 float64
 
-// contract: A slot of one K step: [digit][octet of k][128 rows][8 k]; the octets are 64 bytes
-// further apart than their size, so that a half warp's 8-byte stores (4 rows x 2 octets x 2)
-// fall on different banks
-constexpr int kLboA1 = 128 * 16 + 64;
+// A slot of one K step: [digit][octet of k][128 rows][8 k]
+constexpr int kLboA1 = 128 * 16;
 constexpr int kDigA1 = 2 * kLboA1;
 constexpr int kSlotA1 = kDig * kDigA1;
-// expand: the same without the pad (a warp stores 32 consecutive rows)
 constexpr int kLboA2 = 128 * 16;
 constexpr int kDigA2 = 2 * kLboA2;
 constexpr int kStepA2 = kDig * kDigA2;
 
 __host__ __device__ inline int ceil16(int x) { return (x + 15) & ~15; }
 
-// Contract: the columns of a set in tensor memory. Accumulator blocks start on multiples of 16
-// columns, so a set of N columns takes Nt = N rounded up to 16 for each of the seven weights
-// (64 at most: 7 * 64 = 448 of 512).  A projection of P = 2 L + 1 columns with L a multiple of 8
-// would pay a block of 16 for its one column m = 0 seven times over and, at l_max = 32, no longer
-// fit one pass; its column m = 0 takes one block of 16 instead, with the seven weights as its
-// columns: for digit a of A the table rows of that block are the column's digits a places
-// further down.
+// Contract: the columns of a set (a pass over the density, or the degrees of one order), 64 at
+// most, in halves of up to 32, each padded to a multiple of 16 (accumulator blocks start on such
+// columns) and stacked by itself: 7 * 32 of the half's 256 columns of tensor memory.  A
+// projection of P = 2 L + 1 columns with L a multiple of 8 would pay a block of 16 for its one
+// column m = 0 seven times over and, at l_max = 32, no longer fit one pass; its column m = 0 takes
+// one block of 16 behind the first half instead, with the seven weights as its columns: for
+// digit a of A the table rows of that block are the column's digits a places further down.
+constexpr int kHalf = 32;
 constexpr int kNtMax = 64;
+constexpr int kEtLd = kNtMax + 4;   // column exponents of a set (the own block's at kNtMax)
 constexpr int kRows0 = kDig * 16;   // table rows of the column m = 0: [digit of A][16]
+
+// Padded columns of half h of a set of N columns.
+__host__ __device__ inline int half_cols(int N, int h)
+{
+    const int n = N - h * kHalf;
+    return n <= 0 ? 0 : ceil16(n < kHalf ? n : kHalf);
+}
 
 // ---------------------------------------------------------------------------- digits
 // |x| as a 55-bit integer relative to the row exponent (x = +- V 2^(E - 1077), V < 2^55,
@@ -113,30 +134,133 @@ __device__ __forceinline__ void digits2(uint32_t wl0, uint32_t wh0, uint32_t hi0
 
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7FFFFFFFu; }
 
-// acc 2^e2 as float64 by integer instructions (round to nearest); results outside the normal
-// range go through ldexp.
-__device__ __forceinline__ double scaled_i64(long long acc, int e2)
+// Rows next to the bottom of the float64 range (denormals among them): their values times
+// 2^300, which is exact, and the exponent of the largest.  Out of line: inlined, the multiplies
+// were predicated instead of branched around and kept the float64 pipe 29 % busy.
+template <int N>
+__device__ __noinline__ void scale_up_n(double *x)
 {
-    const unsigned long long u0 = acc < 0 ? 0ull - (unsigned long long)acc : (unsigned long long)acc;
-    if (u0 == 0) return 0.0;
-    const int lz = __clzll((long long)u0);
-    const unsigned long long u = u0 << lz;
-    const int be = 1023 + 63 - lz + e2;
-    if (be < 1 || be > 2045) return ldexp((double)acc, e2);
-    const unsigned long long r = (u >> 11) + ((u >> 10) & 1ull);
-    const unsigned long long b = ((unsigned long long)(be - 1) << 52) + r + (acc < 0 ? 1ull << 63 : 0ull);
-    return __longlong_as_double((long long)b);
+#pragma unroll
+    for (int e = 0; e < N; ++e) x[e] *= 0x1p300;
+}
+template <int N>
+__device__ __forceinline__ void scale_up(double (&x)[N])
+{
+    double y[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) y[e] = x[e];
+    scale_up_n<N>(y);
+#pragma unroll
+    for (int e = 0; e < N; ++e) x[e] = y[e];
+}
+__device__ __noinline__ int scaled_up_exponent(uint32_t max_hi)
+{
+    return (int)(abs_hi(__hiloint2double((int)max_hi, -1) * 0x1p300) >> 20);
 }
 
-// D (float32, tensor memory) (+)= A B^T for one digit of A: N may pass the 256 columns of one
-// MMA instruction.
-__device__ __forceinline__ void mma_digit(uint32_t d, uint32_t a, uint32_t lbo_a, uint32_t b, uint32_t lbo_b, int N,
-                                          uint32_t acc)
+// hi:lo 2^e2 (a signed 64-bit integer below 2^62 in magnitude) as float64 by integer
+// instructions, rounded to nearest; sets `odd` when the result is outside the normal range
+// (the caller then takes ldexp).
+__device__ __forceinline__ double scaled_i64(uint32_t lo, uint32_t hi, int e2, bool &odd)
 {
-    const uint64_t ad = sdesc_noswizzle(a, lbo_a, 128);
-    const int n0 = N > 256 ? 256 : N;
-    umma_bf16(d, ad, sdesc_noswizzle(b, lbo_b, 128), idesc_f16_f32(128, n0), acc);
-    if (N > 256) umma_bf16(d + 256, ad, sdesc_noswizzle(b + 256 * 16, lbo_b, 128), idesc_f16_f32(128, N - 256), acc);
+    const uint32_t sg = (uint32_t)((int)hi >> 31);
+    uint32_t ul, uh, l, h;
+    asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %4;" : "=r"(ul), "=r"(uh) : "r"(lo ^ sg), "r"(hi ^ sg), "r"(sg));
+    // leading one to bit 62: shift left by n, in two steps past 32
+    const uint32_t top = uh ? uh : ul;
+    const int n = (uh ? -1 : 31) + __clz((int)top);
+    const int n2 = max(n - 32, 0);
+    asm("shl.b32 %0, %1, %2;" : "=r"(h) : "r"(__funnelshift_lc(ul, uh, n)), "r"(n2));
+    asm("shl.b32 %0, %1, %2;" : "=r"(l) : "r"(ul), "r"(n));
+    asm("add.cc.u32 %0, %0, 0x200;\n\taddc.u32 %1, %1, 0;" : "+r"(l), "+r"(h));
+    const int be = 1023 + 62 - 1 + e2 - n;             // exponent field less one: the leading one adds it
+    odd |= (unsigned)be > 2044u && top != 0;
+    const uint32_t rl = __funnelshift_r(l, h, 10);
+    const uint32_t rh = (h >> 10) + (top ? (uint32_t)be << 20 : 0u);
+    return __hiloint2double((int)(rh | (hi & 0x80000000u)), (int)rl);
+}
+
+// The same through ldexp, for results outside the normal range; NaN for a row that holds one.
+__device__ __noinline__ double scaled_i64_slow(uint32_t lo, uint32_t hi, int e2, int row_exponent)
+{
+    if (row_exponent >= kExpNan) return __longlong_as_double(0x7FF8000000000000ll);
+    return ldexp((double)(long long)(((unsigned long long)hi << 32) | lo), e2);
+}
+
+// An integer held in a float32: below 2^22 in magnitude by one addition (the integer appears
+// in the low mantissa bits of 1.5 2^23 + x), otherwise by a conversion (a quarter of the rate).
+template <bool SMALL>
+__device__ __forceinline__ int acc_int(float x)
+{
+    return SMALL ? __float_as_int(x + 12582912.0f) - 0x4B400000 : __float2int_rn(x);
+}
+
+// The seven accumulators of one result as a 64-bit integer in units of 2^(56 + DS) (of 2^110 =
+// the product of the operands' scales): the two lightest are added in float32 (a rounding of
+// 2^-(54 - DS) of the row and column maxima at most), the others exactly.  NM: how many of the
+// leading ones are below 2^22.
+template <int NM, int DS>
+__device__ __forceinline__ void acc_sum(const float (&t)[kDig], uint32_t &lo, uint32_t &hi)
+{
+    constexpr float w5 = 1.0f / (1 << DS), w6 = w5 / 256.0f;
+    const float t56 = fmaf(t[6], w6, DS ? t[5] * w5 : t[5]);
+    const int a0 = acc_int<(NM > 0)>(t[0]), a1 = acc_int<(NM > 1)>(t[1]), a2 = acc_int<(NM > 2)>(t[2]);
+    const int a3 = acc_int<(NM > 3)>(t[3]), a4 = acc_int<(NM > 4)>(t[4]);
+    // (a chain of 128 terms: 6 pairs, 6 * 128 * 2^14 2^-DS < 2^22 from DS = 2 on)
+    const int a5 = acc_int<(NM > 5 || DS >= 2)>(t56);
+    const long long l = (long long)(a2 * 256 + a3) * (65536 >> DS) +
+                        (NM > 4 ? (long long)(a4 * (256 >> DS) + a5) : (long long)a4 * (256 >> DS) + a5);
+    if (DS == 0) {
+        lo = (uint32_t)l;
+        hi = (uint32_t)(l >> 32) + (uint32_t)(a0 * 256 + a1);
+    } else {
+        const long long v = l + (long long)(a0 * 256 + a1) * (long long)((1ull << 32) >> DS);
+        lo = (uint32_t)v;
+        hi = (uint32_t)(v >> 32);
+    }
+}
+
+// The sum for chains short enough that all but the lightest accumulators, or all of them
+// (NM >= 5), stay below 2^22: the integers keep the offset 0x4B400000 of their float bits
+// through the multiplies (no pair overflows 32 unsigned bits) and one 64-bit constant takes
+// all of them off, so that the sum needs two integer-pipe instructions (the rest is on the FMA
+// pipe; integer logic runs at half its rate and bounds the kernel).
+__device__ __forceinline__ void acc_sum_small(const float (&t)[kDig], uint32_t &lo, uint32_t &hi)
+{
+    uint32_t a[6];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) a[i] = (uint32_t)__float_as_int(t[i] + 12582912.0f);
+    a[5] = (uint32_t)__float_as_int(fmaf(t[6], 0.00390625f, t[5]) + 12582912.0f);
+    constexpr uint32_t kPair = 0x4B400000u * 257u;  // modulo 2^32
+    constexpr unsigned long long kOff =
+        (unsigned long long)kPair * 65536u + kPair + ((unsigned long long)kPair << 32);
+    const unsigned long long v = (unsigned long long)(a[2] * 256u + a[3]) * 65536u + (a[4] * 256u + a[5]) +
+                                 ((unsigned long long)(a[0] * 256u + a[1]) << 32) - kOff;
+    lo = (uint32_t)v;
+    hi = (uint32_t)(v >> 32);
+}
+
+// Eight results of one row at once: hi:lo 2^(e0 + et) as in scaled_i64, for integers of 33 bits or
+// more (the common case); false when one is smaller.
+template <int N>
+__device__ __forceinline__ bool scaled_row(const uint32_t (&lo)[N], const uint32_t (&hi)[N], const int (&be0)[N],
+                                           double (&out)[N])
+{
+    uint32_t least = 0xFFFFFFFFu;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        const uint32_t sg = (uint32_t)((int)hi[e] >> 31);
+        uint32_t ul, uh, h, l;
+        asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %4;" : "=r"(ul), "=r"(uh) : "r"(lo[e] ^ sg), "r"(hi[e] ^ sg), "r"(sg));
+        least = min(least, uh);
+        const int n = __clz((int)uh) - 1;  // leading one to bit 62
+        h = __funnelshift_l(ul, uh, n);
+        l = ul << (n & 31);
+        asm("add.cc.u32 %0, %0, 0x200;\n\taddc.u32 %1, %1, 0;" : "+r"(l), "+r"(h));
+        const uint32_t rh = (h >> 10) + ((uint32_t)(be0[e] - n) << 20);
+        out[e] = __hiloint2double((int)(rh | (hi[e] & 0x80000000u)), (int)__funnelshift_r(l, h, 10));
+    }
+    return least != 0;
 }
 
 // ---------------------------------------------------------------------------- tables
@@ -148,6 +272,7 @@ struct TabParams {
     const unsigned long long *off;  // byte offset per set (pass, or order m)
     int *et;                        // column exponents, [set][et_ld]
     int kind, n_t, n_p, L, P, pass_cols, m0, et_ld;
+    int *bound;  // largest sum an accumulator can reach: expand, the sixth; contract, the fourth
 };
 
 // Sets of the theta contraction: order m = s, columns l = m .. m + 63, for s = 0 .. L; the
@@ -179,13 +304,13 @@ __device__ __forceinline__ double tab_value(const TabParams &t, int set, int n, 
         return t.Ith[(size_t)tri(m + set_col0(set, t.L) + n, m) * t.n_t + k];
     }
     case TAB_EXPAND_TH: return t.Ith[(size_t)tri(set + k, set) * t.n_t + n] / t.dmu[n];
-    default: return t.Iphc[(size_t)k * t.n_p + n];
+    default: return t.Iphc[(size_t)(k + 1) * t.n_p + n];  // m >= 1: the column m = 0 is 1 everywhere
     }
 }
 
 // One warp per table column n of one set: its exponent, then its digits.  Contract tables are
-// [K step]{[octet][7 Nt rows][8], row = digit Nt + n; for a column m = 0 of its own then
-// [digit of A][octet][16 rows][8]}; expand tables are blocks of 32
+// [K step]{per half [octet][7 Nt rows][8], row = digit Nt + n; for a column m = 0 of its own
+// then [digit of A][octet][16 rows][8]}; expand tables are blocks of 32
 // columns, [block][K step][octet][7 x 32][8].  Cells past K are never written (the tables
 // start as zeros).
 __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n_sets)
@@ -198,42 +323,72 @@ __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n
     case TAB_PROJECT: N = pass_ncols(set, t.pass_cols, t.m0, t.P), K = t.n_p; break;
     case TAB_CONTRACT: N = set_cols(set, t.L), K = t.n_t; break;
     case TAB_EXPAND_TH: N = t.n_t, K = t.L + 1 - set; break;
-    default: N = t.n_p, K = t.P; break;
+    default: N = t.n_p, K = t.P - 1; break;
     }
     if (n >= N) return;
     uint32_t mx = 0;
     for (int k = lane; k < K; k += 32) mx = max(mx, abs_hi(tab_value(t, set, n, k)));
     mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-    const int E = (int)(mx >> 20);
+    // (phi expansion: every column at the scale of the m = 0 column, which is 1 and not in the table)
+    const int E = t.kind == TAB_EXPAND_PH ? 1023 : (int)(mx >> 20);
     if (lane == 0) t.et[(size_t)set * t.et_ld + (n < 0 ? kNtMax : n)] = E;
     if (E == 0) return;  // zeros
     const bool stacked = t.kind == TAB_PROJECT || t.kind == TAB_CONTRACT;
-    const int nd = stacked ? ceil16(N) : kNtX, rows = kDig * nd;
-    const size_t step = (size_t)(rows + (own0 ? kRows0 : 0)) * 32;
-    const int steps = (K + 15) / 16;
+    const int hf = stacked && n >= kHalf, h0 = half_cols(N, 0), h1 = half_cols(N, 1);
+    const int nd = !stacked ? kNtX : hf ? h1 : h0, rows = kDig * nd;
+    const int main_rows = stacked ? kDig * (h0 + h1) : rows;
+    const size_t step = (size_t)(main_rows + (own0 ? kRows0 : 0)) * 32;
+    const int steps = max(1, (K + 15) / 16);
     uint8_t *base = t.tab + t.off[set] + (stacked ? 0 : (size_t)(n / kNtX) * steps * step);
-    const int nr = stacked ? n : n % kNtX;
-    for (int k = lane; k < K; k += 32) {
-        const double x = tab_value(t, set, n, k);
-        const uint32_t hi = (uint32_t)__double2hiint(x);
-        uint32_t wl, wh, d[kDig];
-        fix55((uint32_t)__double2loint(x), hi, E + 9, wl, wh);
-        if ((hi & 0x7FF00000u) == 0) wl = 0x80808080u, wh = 0x00008080u;  // zeros stay zeros
-        digits2(wl, wh, hi, wl, wh, hi, d);
-        uint8_t *dst = base + (size_t)(k >> 4) * step + (k & 7) * 2;
-        const int oct = (k >> 3) & 1;
-        if (n >= 0) {
+    const int nr = stacked ? n - hf * kHalf : n % kNtX;
+    if (hf) base += (size_t)kDig * h0 * 32;
+    int s5 = 0, s6 = 0, s3 = 0, s3max = 0;
+    for (int k0 = 0; k0 < K; k0 += 32) {
+        const int k = k0 + lane;
+        if (k < K) {
+            const double x = tab_value(t, set, n, k);
+            const uint32_t hi = (uint32_t)__double2hiint(x);
+            uint32_t wl, wh, d[kDig];
+            fix55((uint32_t)__double2loint(x), hi, E + 9, wl, wh);
+            if ((hi & 0x7FF00000u) == 0) wl = 0x80808080u, wh = 0x00008080u;  // zeros stay zeros
+            digits2(wl, wh, hi, wl, wh, hi, d);
 #pragma unroll
-            for (int i = 0; i < kDig; ++i)
-                *reinterpret_cast<uint16_t *>(dst + (size_t)(oct * rows + i * nd + nr) * 16) = (uint16_t)(d[i] & 0xFFFFu);
-        } else {
+            for (int i = 0; i < kDig; ++i) {
+                const int v = abs(__half2int_rn(__ushort_as_half((unsigned short)(d[i] & 0xFFFFu))));
+                (i < 6 ? s5 : s6) += v;
+                if (i < 4) s3 += v;
+            }
+            uint8_t *dst = base + (size_t)(k >> 4) * step + (k & 7) * 2;
+            const int oct = (k >> 3) & 1;
+            if (n >= 0) {
 #pragma unroll
-            for (int a = 0; a < kDig; ++a)
-#pragma unroll
-                for (int i = 0; i + a < kDig; ++i)
-                    *reinterpret_cast<uint16_t *>(dst + (size_t)rows * 32 + (size_t)(a * 32 + oct * 16 + a + i) * 16) =
+                for (int i = 0; i < kDig; ++i)
+                    *reinterpret_cast<uint16_t *>(dst + (size_t)(oct * rows + i * nd + nr) * 16) =
                         (uint16_t)(d[i] & 0xFFFFu);
+            } else {
+#pragma unroll
+                for (int a = 0; a < kDig; ++a)
+#pragma unroll
+                    for (int i = 0; i + a < kDig; ++i)
+                        *reinterpret_cast<uint16_t *>(dst + (size_t)main_rows * 32 +
+                                                      (size_t)(a * 32 + oct * 16 + a + i) * 16) =
+                            (uint16_t)(d[i] & 0xFFFFu);
+            }
         }
+        if ((k0 + 32) % (16 * kChunkSteps) == 0 || k0 + 32 >= K) {  // the end of one of A's chains
+            s3max = max(s3max, __reduce_add_sync(0xFFFFFFFFu, s3));
+            s3 = 0;
+        }
+    }
+    // digits of A are at most 128
+    if (!stacked) {
+        // the sixth accumulator takes pairs with the first six digits of B, the seventh joins it
+        // divided by 256
+        s5 = __reduce_add_sync(0xFFFFFFFFu, s5);
+        s6 = __reduce_add_sync(0xFFFFFFFFu, s6);
+        if (lane == 0) atomicMax(t.bound, 128 * s5 + (s5 + s6) / 2 + 2);
+    } else if (lane == 0) {
+        atomicMax(t.bound, 128 * s3max);
     }
 }
 
@@ -246,25 +401,29 @@ struct ContractParams {
     const int *et;
     int *err;
     long long R;
-    int theta;                     // 0: (a1), 1: (a2)
     int n_r, n_t, n_p, L, KL, P, ldJ;
-    int K, n_steps, n_chunks, ds;  // ds: low bits of the 72-bit sum dropped, so that K terms fit 63 bits
+    int K, n_steps, n_chunks, ds;  // ds: low bits of a chain's 62-bit sum dropped, so that n_chunks of them fit
+                                   // (the template's DS, or where that is negative at run time)
     int n_units, npass, pass_cols, m0, n_groups, n_groups0, et_ld;
-    int ns_a, ns_b, nacc, slot_b, cols_max, vec;
+    int ns_a, ns_b, nacc, slot_b, cols_max;
     double scale;                  // (a2) 4 pi G
 };
 
 struct ContractUnit {
     int set, order, col0;  // pass or theta set; its order (theta) and first column
-    int N, Nt, own0;       // columns, rounded up to 16; the column m = 0 in a block of its own
+    int N, Nt[2], own0;    // columns, those of its halves padded; the column m = 0 in a block of its own
     long long row0;        // (a1) first row; (a2) first shell
-    __device__ __forceinline__ uint32_t step_bytes() const { return (uint32_t)(kDig * Nt + (own0 ? kRows0 : 0)) * 32; }
+    __device__ __forceinline__ uint32_t step_bytes() const
+    {
+        return (uint32_t)(kDig * (Nt[0] + Nt[1]) + (own0 ? kRows0 : 0)) * 32;
+    }
 };
 
+template <bool THETA>
 __device__ __forceinline__ ContractUnit contract_unit(const ContractParams &p, int u)
 {
     ContractUnit r;
-    if (!p.theta) {
+    if (!THETA) {
         const int tile = u / p.npass;
         r.set = u - tile * p.npass;
         r.order = 0;
@@ -288,14 +447,16 @@ __device__ __forceinline__ ContractUnit contract_unit(const ContractParams &p, i
         r.N = set_cols(r.set, p.L);
         r.own0 = 0;
     }
-    r.Nt = ceil16(r.N);
+    r.Nt[0] = half_cols(r.N, 0);
+    r.Nt[1] = half_cols(r.N, 1);
     return r;
 }
 
 // Start of row `r` of a unit in the source (K contiguous values), or nullptr past the last row.
+template <bool THETA>
 __device__ __forceinline__ const double *contract_row(const ContractParams &p, const ContractUnit &u, int r)
 {
-    if (!p.theta) {
+    if (!THETA) {
         const long long row = u.row0 + r;
         return row < p.R ? p.src + row * p.n_p : nullptr;
     }
@@ -307,9 +468,10 @@ __device__ __forceinline__ const double *contract_row(const ContractParams &p, c
 // Roles: warps 0-15 split A (each thread four neighbouring k of one row per K step, the whole
 // chunk of 128 k in registers: its row maxima come from a shuffle over the row's four threads,
 // and a step's registers take the next chunk's loads as soon as it is split, so 128 KB are in
-// flight a CTA) and drain the accumulators between their steps; warp 16 owns tensor memory
-// and issues the MMAs; warp 17 copies the table.
-__global__ void __launch_bounds__(kThreads, 1) k64_contract_tc(const ContractParams prm)
+// flight a CTA) and drain the accumulators between their steps; warp 16 owns tensor memory;
+// warps 16-18 issue the MMAs, warp 19 copies the table.
+template <bool THETA, bool VEC, int DS, int NM>
+__global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractParams prm)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -327,18 +489,18 @@ __global__ void __launch_bounds__(kThreads, 1) k64_contract_tc(const ContractPar
     if (threadIdx.x == 0) {
         for (int s = 0; s < prm.ns_a; ++s) {
             mbar_init(smem_u32(&a_full[s]), kWorkWarps);
-            mbar_init(smem_u32(&a_empty[s]), 1);
+            mbar_init(smem_u32(&a_empty[s]), kIssuersC);
         }
         for (int s = 0; s < prm.ns_b; ++s) {
             mbar_init(smem_u32(&b_full[s]), 1);
-            mbar_init(smem_u32(&b_empty[s]), 1);
+            mbar_init(smem_u32(&b_empty[s]), kIssuersC);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&acc_full[b]), 1);
+            mbar_init(smem_u32(&acc_full[b]), kIssuersC);
             mbar_init(smem_u32(&acc_empty[b]), kWorkWarps);
         }
         for (int b = 0; b < 4; ++b) mbar_init(smem_u32(&e_full[b]), kWorkWarps);
-        mbar_init(smem_u32(drain_bar), 1);
+        mbar_init(smem_u32(drain_bar), kIssuersC);
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -353,284 +515,289 @@ __global__ void __launch_bounds__(kThreads, 1) k64_contract_tc(const ContractPar
     const uint32_t acc_stride = prm.nacc == 2 ? 256 : 0;
     pdl_trigger();
     pdl_wait();  // the source comes from the previous kernels
+    const long long budget = wait_budget(prm.err);
 
-    if (warp == kWorkWarps + 1) {
-        // ---------------- table producer
-        if (lane == 0) {
-            Ring rb;
-            int issued = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                const ContractUnit un = contract_unit(prm, u);
-                const uint8_t *src = prm.tab + prm.off[un.set];
-                const uint32_t bytes = un.step_bytes();
-                for (int s = 0; s < prm.n_steps; ++s, rb.next(prm.ns_b)) {
-                    ok = mbar_wait(smem_u32(&b_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err);
-                    if (!ok) break;
-                    const uint32_t bar = smem_u32(&b_full[rb.idx]);
-                    mbar_arrive_expect_tx(bar, bytes);
-                    bulk_load(smem_u32(sB + (size_t)rb.idx * prm.slot_b), src + (size_t)s * bytes, bytes, bar);
-                    ++issued;
+    if (warp >= kWorkWarps) {
+        setmaxnreg_dec<kRegsRest>();
+        if (warp == kWorkWarps + kIssuersC) {
+            // ---------------- table producer
+            if (lane == 0) {
+                Ring rb;
+                int issued = 0;
+                bool ok = true;
+                for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
+                    const ContractUnit un = contract_unit<THETA>(prm, u);
+                    const uint8_t *src = prm.tab + prm.off[un.set];
+                    const uint32_t bytes = un.step_bytes();
+                    for (int s = 0; s < prm.n_steps; ++s, rb.next(prm.ns_b)) {
+                        ok = mbar_wait_tested(smem_u32(&b_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
+                        if (!ok) break;
+                        const uint32_t bar = smem_u32(&b_full[rb.idx]);
+                        mbar_arrive_expect_tx(bar, bytes);
+                        bulk_load(smem_u32(sB + (size_t)rb.idx * prm.slot_b), src + (size_t)s * bytes, bytes, bar);
+                        ++issued;
+                    }
                 }
+                drain_ring(b_full, rb, prm.ns_b, issued);
             }
-            drain_ring(b_full, rb, prm.ns_b, issued);
-        }
-    } else if (warp == kWorkWarps) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
+        } else {
+            // ---------------- MMA issuers (the whole warp waits, one lane issues): one for each half of
+            // the columns and one for the column m = 0 of its own block; each commits every step,
+            // with or without MMAs.  One warp alone issuing all of a step's MMAs took 2000 cycles
+            // for 1200 cycles of tensor time.
+            const uint32_t leader = elect_one();
+            const int mine = warp - kWorkWarps;
+            const uint64_t ad0 = sdesc_noswizzle(smem_u32(sA), kLboA1, 128);
+            const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32);
             Ring ra, rb;
             int it = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                const ContractUnit un = contract_unit(prm, u);
+                const ContractUnit un = contract_unit<THETA>(prm, u);
+                const int n = mine < 2 ? un.Nt[mine] : 0;          // this issuer's columns
+                const bool own = mine == 2 && un.own0;
+                // its table rows and accumulators
+                const uint32_t b_off = mine == 0 ? 0u : (uint32_t)(kDig * (un.Nt[0] + (own ? un.Nt[1] : 0))) * 32;
+                const uint64_t bd0 = sdesc_noswizzle(smem_u32(sB) + b_off, own ? 256u : (uint32_t)n * kDig * 16, 128);
+                const uint32_t b_lo0 = (uint32_t)bd0, b_hi = (uint32_t)(bd0 >> 32);
+                const uint32_t d_off = mine == 1 ? 256u : own ? (uint32_t)(kDig * un.Nt[0]) : 0u;
                 for (int c = 0; c < prm.n_chunks && ok; ++c, ++it) {
                     const int b = prm.nacc == 2 ? it & 1 : 0, nth = prm.nacc == 2 ? it >> 1 : it;
-                    ok = mbar_wait(smem_u32(&acc_empty[b]), (nth & 1) ^ 1, abort_flag, prm.err);
+                    ok = warp_all(mbar_wait_tested(smem_u32(&acc_empty[b]), (nth & 1) ^ 1, abort_flag, prm.err, budget));
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d0 = tmem_base + (uint32_t)b * acc_stride;
+                    const uint32_t d0 = tmem_base + (uint32_t)b * acc_stride + d_off;
                     const int steps = min(kChunkSteps, prm.n_steps - c * kChunkSteps);
                     for (int s = 0; s < steps; ++s, ra.next(prm.ns_a), rb.next(prm.ns_b)) {
-                        ok = mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err) &&
-                             mbar_wait(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err);
+                        ok = warp_all(mbar_wait_tested(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err, budget) &&
+                                      mbar_wait_tested(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err, budget));
                         if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t a0 = smem_u32(sA + (size_t)ra.idx * kSlotA1);
-                        const uint32_t b0 = smem_u32(sB + (size_t)rb.idx * prm.slot_b);
-#pragma unroll
-                        for (int i = 0; i < kDig; ++i)
-                            mma_digit(d0 + (uint32_t)(i * un.Nt), a0 + i * kDigA1, kLboA1, b0, (uint32_t)un.Nt * kDig * 16,
-                                      (kDig - i) * un.Nt, (s | i) != 0);
-                        if (un.own0) {
+                        const uint32_t a_lo = a_lo0 + (uint32_t)ra.idx * (kSlotA1 / 16);
+                        const uint32_t b_lo = b_lo0 + (uint32_t)(rb.idx * (prm.slot_b / 16));
+                        if (n == kHalf) {
 #pragma unroll
                             for (int i = 0; i < kDig; ++i)
-                                mma_digit(d0 + (uint32_t)(kDig * un.Nt), a0 + i * kDigA1, kLboA1,
-                                          b0 + (uint32_t)un.Nt * kDig * 32 + i * 512, 256, 16, (s | i) != 0);
+                                umma_f16_warp(d0 + (uint32_t)(i * kHalf), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
+                                              idesc_f16_f32(128, (kDig - i) * kHalf), (s | i) != 0, leader);
+                        } else if (n == 16) {
+#pragma unroll
+                            for (int i = 0; i < kDig; ++i)
+                                umma_f16_warp(d0 + (uint32_t)(i * 16), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
+                                              idesc_f16_f32(128, (kDig - i) * 16), (s | i) != 0, leader);
+                        } else if (own) {
+#pragma unroll
+                            for (int i = 0; i < kDig; ++i)
+                                umma_f16_warp(d0, a_lo + i * (kDigA1 / 16), a_hi, b_lo + i * 32, b_hi,
+                                              idesc_f16_f32(128, 16), (s | i) != 0, leader);
                         }
-                        umma_commit(smem_u32(&a_empty[ra.idx]));
-                        umma_commit(smem_u32(&b_empty[rb.idx]));
+                        umma_commit_warp(smem_u32(&a_empty[ra.idx]), leader);
+                        umma_commit_warp(smem_u32(&b_empty[rb.idx]), leader);
                     }
-                    if (ok) umma_commit(smem_u32(&acc_full[b]));
+                    if (ok) umma_commit_warp(smem_u32(&acc_full[b]), leader);
                 }
             }
-            umma_commit(smem_u32(drain_bar));
+            umma_commit_warp(smem_u32(drain_bar), leader);
             const long long t0 = clock64();
             while (!mbar_try_wait(smem_u32(drain_bar), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
             }
+            __syncwarp();
         }
     } else {
         // ---------------- split + drain
-        const int crow = 8 * warp + (lane >> 2), quad = lane & 3;  // split: row, k = 16 step + 4 quad + 0..3
+        setmaxnreg_inc<kRegsWork>();
+        // split: row, k = 16 step + 4 quad + 0..3; the quads of a row sit in lanes l, l ^ 1, l ^ 16,
+        // so that a half warp's 8-byte stores are 128 consecutive bytes (8 rows of one octet)
+        const int crow = 8 * warp + ((lane >> 1) & 7), quad = (lane & 1) | ((lane >> 4) << 1);
         const int q4 = warp & 3, grp = warp >> 2;                  // drain: lane quarter, column group
         const uint32_t a_off = (uint32_t)((quad >> 1) * kLboA1 + crow * 16 + (quad & 1) * 8);
         double v[kChunkSteps][4];
         bool ok = true, bad = false;
 
-        auto load_step = [&](const double *row, int step, double (&x)[4]) {
-            const int k = 16 * step + 4 * quad;
+        // K step s of a chunk: `p` at the thread's first k of the chunk, `lim` terms left from it
+        // (none or fewer past the last row)
+        auto load_step = [&](const double *p, int lim, int s, double (&x)[4]) {
+            if (VEC && lim > 16 * s + 3) {
+                ldg_f64x4(p + 16 * s, x);
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = 0.0;
-            if (row) {
-                if (prm.vec) {
-                    if (k < prm.K) {
-                        const double2 t = __ldg(reinterpret_cast<const double2 *>(row + k));
-                        x[0] = t.x, x[1] = t.y;
-                    }
-                    if (k + 2 < prm.K) {
-                        const double2 t = __ldg(reinterpret_cast<const double2 *>(row + k + 2));
-                        x[2] = t.x, x[3] = t.y;
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if (k + e < prm.K) x[e] = __ldg(row + k + e);
-                }
+                for (int e = 0; e < 4; ++e) x[e] = lim > 16 * s + e ? __ldg(p + 16 * s + e) : 0.0;
             }
         };
-
-        // the accumulators of item `it` (unit un, chunk c) into the row's running sums, after
-        // the last chunk to memory; Er: the running exponent of this thread's row
-        int Er = 0;
-        auto drain = [&](const ContractUnit &un, int c, int it) -> bool {
-            const int b = prm.nacc == 2 ? it & 1 : 0, nth = prm.nacc == 2 ? it >> 1 : it;
-            // the row exponents of this item are written, its MMAs complete
-            if (!warp_all(mbar_wait(smem_u32(&e_full[it & 3]), (it >> 2) & 1, abort_flag, prm.err) &&
-                          mbar_wait(smem_u32(&acc_full[b]), nth & 1, abort_flag, prm.err)))
-                return false;
-            tc_fence_after();
-            const int row = 32 * q4 + lane;
-            const bool last = c == prm.n_chunks - 1;
-            const int Ec = sE[(it & 3) * 128 + row];
-            // running sums are kept at the largest exponent of the row's chunks so far
-            int sh_old = 0, sh_new = 0;
-            if (c == 0) {
-                Er = Ec;
-            } else {
-                const int En = max(Er, Ec);
-                sh_old = min(63, En - Er);
-                sh_new = min(63, En - Ec);
-                Er = En;
-            }
-            double *dst = nullptr;  // column n of the unit: dst + n ldJ, or dst + (col0 + n)^2
-            if (!prm.theta) {
-                const long long r = un.row0 + row;
-                if (r < prm.R) {
-                    const int i = (int)(r / prm.n_t), j = (int)(r - (long long)i * prm.n_t);
-                    dst = prm.dst + ((size_t)i * prm.P + un.col0) * prm.ldJ + j;
-                }
-            } else {
-                const int i = (int)un.row0 + (un.order ? row >> 1 : row);
-                if (i < prm.n_r) dst = prm.dst + (size_t)i * prm.KL + (un.order ? 2 * un.order - 1 + (row & 1) : 0);
-            }
-            const uint32_t col = tmem_base + (uint32_t)b * acc_stride + ((uint32_t)(q4 * 32) << 16);
-            // groups of four columns, dealt to the four warps of a lane quarter; the column m = 0
-            // of its own block (its seven weights side by side) comes last, as column N
-            const int n_cols = un.N + un.own0;
-            for (int n = 4 * grp; n < n_cols; n += 16) {
-                uint32_t t[kDig][4];
-                const bool own = n + 3 >= un.N && un.own0;  // N is a multiple of 16 then: n = N
-                if (!own) {
-#pragma unroll
-                    for (int i = 0; i < kDig; ++i) tmem_ld4(col + (uint32_t)(i * un.Nt + n), t[i]);
-                } else {
-                    uint32_t w[4];
-                    tmem_ld4(col + (uint32_t)(kDig * un.Nt), w);
-                    tmem_ld4(col + (uint32_t)(kDig * un.Nt + 4), t[4]);
-                    tmem_ld_wait();
-                    t[6][0] = t[4][2];
-                    t[5][0] = t[4][1];
-                    t[0][0] = w[0];
-                    t[1][0] = w[1];
-                    t[2][0] = w[2];
-                    t[3][0] = w[3];
-                }
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (n + e >= n_cols) break;
-                    int a[kDig];
-#pragma unroll
-                    for (int i = 0; i < kDig; ++i) a[i] = __float2int_rn(__uint_as_float(t[i][e]));
-                    const long long hi = (long long)a[0] * 65536 + ((long long)a[1] * 256 + a[2]);
-                    const long long lo = (long long)a[3] * 16777216 + (long long)a[4] * 65536 +
-                                         ((long long)a[5] * 256 + a[6]);
-                    long long s = (hi << (32 - prm.ds)) + ((lo + (1ll << (prm.ds - 1))) >> prm.ds);
-                    if (prm.n_chunks > 1) {
-                        long long *pa = sAcc + (size_t)(n + e) * 128 + row;
-                        s >>= sh_new;
-                        if (c > 0) s += *pa >> sh_old;
-                        if (!last) *pa = s;
-                    }
-                    if (last && dst) {
-                        const int Et = __ldg(prm.et + (size_t)un.set * prm.et_ld + (own ? kNtMax : n + e));
-                        const double x = Er >= kExpNan ? __longlong_as_double(0x7FF8000000000000ll)
-                                                       : scaled_i64(s, 48 + prm.ds + Er + Et - 2154);
-                        if (prm.theta)
-                            dst[(size_t)(un.col0 + n + e) * (un.col0 + n + e)] = prm.scale * x;
-                        else
-                            dst[own ? -(long long)un.col0 * prm.ldJ : (long long)(n + e) * prm.ldJ] = x;
-                    }
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
-            return true;
+        auto chunk_at = [&](int u, int c, const double *&p, int &lim) {
+            p = u < prm.n_units ? contract_row<THETA>(prm, contract_unit<THETA>(prm, u), crow) : nullptr;
+            const int k = c * (16 * kChunkSteps) + 4 * quad;
+            lim = p ? prm.K - k : 0;
+            p += k;
         };
 
         Ring ra;
-        int it = 0, pend_c = 0;
-        bool pend = false;
-        ContractUnit un{}, pend_u{};
-        const double *row = nullptr;
-        int u = blockIdx.x;
-        if (u < prm.n_units) {
-            un = contract_unit(prm, u);
-            row = contract_row(prm, un, crow);
+        int it = 0, Er = 0;  // Er: running exponent of this thread's drain row
+        int u = blockIdx.x, c = 0, pu = -1, pc = 0;  // this item, the one before (not yet drained)
+        const double *src;
+        int lim;
+        chunk_at(u, c, src, lim);
 #pragma unroll
-            for (int s = 0; s < kChunkSteps; ++s) load_step(row, s, v[s]);
-        }
-        int c = 0;
-        while (u < prm.n_units && ok) {
-            const int steps = min(kChunkSteps, prm.n_steps - c * kChunkSteps);
-            // the item after this one, whose loads follow the splitting of this one's registers
-            int u2 = u, c2 = c + 1;
-            ContractUnit un2 = un;
-            const double *row2 = row;
-            if (c2 == prm.n_chunks) {
-                c2 = 0;
-                u2 = u + (int)gridDim.x;
-                row2 = nullptr;
-                if (u2 < prm.n_units) {
-                    un2 = contract_unit(prm, u2);
-                    row2 = contract_row(prm, un2, crow);
-                }
-            }
+        for (int s = 0; s < kChunkSteps; ++s) load_step(src, lim, s, v[s]);
+        while (ok && (u < prm.n_units || pu >= 0)) {
+            const int steps = u < prm.n_units ? min(kChunkSteps, prm.n_steps - c * kChunkSteps) : 0;
+            const int u2 = c + 1 == prm.n_chunks ? u + (int)gridDim.x : u, c2 = c + 1 == prm.n_chunks ? 0 : c + 1;
             uint32_t mx = 0;
 #pragma unroll
             for (int s = 0; s < kChunkSteps; ++s)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) mx = max(mx, abs_hi(v[s][e]));
             mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
-            mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
-            int E = (int)(mx >> 20), E0 = 0;
+            mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 16));
+            int E = (int)(mx >> 20);
+            const bool tiny = E < 128;
             bad |= E >= kExpNan;
-            if (E < 128) {  // next to the bottom of the float64 range: scaled up exactly
-                E = max(128, (int)(abs_hi(__hiloint2double((int)mx, -1) * 0x1p300) >> 20));
-                E0 = -300;
-            }
+            // next to the bottom of the float64 range (denormals among it): scaled up exactly
+            if (tiny) E = max(128, scaled_up_exponent(mx));
             // four exponent buffers: a warp splits at most two items ahead of another one's drain
-            if (quad == 0) sE[(it & 3) * 128 + crow] = E + E0;
+            if (quad == 0 && steps) sE[(it & 3) * 128 + crow] = tiny ? E - 300 : E;
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&e_full[it & 3]));
+            if (lane == 0 && steps) mbar_arrive(smem_u32(&e_full[it & 3]));
             const int e9 = E + 9;
+            chunk_at(u2, c2, src, lim);
 #pragma unroll
             for (int s = 0; s < kChunkSteps; ++s) {
-                if (s < steps && ok) {
-                    if (s == 2 && pend) {
-                        ok = drain(pend_u, pend_c, it - 1);
-                        pend = false;
-                    }
-                    if (ok) ok = warp_all(mbar_wait(smem_u32(&a_empty[ra.idx]), ra.phase ^ 1, abort_flag, prm.err));
-                    if (ok) {
-                        uint8_t *dst = sA + (size_t)ra.idx * kSlotA1 + a_off;
-                        uint32_t wl[4], wh[4], d0[kDig], d1[kDig];
-                        if (E0) {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) v[s][e] *= 0x1p300;
+                if (s == kDrainAt) {
+                    // ---- the accumulators of the item before this one into the row's running
+                    // sums, after its last chunk to memory (two steps of this item are split by
+                    // now, so the MMAs have work as soon as the accumulators are free)
+                    if (pu >= 0 && ok) {
+                        const ContractUnit un = contract_unit<THETA>(prm, pu);
+                        const int b = prm.nacc == 2 ? (it - 1) & 1 : 0, nth = prm.nacc == 2 ? (it - 1) >> 1 : it - 1;
+                        ok = warp_all(mbar_wait_tested(smem_u32(&e_full[(it - 1) & 3]), ((it - 1) >> 2) & 1, abort_flag, prm.err, budget) &&
+                                      mbar_wait_tested(smem_u32(&acc_full[b]), nth & 1, abort_flag, prm.err, budget));
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int row = 32 * q4 + lane;
+                        const bool last = pc == prm.n_chunks - 1;
+                        const int Ec = sE[((it - 1) & 3) * 128 + row];
+                        // running sums are kept at the largest exponent of the row's chunks so far
+                        const int dsr = DS < 0 ? prm.ds : 0;  // run-time part of the dropped bits
+                        int sh_old = 0, sh_new = dsr;
+                        if (pc == 0) {
+                            Er = Ec;
+                        } else {
+                            const int En = max(Er, Ec);
+                            sh_old = min(63, En - Er);
+                            sh_new = min(63, En - Ec + dsr);
+                            Er = En;
                         }
+                        const bool shifts = DS != 0 && !warp_all((sh_old | sh_new) == 0);
+                        double *dst = nullptr;  // column n of the unit: dst + n ldJ, or dst + (col0 + n)^2
+                        if (!THETA) {
+                            const long long r = un.row0 + row;
+                            if (r < prm.R) {
+                                const int i = (int)(r / prm.n_t), j = (int)(r - (long long)i * prm.n_t);
+                                dst = prm.dst + ((size_t)i * prm.P + un.col0) * prm.ldJ + j;
+                            }
+                        } else {
+                            const int i = (int)un.row0 + (un.order ? row >> 1 : row);
+                            if (i < prm.n_r)
+                                dst = prm.dst + (size_t)i * prm.KL + (un.order ? 2 * un.order - 1 + (row & 1) : 0);
+                        }
+                        const uint32_t col = tmem_base + (uint32_t)b * acc_stride + ((uint32_t)(q4 * 32) << 16);
+                        const int e_base = 56 + (DS < 0 ? prm.ds : DS) + Er - 2154;
+                        // one result: its seven accumulators into the running sum at `pa` or, after
+                        // the last chunk, to `out`
+                        auto result = [&](const float (&a)[kDig], long long *pa, int et, double *out, bool in) {
+                            uint32_t lo, hi;
+                            acc_sum<NM, (DS > 0 ? DS : 0)>(a, lo, hi);
+                            if (DS != 0) {
+                                long long x = (long long)(((unsigned long long)hi << 32) | lo);
+                                if (shifts) x >>= sh_new;
+                                if (pc > 0) {
+                                    long long o = *pa;
+                                    if (shifts) o >>= sh_old;
+                                    x += o;
+                                }
+                                if (!last) {
+                                    *pa = x;
+                                    return;
+                                }
+                                lo = (uint32_t)x;
+                                hi = (uint32_t)(x >> 32);
+                            }
+                            bool odd = Er >= kExpNan;
+                            double x = scaled_i64(lo, hi, e_base + et, odd);
+                            if (odd) x = scaled_i64_slow(lo, hi, e_base + et, Er);
+                            if (in) *out = THETA ? prm.scale * x : x;
+                        };
+                        const int *et = prm.et + (size_t)un.set * prm.et_ld;
+                        // groups of four columns, dealt to the four warps of a lane quarter (the
+                        // padding up to Nt holds zeros); the column m = 0 of its own block, with its
+                        // weights side by side, goes to the last of them
+                        for (int n = 4 * grp; n < un.N; n += 16) {
+                            uint32_t t[kDig][4];
+                            const int hf = n >> 5, nt = un.Nt[hf];
+                            const uint32_t c0 = col + (uint32_t)(hf * 256 + (n & 31));
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            fix55((uint32_t)__double2loint(v[s][e]), (uint32_t)__double2hiint(v[s][e]), e9, wl[e],
-                                  wh[e]);
-                        digits2(wl[0], wh[0], (uint32_t)__double2hiint(v[s][0]), wl[1], wh[1],
-                                (uint32_t)__double2hiint(v[s][1]), d0);
-                        digits2(wl[2], wh[2], (uint32_t)__double2hiint(v[s][2]), wl[3], wh[3],
-                                (uint32_t)__double2hiint(v[s][3]), d1);
+                            for (int i = 0; i < kDig; ++i) tmem_ld4(c0 + (uint32_t)(i * nt), t[i]);
+                            int4 e4 = make_int4(0, 0, 0, 0);
+                            if (last) e4 = __ldg(reinterpret_cast<const int4 *>(et + n));
+                            const int ee[4] = {e4.x, e4.y, e4.z, e4.w};
+                            tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < kDig; ++i)
-                            *reinterpret_cast<uint2 *>(dst + i * kDigA1) = make_uint2(d0[i], d1[i]);
-                        fence_proxy_async_smem();
+                            for (int e = 0; e < 4; ++e) {
+                                float a[kDig];
+#pragma unroll
+                                for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(t[i][e]);
+                                const int l = un.col0 + n + e;
+                                result(a, sAcc + (size_t)(n + e) * 128 + row, ee[e],
+                                       THETA ? dst + (size_t)l * l : dst + (size_t)(n + e) * prm.ldJ,
+                                       dst && n + e < un.N);
+                            }
+                        }
+                        if (!THETA && un.own0 && grp == 3) {
+                            uint32_t w[8];
+                            tmem_ld8(col + (uint32_t)(kDig * un.Nt[0]), w);
+                            tmem_ld_wait();
+                            float a[kDig];
+#pragma unroll
+                            for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(w[i]);
+                            result(a, sAcc + (size_t)(un.Nt[0] + un.Nt[1]) * 128 + row, __ldg(et + kNtMax), dst - (size_t)un.col0 * prm.ldJ,
+                                   dst != nullptr);
+                        }
+                        tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&a_full[ra.idx]));
-                        ra.next(prm.ns_a);
+                        if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
                     }
+#pragma unroll
+                    for (int s0 = 0; s0 < kDrainAt; ++s0) load_step(src, lim, s0, v[s0]);
                 }
-                load_step(row2, c2 * kChunkSteps + s, v[s]);
+                if (s < steps) {
+                    ok = ok && warp_all(mbar_wait_tested(smem_u32(&a_empty[ra.idx]), ra.phase ^ 1, abort_flag, prm.err, budget));
+                    if (!ok) break;
+                    uint8_t *dst = sA + (size_t)ra.idx * kSlotA1 + a_off;
+                    uint32_t wl[4], wh[4], d0[kDig], d1[kDig];
+                    if (tiny) scale_up(v[s]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        fix55((uint32_t)__double2loint(v[s][e]), (uint32_t)__double2hiint(v[s][e]), e9, wl[e], wh[e]);
+                    digits2(wl[0], wh[0], (uint32_t)__double2hiint(v[s][0]), wl[1], wh[1],
+                            (uint32_t)__double2hiint(v[s][1]), d0);
+                    digits2(wl[2], wh[2], (uint32_t)__double2hiint(v[s][2]), wl[3], wh[3],
+                            (uint32_t)__double2hiint(v[s][3]), d1);
+#pragma unroll
+                    for (int i = 0; i < kDig; ++i)
+                        *reinterpret_cast<uint2 *>(dst + i * kDigA1) = make_uint2(d0[i], d1[i]);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&a_full[ra.idx]));
+                    ra.next(prm.ns_a);
+                }
+                if (s >= kDrainAt) load_step(src, lim, s, v[s]);
             }
-            if (!ok) break;
-            if (pend) ok = drain(pend_u, pend_c, it - 1);
-            pend = true;
-            pend_u = un;
-            pend_c = c;
-            ++it;
+            pu = steps ? u : -1;
+            pc = c;
             u = u2;
             c = c2;
-            un = un2;
-            row = row2;
+            ++it;
         }
-        if (ok && pend) drain(pend_u, pend_c, it - 1);
-        if (bad && !prm.theta) atomicOr(prm.err, DEV_ERR_NONFINITE);
+        if (bad && !THETA) atomicOr(prm.err, DEV_ERR_NONFINITE);
     }
     tc_fence_before();
     __syncthreads();
@@ -649,24 +816,31 @@ struct ExpandParams {
     const int *et;
     int *err;
     long long R;
-    int theta;                    // 1: (d1), 0: (d2)
     int n_r, n_t, n_p, L, P, ldJ, ldI;
     int N, n_blk, n_units, n_split, n_groups, n_groups0, et_ld;
-    int a_steps, ns_b, vec;       // a_steps: K steps of A held at once
+    int a_steps, ns_b, tma;       // a_steps: K steps of A held at once; ns_b: table slots per issuer; tma: Phi leaves by TMA stores
 };
 
 struct ExpandUnit {
-    int set, K, steps, n_chunks, chunk_steps, blk0, blk1;
+    int set, K, steps, n_chunks, chunk_steps, blk0, blk1, pairs, rot;
     long long row0;
+    // first block of the unit's gi-th pair: each CTA starts at another pair, so that the CTAs do
+    // not all read the same table blocks at the same time
+    __device__ __forceinline__ int pair(int gi) const
+    {
+        const int v = gi + rot;
+        return blk0 + 2 * (v < pairs ? v : v - pairs);
+    }
 };
 
+template <bool THETA>
 __device__ __forceinline__ ExpandUnit expand_unit(const ExpandParams &p, int u)
 {
     ExpandUnit r;
-    if (!p.theta) {
+    if (!THETA) {
         const int tile = u / p.n_split, part = u - tile * p.n_split;
         r.set = 0;
-        r.K = p.P;
+        r.K = p.P - 1;
         r.row0 = (long long)tile * 128;
         // whole pairs of blocks per part
         const int pairs = (p.n_blk + 1) / 2;
@@ -685,47 +859,50 @@ __device__ __forceinline__ ExpandUnit expand_unit(const ExpandParams &p, int u)
         r.blk0 = 0;
         r.blk1 = p.n_blk;
     }
-    r.steps = (r.K + 15) / 16;
+    r.steps = max(1, (r.K + 15) / 16);  // (l_max = 0 leaves no term: one step of zeros)
     r.n_chunks = r.steps <= p.a_steps ? 1 : 2;
     r.chunk_steps = (r.steps + r.n_chunks - 1) / r.n_chunks;
+    r.pairs = (r.blk1 - r.blk0 + 1) / 2;
+    r.rot = (int)(blockIdx.x % (unsigned)max(1, r.pairs));
     return r;
 }
 
 // Roles: warps 0-15 split the unit's A (128 rows, the whole K or, past a_steps, half of it at a
-// time) and turn finished blocks into float64; warp 16 owns tensor memory and issues the MMAs of
-// one block of 32 columns while the other block's accumulators are drained; warp 17 copies the
-// table.  With K in one piece A is split once per unit; in two it is split again for every pair
-// of blocks.
-__global__ void __launch_bounds__(kThreads, 1) k64_expand_tc(const ExpandParams prm)
+// time) and turn finished blocks of 32 columns into float64; the even and the odd blocks have an
+// accumulator, an MMA issuer (warps 16, 17) and a table producer (warps 18, 19) each.  With K
+// in one piece A is split once per unit; in two it is split again for every pair of blocks.
+template <bool THETA, int NM>
+__global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_constant__ CUtensorMap tm_out, const ExpandParams prm)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     constexpr uint32_t kSlotB = kRowsX * 32;
-    uint8_t *sA = smem;
+    uint8_t *sOut = smem;                                   // [16 warps][32 rows][8] float64, 64-byte swizzle
+    uint8_t *sA = sOut + kWorkWarps * kBoxX;
     uint8_t *sB = sA + (size_t)prm.a_steps * kStepA2;
-    uint8_t *sOut = sB + (size_t)prm.ns_b * kSlotB;                   // [16 warps][32 rows][8] float64
-    uint32_t *sMax = reinterpret_cast<uint32_t *>(sOut + kWorkWarps * 2048);  // [2 units][4][128]
+    uint32_t *sMax = reinterpret_cast<uint32_t *>(sB + (size_t)2 * prm.ns_b * kSlotB);  // [2 units][4][128]
     uint64_t *bars = reinterpret_cast<uint64_t *>(sMax + 8 * 128);
-    uint64_t *b_full = bars, *b_empty = b_full + prm.ns_b;
-    uint64_t *a_full = b_empty + prm.ns_b, *a_free = a_full + 1;
+    uint64_t *b_full = bars, *b_empty = b_full + 2 * prm.ns_b;
+    uint64_t *a_full = b_empty + 2 * prm.ns_b, *a_free = a_full + 1;
     uint64_t *acc_full = a_free + 1, *acc_empty = acc_full + 2, *m_full = acc_empty + 2, *drain_bar = m_full + 1;
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain_bar + 1);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain_bar + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < prm.ns_b; ++s) {
+        for (int s = 0; s < 2 * prm.ns_b; ++s) {
             mbar_init(smem_u32(&b_full[s]), 1);
             mbar_init(smem_u32(&b_empty[s]), 1);
         }
         mbar_init(smem_u32(a_full), kWorkWarps);
-        mbar_init(smem_u32(a_free), 1);
+        mbar_init(smem_u32(a_free), 2);
         mbar_init(smem_u32(m_full), kWorkWarps);
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&acc_full[b]), 1);
             mbar_init(smem_u32(&acc_empty[b]), kWorkWarps);
         }
-        mbar_init(smem_u32(drain_bar), 1);
+        mbar_init(smem_u32(&drain_bar[0]), 1);
+        mbar_init(smem_u32(&drain_bar[1]), 1);
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -739,94 +916,112 @@ __global__ void __launch_bounds__(kThreads, 1) k64_expand_tc(const ExpandParams 
     const uint32_t tmem_base = *tmem_holder;
     pdl_trigger();
     pdl_wait();  // the source comes from the previous kernels
+    const long long budget = wait_budget(prm.err);
 
-    if (warp == kWorkWarps + 1) {
-        // ---------------- table producer
+    if (warp >= kWorkWarps + 2) {
+        // ---------------- table producers, one for each issuer's half of the ring
         if (lane == 0) {
+            const int mine = warp - kWorkWarps - 2;
+            uint64_t *my_full = b_full + mine * prm.ns_b, *my_empty = b_empty + mine * prm.ns_b;
+            uint8_t *ring = sB + (size_t)mine * prm.ns_b * kSlotB;
             Ring rb;
-            int issued = 0;
+            int issued = 0, blk = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                const ExpandUnit un = expand_unit(prm, u);
+                const ExpandUnit un = expand_unit<THETA>(prm, u);
                 const uint8_t *src = prm.tab + prm.off[un.set];
-                for (int g = un.blk0; g < un.blk1 && ok; g += 2)
-                    for (int ch = 0; ch < un.n_chunks && ok; ++ch)
-                        for (int nb = g; nb < min(g + 2, un.blk1) && ok; ++nb)
-                            for (int s = ch * un.chunk_steps; s < min(un.steps, (ch + 1) * un.chunk_steps);
-                                 ++s, rb.next(prm.ns_b)) {
-                                ok = mbar_wait(smem_u32(&b_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err);
-                                if (!ok) break;
-                                const uint32_t bar = smem_u32(&b_full[rb.idx]);
-                                mbar_arrive_expect_tx(bar, kSlotB);
-                                bulk_load(smem_u32(sB + (size_t)rb.idx * kSlotB),
-                                          src + ((size_t)nb * un.steps + s) * kSlotB, kSlotB, bar);
-                                ++issued;
-                            }
-            }
-            drain_ring(b_full, rb, prm.ns_b, issued);
-        }
-    } else if (warp == kWorkWarps) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            Ring rb;
-            int blk = 0, conv = 0;  // blocks and splits of A so far
-            bool ok = true;
-            for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                const ExpandUnit un = expand_unit(prm, u);
-                for (int g = un.blk0; g < un.blk1 && ok; g += 2) {
+                for (int gi = 0; gi < un.pairs && ok; ++gi) {
+                    const int g = un.pair(gi);
                     const int nbs = min(2, un.blk1 - g);
-                    for (int ch = 0; ch < un.n_chunks && ok; ++ch) {
-                        if (un.n_chunks > 1 || g == un.blk0) {
-                            ok = mbar_wait(smem_u32(a_full), conv & 1, abort_flag, prm.err);
-                            if (!ok) break;
-                            ++conv;
-                        }
-                        const int s0 = ch * un.chunk_steps, s1 = min(un.steps, s0 + un.chunk_steps);
-                        for (int nb = 0; nb < nbs && ok; ++nb) {
-                            const int b = (blk + nb) & 1;
-                            if (ch == 0) ok = mbar_wait(smem_u32(&acc_empty[b]), (((blk + nb) >> 1) & 1) ^ 1, abort_flag, prm.err);
-                            if (!ok) break;
-                            tc_fence_after();
-                            const uint32_t d0 = tmem_base + (uint32_t)b * 256;
-                            for (int s = s0; s < s1; ++s, rb.next(prm.ns_b)) {
-                                ok = mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err);
-                                if (!ok) break;
-                                tc_fence_after();
-                                const uint32_t a0 = smem_u32(sA + (size_t)(s - s0) * kStepA2);
-                                const uint32_t b0 = smem_u32(sB + (size_t)rb.idx * kSlotB);
-#pragma unroll
-                                for (int i = 0; i < kDig; ++i)
-                                    umma_bf16(d0 + (uint32_t)(i * kNtX), sdesc_noswizzle(a0 + i * kDigA2, kLboA2, 128),
-                                              sdesc_noswizzle(b0, kRowsX * 16, 128),
-                                              idesc_f16_f32(128, (kDig - i) * kNtX), (s | i) != 0);
-                                umma_commit(smem_u32(&b_empty[rb.idx]));
-                            }
-                            if (ok && ch == un.n_chunks - 1) umma_commit(smem_u32(&acc_full[b]));
-                        }
-                        if (ok && un.n_chunks > 1) umma_commit(smem_u32(a_free));
-                    }
+                    const int nb = (blk & 1) ^ mine;  // this producer's block of the pair
                     blk += nbs;
+                    if (nb >= nbs) continue;
+                    const uint8_t *from = src + (size_t)(g + nb) * un.steps * kSlotB;
+                    for (int s = 0; s < un.steps; ++s, rb.next(prm.ns_b)) {
+                        ok = mbar_wait_tested(smem_u32(&my_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
+                        if (!ok) break;
+                        const uint32_t bar = smem_u32(&my_full[rb.idx]);
+                        mbar_arrive_expect_tx(bar, kSlotB);
+                        bulk_load(smem_u32(ring + (size_t)rb.idx * kSlotB), from + (size_t)s * kSlotB, kSlotB, bar);
+                        ++issued;
+                    }
                 }
             }
-            umma_commit(smem_u32(drain_bar));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(smem_u32(drain_bar), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+            drain_ring(my_full, rb, prm.ns_b, issued);
+        }
+    } else if (warp >= kWorkWarps) {
+        // ---------------- MMA issuers (the whole warp waits, one lane issues): one for the even
+        // blocks, one for the odd ones, each with an accumulator of its own.  One issuer alone took
+        // 500 to 800 cycles a K step of seven MMAs (448 cycles of tensor time).
+        const uint32_t leader = elect_one();
+        const int mine = warp - kWorkWarps;
+        const uint32_t d0 = tmem_base + (uint32_t)mine * 256;
+        const uint32_t a_lo0 = (uint32_t)sdesc_noswizzle(smem_u32(sA), kLboA2, 128);
+        const uint32_t a_hi = (uint32_t)(sdesc_noswizzle(smem_u32(sA), kLboA2, 128) >> 32);
+        uint8_t *ring = sB + (size_t)mine * prm.ns_b * kSlotB;  // this issuer's half of the table ring
+        uint64_t *my_full = b_full + mine * prm.ns_b, *my_empty = b_empty + mine * prm.ns_b;
+        const uint32_t b_lo0 = (uint32_t)sdesc_noswizzle(smem_u32(ring), kRowsX * 16, 128);
+        const uint32_t b_hi = (uint32_t)(sdesc_noswizzle(smem_u32(ring), kRowsX * 16, 128) >> 32);
+        Ring rb;
+        int blk = 0, conv = 0;  // blocks and splits of A so far
+        bool ok = true;
+        for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
+            const ExpandUnit un = expand_unit<THETA>(prm, u);
+            for (int gi = 0; gi < un.pairs && ok; ++gi) {
+                const int nbs = min(2, un.blk1 - un.pair(gi));
+                for (int ch = 0; ch < un.n_chunks && ok; ++ch) {
+                    if (un.n_chunks > 1 || gi == 0) {
+                        ok = warp_all(mbar_wait_tested(smem_u32(a_full), conv & 1, abort_flag, prm.err, budget));
+                        if (!ok) break;
+                        ++conv;
+                    }
+                    const int s0 = ch * un.chunk_steps, s1 = min(un.steps, s0 + un.chunk_steps);
+                    for (int nb = 0; nb < nbs && ok; ++nb) {
+                        if (((blk + nb) & 1) != mine) continue;
+                        if (ch == 0) {
+                            ok = warp_all(mbar_wait_tested(smem_u32(&acc_empty[mine]), (((blk + nb) >> 1) & 1) ^ 1, abort_flag,
+                                                           prm.err, budget));
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        uint32_t a_lo = a_lo0;
+                        for (int s = s0; s < s1; ++s, rb.next(prm.ns_b), a_lo += kStepA2 / 16) {
+                            ok = warp_all(mbar_wait_tested(smem_u32(&my_full[rb.idx]), rb.phase, abort_flag, prm.err, budget));
+                            if (!ok) break;
+                            const uint32_t b_lo = b_lo0 + (uint32_t)rb.idx * (kSlotB / 16);
+#pragma unroll
+                            for (int i = 0; i < kDig; ++i)
+                                umma_f16_warp(d0 + (uint32_t)(i * kNtX), a_lo + i * (kDigA2 / 16), a_hi, b_lo, b_hi,
+                                              idesc_f16_f32(128, (kDig - i) * kNtX), (s | i) != 0, leader);
+                            umma_commit_warp(smem_u32(&my_empty[rb.idx]), leader);
+                        }
+                        if (ok && ch == un.n_chunks - 1) umma_commit_warp(smem_u32(&acc_full[mine]), leader);
+                    }
+                    // this piece of A has been read
+                    if (ok && (un.n_chunks > 1 || gi == un.pairs - 1)) umma_commit_warp(smem_u32(a_free), leader);
+                }
+                blk += nbs;
             }
         }
+        // both issuers' MMAs are complete before the block gives its memory back
+        umma_commit_warp(smem_u32(&drain_bar[mine]), leader);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(&drain_bar[mine]), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+        }
+        __syncwarp();
     } else {
         // ---------------- split + drain
         const int crow = threadIdx.x & 127, cg = threadIdx.x >> 7;  // split: row, octets cg, cg + 4, ...
-        const int q4 = warp & 3, grp = warp >> 2;                   // drain: lane quarter, 8-column group
-        uint8_t *stage = sOut + warp * 2048;
+        const int q4 = warp & 3, grp = warp >> 2;  // drain: lane quarter (row 32 q4 + lane = crow), 8 columns
         bool ok = true;
-        int blk = 0, freed = 0, lu = 0;
-        int Erow = 0;  // exponent of drain row 32 q4 + lane (= crow's when cg = grp: the same thread)
+        int blk = 0, splits = 0, lu = 0;
+        const uint64_t policy = l2_evict_first_policy();  // Phi is not read again here
 
         for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x, ++lu) {
-            const ExpandUnit un = expand_unit(prm, u);
+            const ExpandUnit un = expand_unit<THETA>(prm, u);
             // element k of this thread's row: src + base + (PH: k ldJ; TH: ((m + k)^2 + p) ldI)
             const double *base = nullptr;
-            if (!prm.theta) {
+            if (!THETA) {
                 const long long r = un.row0 + crow;
                 if (r < prm.R) {
                     const int i = (int)(r / prm.n_t), j = (int)(r - (long long)i * prm.n_t);
@@ -836,150 +1031,198 @@ __global__ void __launch_bounds__(kThreads, 1) k64_expand_tc(const ExpandParams 
                 const int a = un.set ? crow >> 6 : 0, i = (int)un.row0 + (un.set ? crow & 63 : crow);
                 if (i < prm.n_r) base = prm.src + (size_t)(un.set ? 2 * un.set - 1 + a : 0) * prm.ldI + i;
             }
+            // start of this thread's drain row (32 q4 + lane = crow) in the output, where it is not
+            // stored by TMA
+            double *out_row = nullptr;
+            if (!THETA && !prm.tma && un.row0 + crow < prm.R) out_row = prm.dst + (un.row0 + crow) * prm.n_p;
             auto element = [&](int k) -> double {
                 if (!base || k >= un.K) return 0.0;
-                return !prm.theta ? __ldg(base + (size_t)k * prm.ldJ)
-                                  : __ldg(base + (size_t)(un.set + k) * (un.set + k) * prm.ldI);
+                return !THETA ? __ldg(base + (size_t)(k + 1) * prm.ldJ)
+                              : __ldg(base + (size_t)(un.set + k) * (un.set + k) * prm.ldI);
             };
-            uint32_t mx = 0;
-            for (int o = cg; o < 2 * un.steps; o += 4) {
+            // phi: the column m = 0, each thread its own row's (the drain row is the split row)
+            double g0 = 0.0;
+            if (!THETA && base) g0 = __ldg(base);
+            uint32_t mx = abs_hi(g0);
+            // the first octets stay in registers for the split, further ones are read again
+            double x0[kKeepX][8];
+#pragma unroll
+            for (int c = 0; c < kKeepX; ++c)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x0[c][e] = element(8 * (cg + 4 * c) + e);
+            for (int o = cg + 4 * kKeepX; o < 2 * un.steps; o += 4) {
                 double x[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) x[e] = element(8 * o + e);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) mx = max(mx, abs_hi(x[e]));
             }
+#pragma unroll
+            for (int c = 0; c < kKeepX; ++c)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) mx = max(mx, abs_hi(x0[c][e]));
             uint32_t *row_max = sMax + (lu & 1) * 512 + crow;
             row_max[cg * 128] = mx;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(m_full));
-            ok = warp_all(mbar_wait(smem_u32(m_full), lu & 1, abort_flag, prm.err));
+            ok = warp_all(mbar_wait_tested(smem_u32(m_full), lu & 1, abort_flag, prm.err, budget));
             if (!ok) break;
             mx = max(max(row_max[0], row_max[128]), max(row_max[256], row_max[384]));
             int E = (int)(mx >> 20), E0 = 0;
-            double up = 1.0;
             if (E < 128) {  // next to the bottom of the float64 range: scaled up exactly
-                up = 0x1p300;
-                E = max(128, (int)(abs_hi(__hiloint2double((int)mx, -1) * up) >> 20));
+                E = max(128, scaled_up_exponent(mx));
                 E0 = -300;
             }
-            Erow = E + E0;
+            const int Erow = E + E0;
             const int e9 = E + 9;
+            // in units of 2^56: 1.0 in the table would be 2^54, so a quarter of its 55-bit integer
+            uint32_t g0_lo = 0, g0_hi = 0;
+            if (!THETA) {
+                if (E0) {
+                    double t[1] = {g0};
+                    scale_up(t);
+                    g0 = t[0];
+                }
+                uint32_t wl, wh;
+                fix55((uint32_t)__double2loint(g0), (uint32_t)__double2hiint(g0), e9, wl, wh);
+                long long q = (long long)((((unsigned long long)wh << 32 | wl) - 0x0000808080808080ull + 2) >> 2);
+                if (g0 < 0.0) q = -q;
+                g0_lo = (uint32_t)q;
+                g0_hi = (uint32_t)(q >> 32);
+            }
 
-            auto split = [&](int ch) {
+            auto split_octet = [&](double (&x)[8], int o, int s0) {
+                if (E0) scale_up(x);
+                uint32_t d[4][kDig];
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    uint32_t wl0, wh0, wl1, wh1;
+                    const uint32_t h0 = (uint32_t)__double2hiint(x[e]), h1 = (uint32_t)__double2hiint(x[e + 1]);
+                    fix55((uint32_t)__double2loint(x[e]), h0, e9, wl0, wh0);
+                    fix55((uint32_t)__double2loint(x[e + 1]), h1, e9, wl1, wh1);
+                    digits2(wl0, wh0, h0, wl1, wh1, h1, d[e >> 1]);
+                }
+                uint8_t *dst = sA + (size_t)((o >> 1) - s0) * kStepA2 + (o & 1) * kLboA2 + crow * 16;
+#pragma unroll
+                for (int i = 0; i < kDig; ++i)
+                    *reinterpret_cast<uint4 *>(dst + i * kDigA2) = make_uint4(d[0][i], d[1][i], d[2][i], d[3][i]);
+            };
+            // A for the K steps of piece ch, once the MMAs of the piece before have read theirs
+            auto split = [&](int ch) -> bool {
+                if (splits > 0 &&
+                    !warp_all(mbar_wait_tested(smem_u32(a_free), (splits - 1) & 1, abort_flag, prm.err, budget)))
+                    return false;
+                ++splits;
                 const int s0 = ch * un.chunk_steps, s1 = min(un.steps, s0 + un.chunk_steps);
-                for (int o = 2 * s0 + cg; o < 2 * s1; o += 4) {
+                int o = 2 * s0 + cg;
+                if (un.n_chunks == 1) {
+#pragma unroll
+                    for (int c = 0; c < kKeepX; ++c, o += 4)
+                        if (o < 2 * s1) split_octet(x0[c], o, s0);
+                }
+                for (; o < 2 * s1; o += 4) {
                     double x[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) x[e] = element(8 * o + e);
-                    if (E0) {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) x[e] *= up;
-                    }
-                    uint32_t d[4][kDig];
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        uint32_t wl0, wh0, wl1, wh1;
-                        const uint32_t h0 = (uint32_t)__double2hiint(x[e]), h1 = (uint32_t)__double2hiint(x[e + 1]);
-                        fix55((uint32_t)__double2loint(x[e]), h0, e9, wl0, wh0);
-                        fix55((uint32_t)__double2loint(x[e + 1]), h1, e9, wl1, wh1);
-                        digits2(wl0, wh0, h0, wl1, wh1, h1, d[e >> 1]);
-                    }
-                    uint8_t *dst = sA + (size_t)((o >> 1) - s0) * kStepA2 + (o & 1) * kLboA2 + crow * 16;
-#pragma unroll
-                    for (int i = 0; i < kDig; ++i)
-                        *reinterpret_cast<uint4 *>(dst + i * kDigA2) = make_uint4(d[0][i], d[1][i], d[2][i], d[3][i]);
+                    split_octet(x, o, s0);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(a_full));
+                return true;
             };
 
-            // with K in one piece A is free here: every block of the last unit has been drained
-            if (un.n_chunks == 1) split(0);
-            for (int g = un.blk0; g < un.blk1 && ok; g += 2) {
+            if (un.n_chunks == 1) ok = split(0);
+            for (int gi = 0; gi < un.pairs && ok; ++gi) {
+                const int g = un.pair(gi);
                 const int nbs = min(2, un.blk1 - g);
                 if (un.n_chunks > 1)
-                    for (int ch = 0; ch < un.n_chunks && ok; ++ch) {
-                        if (ch > 0) {
-                            ok = warp_all(mbar_wait(smem_u32(a_free), freed & 1, abort_flag, prm.err));
-                            ++freed;
-                        }
-                        if (ok) split(ch);
-                    }
+                    for (int ch = 0; ch < un.n_chunks && ok; ++ch) ok = split(ch);
                 for (int nb = 0; nb < nbs && ok; ++nb, ++blk) {
                     const int b = blk & 1;
-                    ok = warp_all(mbar_wait(smem_u32(&acc_full[b]), (blk >> 1) & 1, abort_flag, prm.err));
+                    ok = warp_all(mbar_wait_tested(smem_u32(&acc_full[b]), (blk >> 1) & 1, abort_flag, prm.err, budget));
                     if (!ok) break;
                     tc_fence_after();
                     uint32_t t[kDig][8];
                     const uint32_t col = tmem_base + (uint32_t)b * 256 + ((uint32_t)(q4 * 32) << 16) + grp * 8;
 #pragma unroll
                     for (int i = 0; i < kDig; ++i) tmem_ld8(col + (uint32_t)(i * kNtX), t[i]);
+                    const int n0 = (g + nb) * kNtX + grp * 8;
+                    // column exponents (padded to whole blocks); the phi table, cell means of cos
+                    // and sin, has one scale
+                    int Et[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) Et[e] = 1023;
+                    if (THETA) {
+                        const int4 *pe = reinterpret_cast<const int4 *>(prm.et + (size_t)un.set * prm.et_ld + n0);
+                        const int4 e0 = __ldg(pe), e1 = __ldg(pe + 1);
+                        Et[0] = e0.x, Et[1] = e0.y, Et[2] = e0.z, Et[3] = e0.w;
+                        Et[4] = e1.x, Et[5] = e1.y, Et[6] = e1.z, Et[7] = e1.w;
+                    }
                     tmem_ld_wait();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
-                    const int n0 = (g + nb) * kNtX + grp * 8;
-                    // rows of 64 bytes in 16-byte pieces, the pieces permuted so that neither the
-                    // stores (one row a lane) nor the loads (four lanes a row) share a bank
                     double out[8];
+                    uint32_t lo[8], hi[8];
+                    int be0[8];
+                    const int e_base = 56 + Erow - 2154;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        // the two lightest accumulators as one number (2^-56 of the row and column
-                        // maxima below the rounding); the others are exact integers
-                        const float t56 = fmaf(__uint_as_float(t[6][e]), 0.00390625f, __uint_as_float(t[5][e]));
-                        int a[6];
+                        float a[kDig];
 #pragma unroll
-                        for (int i = 0; i < 5; ++i) a[i] = __float2int_rn(__uint_as_float(t[i][e]));
-                        a[5] = __float2int_rn(t56);
-                        const long long hi = (long long)(a[0] * 256 + a[1]) << 32;
-                        const long long lo = ((long long)a[2] * 256 + a[3]) * 65536 + ((long long)a[4] * 256 + a[5]);
-                        const int n = n0 + e;
-                        const int Et = n < prm.N ? __ldg(prm.et + (size_t)un.set * prm.et_ld + n) : 0;
-                        out[e] = Erow >= kExpNan ? __longlong_as_double(0x7FF8000000000000ll)
-                                                 : scaled_i64(hi + lo, 56 + Erow + Et - 2154);
+                        for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(t[i][e]);
+                        if (NM >= 6)
+                            acc_sum_small(a, lo[e], hi[e]);
+                        else
+                            acc_sum<NM, 0>(a, lo[e], hi[e]);
+                        if (!THETA)
+                            asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(lo[e]), "+r"(hi[e]) : "r"(g0_lo), "r"(g0_hi));
+                        be0[e] = e_base + Et[e] + 1084;
                     }
+                    // exponents in the middle of the range keep every result normal
+                    bool odd = !THETA ? (unsigned)(Erow - 200) > 1600u : Erow >= kExpNan;
+                    if (THETA) {
 #pragma unroll
-                    for (int cpc = 0; cpc < 4; ++cpc)
-                        *reinterpret_cast<double2 *>(stage + lane * 64 + ((cpc ^ ((lane >> 1) & 3)) << 4)) =
-                            make_double2(out[2 * cpc], out[2 * cpc + 1]);
-                    __syncwarp();
+                        for (int e = 0; e < 8; ++e) odd |= (unsigned)(be0[e] - 64) > 1900u;
+                    }
+                    if ((!scaled_row<8>(lo, hi, be0, out) || odd) && base) {
+                        // small integers (zeros among them), rows near the ends of the range or with a NaN
 #pragma unroll
-                    for (int r8 = 0; r8 < 4; ++r8) {
-                        const int rr = 8 * r8 + (lane >> 2), cpc = lane & 3, n = n0 + 2 * cpc;
-                        const double2 x =
-                            *reinterpret_cast<const double2 *>(stage + rr * 64 + ((cpc ^ ((rr >> 1) & 3)) << 4));
-                        const int row = 32 * q4 + rr;
-                        double *dst = nullptr;
-                        if (!prm.theta) {
-                            if (un.row0 + row < prm.R) dst = prm.dst + (un.row0 + row) * prm.n_p;
-                        } else {
-                            const int a = un.set ? row >> 6 : 0, i = (int)un.row0 + (un.set ? row & 63 : row);
-                            if (i < prm.n_r)
-                                dst = prm.dst + ((size_t)i * prm.P + (un.set ? 2 * un.set - 1 + a : 0)) * prm.ldJ;
-                        }
-                        if (dst) {
-                            if (prm.vec && n + 1 < prm.N) {
-                                if (prm.theta)
-                                    *reinterpret_cast<double2 *>(dst + n) = x;  // read again by the next step
-                                else
-                                    __stcs(reinterpret_cast<double2 *>(dst + n), x);
-                            } else {
-                                if (n < prm.N) dst[n] = x.x;
-                                if (n + 1 < prm.N) dst[n + 1] = x.y;
+                        for (int e = 0; e < 8; ++e) out[e] = scaled_i64_slow(lo[e], hi[e], be0[e] - 1084, Erow);
+                    }
+                    if (THETA || prm.tma) {
+                        // the warp's box of 32 rows x 8 columns: 64-byte rows, 16-byte pieces permuted
+                        // by the TMA's 64-byte swizzle
+                        uint8_t *box = sOut + warp * kBoxX;
+                        if (lane == 0) bulk_wait_read_all();  // the box before has left
+                        __syncwarp();
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+                            *reinterpret_cast<double2 *>(box + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) =
+                                make_double2(out[2 * c], out[2 * c + 1]);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (THETA) {
+                                const int r0 = 32 * q4, a = un.set ? r0 >> 6 : 0;
+                                const int i = (int)un.row0 + (un.set ? r0 & 63 : r0);
+                                if (i < prm.n_r && n0 < prm.N)
+                                    tma_store_3d(&tm_out, smem_u32(box), n0, un.set ? 2 * un.set - 1 + a : 0, i);
+                            } else if (n0 < prm.N && un.row0 + 32 * q4 < prm.R) {
+                                tma_store_2d_hint(&tm_out, smem_u32(box), n0, (int)(un.row0 + 32 * q4), policy);
                             }
+                            bulk_commit();
                         }
+                    } else if (out_row) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (n0 + e < prm.N) out_row[n0 + e] = out[e];
                     }
-                    __syncwarp();
-                }
-                // the pair's accumulators have been read, so both splits' MMAs are complete
-                if (un.n_chunks > 1 && ok) {
-                    ok = warp_all(mbar_wait(smem_u32(a_free), freed & 1, abort_flag, prm.err));
-                    ++freed;
                 }
             }
         }
+        if (lane == 0) bulk_wait_all();
     }
     tc_fence_before();
     __syncthreads();
@@ -1008,14 +1251,14 @@ int ceil_log2(int x)
 // a column m = 0 of its own).
 bool plan_contract(int K, int N, int own0, Fp64Contract &c)
 {
-    const int Nt = ceil16(N);
+    const int Nt = half_cols(N, 0) + half_cols(N, 1);
     c.n_steps = (K + 15) / 16;
     c.n_chunks = (c.n_steps + kChunkSteps - 1) / kChunkSteps;
-    c.ds = std::max(1, ceil_log2(K));
-    c.cols_max = N + own0;
-    c.nacc = kDig * Nt + (own0 ? 16 : 0) <= 256 ? 2 : 1;
+    c.ds = c.n_chunks == 1 ? 0 : c.n_chunks <= 4 ? 2 : c.n_chunks <= 16 ? 4 : ceil_log2(c.n_chunks);
+    c.cols_max = Nt + own0;
+    c.nacc = N <= kHalf ? 2 : 1;
     c.slot_b = (kDig * Nt + (own0 ? kRows0 : 0)) * 32;
-    if (Nt > kNtMax || c.ds > 31) return false;
+    if (N > kNtMax || c.ds > 31) return false;
     const int fixed = (c.n_chunks > 1 ? c.cols_max * 1024 : 0) + 4 * 128 * 4 + 512;
     for (auto d : {std::pair<int, int>{4, 4}, {4, 3}, {3, 3}, {3, 2}, {2, 2}}) {
         c.ns_a = d.first;
@@ -1029,11 +1272,11 @@ bool plan_contract(int K, int N, int own0, Fp64Contract &c)
 bool plan_expand(int K, Fp64Expand &x)
 {
     if (K > kExpandKMax) return false;
-    const int steps = (K + 15) / 16;
-    x.a_steps = steps <= 6 ? steps : (steps + 1) / 2;
-    const int fixed = x.a_steps * kStepA2 + kWorkWarps * 2048 + 8 * 128 * 4 + 512;
-    for (x.ns_b = 6; x.ns_b >= 2; --x.ns_b) {
-        x.smem = fixed + x.ns_b * kRowsX * 32;
+    const int steps = std::max(1, (K + 15) / 16);
+    x.a_steps = steps <= 5 ? steps : (steps + 1) / 2;
+    const int fixed = x.a_steps * kStepA2 + kWorkWarps * kBoxX + 8 * 128 * 4 + 1024 + 256;
+    for (x.ns_b = 8; x.ns_b >= 2; --x.ns_b) {
+        x.smem = fixed + 2 * x.ns_b * kRowsX * 32;
         if (x.smem <= kSmemMax) return true;
     }
     return false;
@@ -1062,7 +1305,7 @@ bool plan_fp64_tc(mp_mesh *m)
     }
     // below 16 azimuthal cells (axisymmetric meshes have one) a 16-wide K step is mostly padding
     // and the sums are short: CUDA cores
-    f.phi_on = m->n_p >= 16 && plan_contract(m->n_p, f.pass_cols, f.m0, f.ph_c) && plan_expand(m->P, f.ph_x);
+    f.phi_on = m->n_p >= 16 && plan_contract(m->n_p, f.pass_cols, f.m0, f.ph_c) && plan_expand(m->P - 1, f.ph_x);
     f.on = 1;
     return true;
 }
@@ -1085,7 +1328,7 @@ size_t fp64_tc_arena(mp_mesh *m)
     const int n_blk = (m->n_t + kNtX - 1) / kNtX;
     for (int s = 0; s < n_sets; ++s) {
         oc[s] = c;
-        c += (unsigned long long)f.th_c.n_steps * kDig * ceil16(set_cols(s, L)) * 32;
+        c += (unsigned long long)f.th_c.n_steps * kDig * (half_cols(set_cols(s, L), 0) + half_cols(set_cols(s, L), 1)) * 32;
     }
     for (int mm = 0; mm <= L; ++mm) {
         ox[mm] = x;
@@ -1096,18 +1339,47 @@ size_t fp64_tc_arena(mp_mesh *m)
     f.o_tab_c = take(c);
     f.o_tab_x = take(x);
     f.o_tab_pc = take(f.phi_on ? f.npass * pstep : 0);
-    f.o_tab_px = take(f.phi_on ? (size_t)((m->n_p + kNtX - 1) / kNtX) * ((m->P + 15) / 16) * kRowsX * 32 : 0);
+    f.o_tab_px = take(f.phi_on ? (size_t)((m->n_p + kNtX - 1) / kNtX) * std::max(1, (m->P - 1 + 15) / 16) * kRowsX * 32 : 0);
     f.o_off = take(f.h_off.size() * sizeof(unsigned long long));
-    f.o_et_c = take((size_t)n_sets * (kNtMax + 1) * 4);
-    f.o_et_x = take((size_t)(L + 1) * m->n_t * 4);
-    f.o_et_pc = take((size_t)f.npass * (kNtMax + 1) * 4);
-    f.o_et_px = take((size_t)m->n_p * 4);
+    f.o_et_c = take((size_t)n_sets * kEtLd * 4);
+    f.o_et_x = take((size_t)(L + 1) * round_up(m->n_t, kNtX) * 4);
+    f.o_et_pc = take((size_t)f.npass * kEtLd * 4);
+    f.o_bound = take(4 * sizeof(int));
+    f.o_et_px = take((size_t)round_up(m->n_p, kNtX) * 4);
     return at;
 }
 
 static const unsigned long long *fp64_off(const mp_mesh *m, int which)
 {
     return reinterpret_cast<const unsigned long long *>(m->fp.arena + m->fp.o_off) + (size_t)which * m->fp.off_ld;
+}
+
+// The contraction's variants: theta or phi step, 32-byte loads, the bits dropped from a chain's sum
+// (none for one chain; 2 for up to 4, 4 for up to 16, the number of bits at run time beyond) and,
+// for several chains, whether the table keeps the first four accumulators below 2^22.
+template <int NM>
+static void (*contract_kernel_nm(int theta, int vec, int ds, int n_chunks))(ContractParams)
+{
+    auto pick = [&](auto k0, auto k2, auto k4, auto kr) {
+        return n_chunks == 1 ? k0 : ds == 2 ? k2 : ds == 4 ? k4 : kr;
+    };
+    if (theta)
+        return pick(k64_contract_tc<true, true, 0, 2>, k64_contract_tc<true, true, 2, NM>,
+                    k64_contract_tc<true, true, 4, NM>, k64_contract_tc<true, true, -1, 2>);
+    return vec ? pick(k64_contract_tc<false, true, 0, 2>, k64_contract_tc<false, true, 2, NM>,
+                      k64_contract_tc<false, true, 4, NM>, k64_contract_tc<false, true, -1, 2>)
+               : pick(k64_contract_tc<false, false, 0, 2>, k64_contract_tc<false, false, 2, NM>,
+                      k64_contract_tc<false, false, 4, NM>, k64_contract_tc<false, false, -1, 2>);
+}
+static void (*contract_kernel(int theta, int vec, int ds, int n_chunks, int small))(ContractParams)
+{
+    return small ? contract_kernel_nm<4>(theta, vec, ds, n_chunks) : contract_kernel_nm<2>(theta, vec, ds, n_chunks);
+}
+
+static void (*expand_kernel(int theta, int nm))(const CUtensorMap, ExpandParams)
+{
+    if (theta) return nm == 6 ? k64_expand_tc<true, 6> : nm == 3 ? k64_expand_tc<true, 3> : k64_expand_tc<true, 1>;
+    return nm == 6 ? k64_expand_tc<false, 6> : nm == 3 ? k64_expand_tc<false, 3> : k64_expand_tc<false, 1>;
 }
 
 cudaError_t launch_fp64_tc_tables(mp_mesh *m)
@@ -1121,21 +1393,43 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
     if (e != cudaSuccess) return e;
     auto build = [&](int kind, size_t tab, int off, size_t et, int et_ld, int n_max, int n_sets) {
         TabParams t{m->d_Ith, m->d_Iph, m->d_Iphc, m->d_dmu, f.arena + tab, fp64_off(m, off),
-                    reinterpret_cast<int *>(f.arena + et), kind, m->n_t, m->n_p, L, m->P, f.pass_cols, f.m0, et_ld};
+                    reinterpret_cast<int *>(f.arena + et), kind, m->n_t, m->n_p, L, m->P, f.pass_cols, f.m0, et_ld,
+                    reinterpret_cast<int *>(f.arena + f.o_bound) + kind};
         k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t, n_sets);
     };
-    build(TAB_CONTRACT, f.o_tab_c, 0, f.o_et_c, kNtMax + 1, std::min(L + 1, kNtMax), L + 1 + set_extra(L));
-    build(TAB_EXPAND_TH, f.o_tab_x, 1, f.o_et_x, m->n_t, m->n_t, L + 1);
+    build(TAB_CONTRACT, f.o_tab_c, 0, f.o_et_c, kEtLd, std::min(L + 1, kNtMax), L + 1 + set_extra(L));
+    build(TAB_EXPAND_TH, f.o_tab_x, 1, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
     if (f.phi_on) {
-        build(TAB_PROJECT, f.o_tab_pc, 2, f.o_et_pc, kNtMax + 1, f.pass_cols + f.m0, f.npass);
-        build(TAB_EXPAND_PH, f.o_tab_px, 3, f.o_et_px, m->n_p, m->n_p, 1);
+        build(TAB_PROJECT, f.o_tab_pc, 2, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
+        build(TAB_EXPAND_PH, f.o_tab_px, 3, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
     }
     // 227 KB of dynamic shared memory for the kernels of this file (per device)
-    e = cudaFuncSetAttribute(k64_contract_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k64_expand_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (e != cudaSuccess) return e;
+    for (int theta = 0; theta < 2; ++theta) {
+        for (int vec = 0; vec < 2; ++vec)
+            for (int v = 0; v < 8; ++v) {
+                const int ds = v < 6 ? (v >> 1) * 2 : 5;
+                e = cudaFuncSetAttribute((const void *)contract_kernel(theta, theta || vec, ds, ds ? 2 : 1, v & 1),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+                if (e != cudaSuccess) return e;
+            }
+        for (int nm : {1, 3, 6}) {
+            e = cudaFuncSetAttribute((const void *)expand_kernel(theta, nm), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kSmemMax);
+            if (e != cudaSuccess) return e;
+        }
+    }
     return cudaGetLastError();
+}
+
+cudaError_t fp64_tc_bounds(mp_mesh *m)
+{
+    int b[4] = {0, 0, 0, 0};
+    cudaError_t e = cudaMemcpy(b, m->fp.arena + m->fp.o_bound, sizeof(b), cudaMemcpyDeviceToHost);
+    m->fp.ph_c.small = b[TAB_PROJECT] < (1 << 22);
+    m->fp.th_c.small = b[TAB_CONTRACT] < (1 << 22);
+    m->fp.th_x.small = b[TAB_EXPAND_TH] < (1 << 22);
+    m->fp.ph_x.small = b[TAB_EXPAND_PH] < (1 << 22);
+    return e;
 }
 
 static cudaError_t launch_contract(mp_mesh *m, int theta, const double *src, double *dst, const char *name)
@@ -1150,7 +1444,6 @@ static cudaError_t launch_contract(mp_mesh *m, int theta, const double *src, dou
     p.et = reinterpret_cast<const int *>(f.arena + (theta ? f.o_et_c : f.o_et_pc));
     p.err = m->d_err;
     p.R = m->R;
-    p.theta = theta;
     p.n_r = m->n_r, p.n_t = m->n_t, p.n_p = m->n_p, p.L = m->L, p.KL = m->KL, p.P = m->P, p.ldJ = f.ldJ;
     p.K = theta ? m->n_t : m->n_p;
     p.n_steps = c.n_steps, p.n_chunks = c.n_chunks, p.ds = c.ds;
@@ -1158,14 +1451,15 @@ static cudaError_t launch_contract(mp_mesh *m, int theta, const double *src, dou
     p.n_groups = (m->n_r + 63) / 64, p.n_groups0 = (m->n_r + 127) / 128;
     const int extra = set_extra(m->L);
     p.n_units = theta ? p.n_groups0 * (extra ? 2 : 1) + (m->L + std::max(0, extra - 1)) * p.n_groups : (int)((m->R + 127) / 128) * f.npass;
-    p.et_ld = kNtMax + 1;
+    p.et_ld = kEtLd;
     p.ns_a = c.ns_a, p.ns_b = c.ns_b, p.nacc = c.nacc, p.slot_b = c.slot_b, p.cols_max = c.cols_max;
     p.scale = 12.566370614359172954 * m->G;
-    // 16-byte loads where every row starts on a 16-byte boundary (and K is even)
-    p.vec = theta ? (m->n_t % 2 == 0) : (m->n_p % 2 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0);
+    // 32-byte loads where every row starts on a 32-byte boundary
+    const bool vec = theta || (m->n_p % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 31) == 0);
+    auto kern = contract_kernel(theta, vec, c.ds, c.n_chunks, c.small);
     cudaEvent_t ev;
     prof_begin(m, name, &ev);
-    cudaError_t e = launch_pdl(k64_contract_tc, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreads), c.smem,
+    cudaError_t e = launch_pdl(kern, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreadsC), c.smem,
                                m->stream, p);
     prof_end(m, name, ev);
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1183,22 +1477,33 @@ static cudaError_t launch_expand(mp_mesh *m, int theta, const double *src, doubl
     p.et = reinterpret_cast<const int *>(f.arena + (theta ? f.o_et_x : f.o_et_px));
     p.err = m->d_err;
     p.R = m->R;
-    p.theta = theta;
     p.n_r = m->n_r, p.n_t = m->n_t, p.n_p = m->n_p, p.L = m->L, p.P = m->P, p.ldJ = f.ldJ, p.ldI = f.ldI;
     p.N = theta ? m->n_t : m->n_p;
     p.n_blk = (p.N + kNtX - 1) / kNtX;
     p.n_groups = (m->n_r + 63) / 64, p.n_groups0 = (m->n_r + 127) / 128;
-    p.et_ld = theta ? m->n_t : m->n_p;
+    p.et_ld = round_up(p.N, kNtX);
     p.a_steps = x.a_steps, p.ns_b = x.ns_b;
     const int tiles = (int)((m->R + 127) / 128), pairs = (p.n_blk + 1) / 2;
     // fewer tiles than SMs: a tile's columns go to several CTAs (each splits the tile's A)
     p.n_split = theta ? 1 : std::max(1, std::min(pairs, m->num_sms / std::max(1, tiles)));
     p.n_units = theta ? p.n_groups0 + m->L * p.n_groups : tiles * p.n_split;
-    p.vec = theta || (m->n_p % 2 == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0);
+    // TMA stores where the rows' starts are multiples of 16 bytes
+    p.tma = theta || (m->n_p % 2 == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0);
+    CUtensorMap map = theta ? m->tm_G64 : m->tm_phi;
+    if (!theta && p.tma && m->tm_phi_ptr != dst) {
+        if (make_map_f64_rows(&m->tm_phi, dst, m->R, m->n_p, 32, 8) != MP_OK) return cudaErrorInvalidValue;
+        m->tm_phi_ptr = dst;
+        map = m->tm_phi;
+    }
     cudaEvent_t ev;
     prof_begin(m, name, &ev);
-    cudaError_t e = launch_pdl(k64_expand_tc, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreads), x.smem,
-                               m->stream, p);
+    // leading accumulators below 2^22: all where the table's digits keep them there (l_max up to
+    // about 35), else by the length of the chains (one more pair of digits each)
+    const int K = theta ? m->L + 1 : m->P - 1;
+    const int nm = x.small ? 6 : 3 * K < 256 ? 3 : 1;
+    auto kern = expand_kernel(theta, nm);
+    cudaError_t e = launch_pdl(kern, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreadsX), x.smem,
+                               m->stream, map, p);
     prof_end(m, name, ev);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -62,9 +62,10 @@ struct SplitPlan {
 // offsets of their tables in one device allocation.
 struct Fp64Contract {
     int n_steps = 0, n_chunks = 0, ds = 0, cols_max = 0, nacc = 1, slot_b = 0, ns_a = 0, ns_b = 0, smem = 0;
+    int small = 0;  // the table keeps the leading accumulators below 2^22
 };
 struct Fp64Expand {
-    int a_steps = 0, ns_b = 0, smem = 0;
+    int a_steps = 0, ns_b = 0, smem = 0, small = 0;
 };
 struct Fp64Plan {
     int on = 0;      // theta stages (and the layouts F, G [n_r][P][ldJ], C [K_L][ldI])
@@ -73,7 +74,7 @@ struct Fp64Plan {
     Fp64Contract ph_c, th_c;
     Fp64Expand ph_x, th_x;
     size_t o_tab_c = 0, o_tab_x = 0, o_tab_pc = 0, o_tab_px = 0, o_off = 0, o_et_c = 0, o_et_x = 0, o_et_pc = 0,
-           o_et_px = 0, arena_bytes = 0;
+           o_et_px = 0, o_bound = 0, arena_bytes = 0;
     uint8_t *arena = nullptr;
     std::vector<unsigned long long> h_off;  // table offsets per order / pass, four lists of off_ld
 };
@@ -134,6 +135,7 @@ struct mp_mesh {
     double *d_F64 = nullptr;
     double *d_G64 = nullptr;
     mp::Fp64Plan fp;
+    CUtensorMap tm_G64{};      // [n_r][P][n_theta] of G in boxes of 32 shells x 8 polar cells
 
     // split path tables and workspace
     mp::SplitPlan plan;
@@ -262,6 +264,7 @@ cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double
 bool plan_fp64_tc(mp_mesh *m);             // false: sizes out of its range (l_max > 71)
 size_t fp64_tc_arena(mp_mesh *m);          // lays the tables out; bytes of the arena
 cudaError_t launch_fp64_tc_tables(mp_mesh *m);
+cudaError_t fp64_tc_bounds(mp_mesh *m);    // reads what the finished tables say about the accumulators
 cudaError_t launch_fp64_tc_project(mp_mesh *m, const double *rho);
 cudaError_t launch_fp64_tc_theta(mp_mesh *m);
 cudaError_t launch_fp64_tc_synth_theta(mp_mesh *m);
@@ -295,6 +298,11 @@ cudaError_t launch_gsynth_tc(mp_mesh *m);  // theta synthesis, m >= 1
 // tiled TMA map of a float32 array of up to 3 dimensions (innermost first)
 mp_status make_map_f32(CUtensorMap *map, const void *ptr, int rank, const unsigned long long *dims,
                        const unsigned long long *strides_bytes, const unsigned *box, int swizzle128);
+
+// tiled TMA map of [rows][cols] float64 in boxes of [box_rows][box_cols] (64- or 128-byte swizzle),
+// and of the float64 G [n_r][P][n_theta], rows ldJ apart, in boxes of 32 shells x 8 cells
+mp_status make_map_f64_rows(CUtensorMap *map, const void *ptr, long long rows, int cols, int box_rows, int box_cols);
+mp_status make_map_f64_G(CUtensorMap *map, const void *ptr, int n_r, int P, int n_t, int ldJ);
 
 // ---- gravitational source terms ----
 cudaError_t gravity_prepare(mp_mesh *m);  // stencils from the host edges (once per mesh)

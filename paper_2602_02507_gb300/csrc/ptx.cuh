@@ -90,6 +90,33 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The same, with a first test that does not suspend the thread and the budget looked at before
+// every suspended one (`budget`: wait_budget, read once a kernel): a budget of a few cycles runs out on any phase that is not complete at
+// the first test, however fast the pipeline is.
+__device__ __forceinline__ bool mbar_wait_tested(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
+                                                 long long budget)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    const long long t0 = clock64();
+    while (true) {
+        if (*abort_flag) return false;
+        if (clock64() - t0 > budget) {
+            *abort_flag = 1;
+            atomicOr(err, DEV_ERR_TIMEOUT);
+            return false;
+        }
+        if (mbar_try_wait(bar, parity)) return true;
+    }
+}
+
 // Position in a ring of mbarrier-guarded stages: index and phase advance together.
 struct Ring {
     int idx = 0;
@@ -174,6 +201,13 @@ __device__ __forceinline__ void tma_store_2d(const void *map, uint32_t src, int 
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map),
                  "r"(src), "r"(x), "r"(y)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_store_3d(const void *map, uint32_t src, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(map),
+                 "r"(src), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
 
@@ -291,6 +325,63 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
+}
+
+// One lane of a converged warp (always the same one), as 0 / 1.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(v));
+    return v;
+}
+
+// The two above for a converged warp whose `leader` lane (elect_one) issues: the operands are
+// then warp-uniform and go to the tensor core from uniform registers; under a lane test each
+// MMA first moved its operands there from the one lane's, about 100 cycles an MMA.  The
+// descriptors come as (low word, high word): only the low words change from one MMA to the next,
+// and a lone warp's instructions are what bounds a stream of small MMAs.
+__device__ __forceinline__ void umma_f16_warp(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                              uint32_t idesc, uint32_t accumulate, uint32_t leader)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}\n" ::"r"(d_tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(leader)
+        : "memory");
+}
+
+__device__ __forceinline__ void umma_commit_warp(uint32_t bar, uint32_t leader)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar),
+        "r"(leader)
+        : "memory");
+}
+
+// 32-byte load of four float64 (32-byte aligned address).
+__device__ __forceinline__ void ldg_f64x4(const double *p, double (&x)[4])
+{
+    asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3])
+                 : "l"(p));
+}
+
+// Moves registers of the block's launch allocation between its warpgroups (all four warps of a
+// warpgroup call it; the shares stay within the launch total).
+template <int R>
+__device__ __forceinline__ void setmaxnreg_inc()
+{
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
+}
+template <int R>
+__device__ __forceinline__ void setmaxnreg_dec()
+{
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
 }
 
 // 32 lanes x 4 / 8 / 16 consecutive 32-bit columns; thread t of the warp gets lane
