@@ -19,8 +19,10 @@
 // read through the cache (each value serves the six neighbouring differences:
 // rows j +- 1 and shells i +- 1 are read by nearby blocks while they are still
 // in L2); density, velocity and the outputs stream once (evict-first).  All
-// arithmetic is float64.
+// arithmetic is to float64 accuracy: the differences and their scalings in integers where that is
+// exact work (scaled_difference), the rest on the float64 pipe.
 #include <cmath>
+#include <cstring>
 
 #include "mp_internal.h"
 #include "ptx.cuh"
@@ -29,7 +31,76 @@ namespace mp {
 
 namespace {
 
-__global__ void __launch_bounds__(256) k_gravity(const double *__restrict__ phi, const double *__restrict__ rho,
+// (a - b) w in integer instructions where that is exact work: a and b of one sign and within 2^9
+// of each other, as neighbouring cells of a potential are, subtract exactly as 62-bit integers;
+// the difference (33 bits or more of them) is normalised, multiplied by w's significand (64 x 64
+// -> the upper 64 bits) and rounded to nearest once.  False for anything else (zeros, denormals,
+// infinities, NaN, a sign change, results near the ends of the range), which takes the float64
+// pipe.  That pipe issues one warp's instruction every 64 cycles a scheduler here and bounded the
+// kernel with 12 a cell; three differences and their scalings on the integer pipe leave it 6.
+__device__ __forceinline__ bool scaled_difference(double a, double b, const GradStencil &s, double &g)
+{
+    const uint32_t la = (uint32_t)__double2loint(a), ha = (uint32_t)__double2hiint(a);
+    const uint32_t lb = (uint32_t)__double2loint(b), hb = (uint32_t)__double2hiint(b);
+    // sign and exponent together: of values of different sign the fields are far apart
+    const int ea = (int)(ha >> 20), eb = (int)(hb >> 20), em = max(ea, eb);
+    const int sa = 9 + ea - em, sb = 9 + eb - em;
+    const uint32_t mah = (ha & 0xFFFFFu) | 0x100000u, mbh = (hb & 0xFFFFFu) | 0x100000u;
+    uint32_t dl, dh;
+    asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %5;"
+        : "=r"(dl), "=r"(dh)
+        : "r"(la << (sa & 31)), "r"(__funnelshift_l(la, mah, sa)), "r"(lb << (sb & 31)), "r"(__funnelshift_l(lb, mbh, sb)));
+    const uint32_t sg = (uint32_t)((int)dh >> 31);
+    uint32_t ul, uh;
+    asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %4;" : "=r"(ul), "=r"(uh) : "r"(dl ^ sg), "r"(dh ^ sg), "r"(sg));
+    const int n = __clz((int)uh);
+    const uint32_t n1 = __funnelshift_l(ul, uh, n), n0 = ul << (n & 31);
+    const unsigned long long t = (unsigned long long)n1 * s.w0 + __umulhi(n0, s.w0);
+    const unsigned long long v = (unsigned long long)n0 * s.w1 + (uint32_t)t;
+    const unsigned long long p = (unsigned long long)n1 * s.w1 + (uint32_t)(t >> 32) + (uint32_t)(v >> 32);
+    uint32_t pl = (uint32_t)p, ph = (uint32_t)(p >> 32);
+    // leading one to bit 62, then to bit 52 of the significand
+    const int top = (int)(ph >> 31);
+    pl = __funnelshift_r(pl, ph, top);
+    ph >>= top;
+    asm("add.cc.u32 %0, %0, 0x200;\n\taddc.u32 %1, %1, 0;" : "+r"(pl), "+r"(ph));
+    const int be = (em & 0x7FF) + s.we - 1022 - n + top;  // exponent field less one
+    const uint32_t rl = __funnelshift_r(pl, ph, 10), rh = (ph >> 10) + ((uint32_t)be << 20);
+    g = __hiloint2double((int)(rh | ((ha ^ sg) & 0x80000000u)), (int)rl);
+    return (sa | sb) >= 0 && (unsigned)((em & 0x7FF) - 64) < 1983u && uh != 0 && (unsigned)be < 2045u;
+}
+
+// (out of line: inlined, its instructions were issued for every cell and selected afterwards)
+__device__ __noinline__ double scaled_difference_f64(double a, double b, double w) { return (a - b) * w; }
+
+template <int V>
+__device__ __forceinline__ void load_cells(const double *p, double (&x)[V], bool stream)
+{
+    if (V == 2) {
+        const double2 t = stream ? __ldcs(reinterpret_cast<const double2 *>(p)) : __ldg(reinterpret_cast<const double2 *>(p));
+        x[0] = t.x;
+        x[V - 1] = t.y;
+    } else {
+        x[0] = stream ? __ldcs(p) : __ldg(p);
+    }
+}
+
+template <int V>
+__device__ __forceinline__ void store_cells(double *p, const double (&x)[V])
+{
+    if (V == 2)
+        __stcs(reinterpret_cast<double2 *>(p), make_double2(x[0], x[V - 1]));
+    else
+        __stcs(p, x[0]);
+}
+
+// V neighbouring azimuthal cells a thread: 2 where every row starts on a 16-byte boundary (half
+// the memory instructions, twice the loads in flight).  At 512 x 128 x 256, S and E: 381 us with
+// every operation on the float64 pipe; 294 with the differences on the integer pipe; 251 with
+// two cells a thread in blocks of 64 threads at 64 registers (260 in blocks of 128; 317 with
+// one cell; rows in a loop 296-301).  The float64 pipe's floor is now 163 us, HBM's 178.
+template <int V>
+__global__ void __launch_bounds__(256, V == 2 ? 4 : 6) k_gravity(const double *__restrict__ phi, const double *__restrict__ rho,
                                                  const double *__restrict__ v, double *__restrict__ grad,
                                                  double *__restrict__ S, double *__restrict__ E,
                                                  const GradStencil *__restrict__ st, int n_r, int n_t, int n_p,
@@ -42,28 +113,65 @@ __global__ void __launch_bounds__(256) k_gravity(const double *__restrict__ phi,
     const double *p_row = phi + row * n_p;
     const double *p_rlo = phi + ((long long)gr.lo * n_t + j) * n_p, *p_rhi = phi + ((long long)gr.hi * n_t + j) * n_p;
     const double *p_tlo = phi + ((long long)i * n_t + gt.lo) * n_p, *p_thi = phi + ((long long)i * n_t + gt.hi) * n_p;
-    for (int k = threadIdx.x; k < n_p; k += blockDim.x) {
-        const GradStencil gp = sp[k];
+    for (int k = V * threadIdx.x; k < n_p; k += V * blockDim.x) {
         const long long c = row * n_p + k;
-        const double g0 = (__ldg(p_rhi + k) - __ldg(p_rlo + k)) * gr.w;
-        const double g1 = (__ldg(p_thi + k) - __ldg(p_tlo + k)) * gt.w;
-        const double g2 = (__ldg(p_row + gp.hi) - __ldg(p_row + gp.lo)) * gp.w;
-        if (grad) {
-            __stcs(grad + c, g0);
-            __stcs(grad + N + c, g1);
-            __stcs(grad + 2 * N + c, g2);
+        // every load of the cells first
+        double hi[3][V], lo[3][V], nr[V], v0[V], v1[V], v2[V];
+        GradStencil gp[V];
+        load_cells<V>(p_rhi + k, hi[0], false);
+        load_cells<V>(p_rlo + k, lo[0], false);
+        load_cells<V>(p_thi + k, hi[1], false);
+        load_cells<V>(p_tlo + k, lo[1], false);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            gp[e] = sp[k + e];
+            hi[2][e] = __ldg(p_row + gp[e].hi);
+            lo[2][e] = __ldg(p_row + gp[e].lo);
         }
-        const double nr = -__ldcs(rho + c);
+        load_cells<V>(rho + c, nr, true);
+        if (E) {
+            load_cells<V>(v + c, v0, true);
+            load_cells<V>(v + N + c, v1, true);
+            load_cells<V>(v + 2 * N + c, v2, true);
+        }
+        double g[3][V];
+        bool fits = true;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            fits &= scaled_difference(hi[0][e], lo[0][e], gr, g[0][e]);
+            fits &= scaled_difference(hi[1][e], lo[1][e], gt, g[1][e]);
+            fits &= scaled_difference(hi[2][e], lo[2][e], gp[e], g[2][e]);
+            nr[e] = -nr[e];
+        }
+        if (!fits) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                g[0][e] = scaled_difference_f64(hi[0][e], lo[0][e], gr.w);
+                g[1][e] = scaled_difference_f64(hi[1][e], lo[1][e], gt.w);
+                g[2][e] = scaled_difference_f64(hi[2][e], lo[2][e], gp[e].w);
+            }
+        }
+        if (grad) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) store_cells<V>(grad + a * N + c, g[a]);
+        }
         if (S) {
-            const double s0 = nr * g0, s1 = nr * g1, s2 = nr * g2;
-            __stcs(S + c, s0);
-            __stcs(S + N + c, s1);
-            __stcs(S + 2 * N + c, s2);
-            // E = v^a S_a: the products are already there (12 float64 operations a cell, not 13)
-            if (E) __stcs(E + c, fma(__ldcs(v + 2 * N + c), s2, fma(__ldcs(v + N + c), s1, __ldcs(v + c) * s0)));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+#pragma unroll
+                for (int e = 0; e < V; ++e) g[a][e] *= nr[e];
+                store_cells<V>(S + a * N + c, g[a]);
+            }
+            if (E) {
+                // E = v^a S_a: the products are already there
+#pragma unroll
+                for (int e = 0; e < V; ++e) v0[e] = fma(v2[e], g[2][e], fma(v1[e], g[1][e], v0[e] * g[0][e]));
+                store_cells<V>(E + c, v0);
+            }
         } else if (E) {
-            const double vg = fma(__ldcs(v + 2 * N + c), g2, fma(__ldcs(v + N + c), g1, __ldcs(v + c) * g0));
-            __stcs(E + c, nr * vg);
+#pragma unroll
+            for (int e = 0; e < V; ++e) v0[e] = nr[e] * fma(v2[e], g[2][e], fma(v1[e], g[1][e], v0[e] * g[0][e]));
+            store_cells<V>(E + c, v0);
         }
     }
 }
@@ -130,6 +238,15 @@ void axis_stencil(const std::vector<double> &e, bool periodic, GradStencil *out)
         out[i].lo = lo;
         out[i].hi = hi;
         out[i].w = dx != 0.0 ? 1.0 / dx : 0.0;
+        unsigned long long b;
+        std::memcpy(&b, &out[i].w, sizeof(b));
+        const int e = (int)(b >> 52) & 0x7FF;
+        const unsigned long long m = (b << 11) | (1ull << 63);
+        const bool normal = out[i].w > 0.0 && e > 0 && e < 0x7FF;
+        out[i].w0 = normal ? (uint32_t)m : 0u;
+        out[i].w1 = normal ? (uint32_t)(m >> 32) : 0u;
+        out[i].we = normal ? e : -100000;
+        out[i].unused = 0;
     }
 }
 
@@ -159,9 +276,15 @@ cudaError_t launch_gravity(mp_mesh *m, const double *phi, const double *rho, con
         k_gravity_flat<<<(unsigned)((m->N + 255) / 256), 256, 0, m->stream>>>(phi, rho, v, grad, S, E, m->d_gst, m->n_r,
                                                                               m->n_t, m->n_p, m->N);
     } else {
-        const int threads = std::min(256, 32 * ((m->n_p + 31) / 32));
-        k_gravity<<<(unsigned)m->R, threads, 0, m->stream>>>(phi, rho, v, grad, S, E, m->d_gst, m->n_r, m->n_t,
-                                                             m->n_p, m->N);
+        const auto bits = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+        // two cells a thread where every row of every array starts on a 16-byte boundary (the arrays of
+        // three components are N cells apart) and a row still fills a warp
+        const bool pairs = m->n_p % 2 == 0 && m->n_p >= 64 &&
+                           ((bits(phi) | bits(rho) | bits(v) | bits(grad) | bits(S) | bits(E)) & 15) == 0;
+        const int cells = pairs ? m->n_p / 2 : m->n_p;
+        const int threads = std::min(pairs ? 64 : 256, 32 * ((cells + 31) / 32));
+        auto kern = pairs ? k_gravity<2> : k_gravity<1>;
+        kern<<<(unsigned)m->R, threads, 0, m->stream>>>(phi, rho, v, grad, S, E, m->d_gst, m->n_r, m->n_t, m->n_p, m->N);
     }
     prof_end(m, "gravity_sources", ev);
     return cudaGetLastError();

@@ -90,10 +90,13 @@ struct CbOut {
 };
 
 // Centred difference along one axis at one cell: (Phi[hi] - Phi[lo]) * w, w = 1 / (x_c[hi] - x_c[lo])
-// (0 where the derivative is zero)
-struct GradStencil {
+// (0 where the derivative is zero); w also as its significand with the leading one at bit 63
+// (w1:w0) and its exponent field we (a field no result accepts where w is 0)
+struct alignas(16) GradStencil {
     int lo, hi;
     double w;
+    uint32_t w0, w1;
+    int we, unused;
 };
 
 struct ProfileEntry {
