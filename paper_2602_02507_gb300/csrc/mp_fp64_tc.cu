@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                     const uint8_t *src = prm.tab + prm.off[un.set];
                     const uint32_t bytes = un.step_bytes();
                     for (int s = 0; s < prm.n_steps; ++s, rb.next(prm.ns_b)) {
-                        ok = mbar_wait_tested(smem_u32(&b_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
+                        ok = mbar_wait(smem_u32(&b_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&b_full[rb.idx]);
                         mbar_arrive_expect_tx(bar, bytes);
@@ -563,31 +563,31 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                 const uint32_t d_off = mine == 1 ? 256u : own ? (uint32_t)(kDig * un.Nt[0]) : 0u;
                 for (int c = 0; c < prm.n_chunks && ok; ++c, ++it) {
                     const int b = prm.nacc == 2 ? it & 1 : 0, nth = prm.nacc == 2 ? it >> 1 : it;
-                    ok = warp_all(mbar_wait_tested(smem_u32(&acc_empty[b]), (nth & 1) ^ 1, abort_flag, prm.err, budget));
+                    ok = warp_all(mbar_wait(smem_u32(&acc_empty[b]), (nth & 1) ^ 1, abort_flag, prm.err, budget));
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d0 = tmem_base + (uint32_t)b * acc_stride + d_off;
                     const int steps = min(kChunkSteps, prm.n_steps - c * kChunkSteps);
                     for (int s = 0; s < steps; ++s, ra.next(prm.ns_a), rb.next(prm.ns_b)) {
-                        ok = warp_all(mbar_wait_tested(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err, budget) &&
-                                      mbar_wait_tested(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err, budget));
+                        ok = warp_all(mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err, budget) &&
+                                      mbar_wait(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err, budget));
                         if (!ok) break;
                         const uint32_t a_lo = a_lo0 + (uint32_t)ra.idx * (kSlotA1 / 16);
                         const uint32_t b_lo = b_lo0 + (uint32_t)(rb.idx * (prm.slot_b / 16));
                         if (n == kHalf) {
 #pragma unroll
                             for (int i = 0; i < kDig; ++i)
-                                umma_f16_warp(d0 + (uint32_t)(i * kHalf), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
+                                umma_warp(d0 + (uint32_t)(i * kHalf), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
                                               idesc_f16_f32(128, (kDig - i) * kHalf), (s | i) != 0, leader);
                         } else if (n == 16) {
 #pragma unroll
                             for (int i = 0; i < kDig; ++i)
-                                umma_f16_warp(d0 + (uint32_t)(i * 16), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
+                                umma_warp(d0 + (uint32_t)(i * 16), a_lo + i * (kDigA1 / 16), a_hi, b_lo, b_hi,
                                               idesc_f16_f32(128, (kDig - i) * 16), (s | i) != 0, leader);
                         } else if (own) {
 #pragma unroll
                             for (int i = 0; i < kDig; ++i)
-                                umma_f16_warp(d0, a_lo + i * (kDigA1 / 16), a_hi, b_lo + i * 32, b_hi,
+                                umma_warp(d0, a_lo + i * (kDigA1 / 16), a_hi, b_lo + i * 32, b_hi,
                                               idesc_f16_f32(128, 16), (s | i) != 0, leader);
                         }
                         umma_commit_warp(smem_u32(&a_empty[ra.idx]), leader);
@@ -668,8 +668,8 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                     if (pu >= 0 && ok) {
                         const ContractUnit un = contract_unit<THETA>(prm, pu);
                         const int b = prm.nacc == 2 ? (it - 1) & 1 : 0, nth = prm.nacc == 2 ? (it - 1) >> 1 : it - 1;
-                        ok = warp_all(mbar_wait_tested(smem_u32(&e_full[(it - 1) & 3]), ((it - 1) >> 2) & 1, abort_flag, prm.err, budget) &&
-                                      mbar_wait_tested(smem_u32(&acc_full[b]), nth & 1, abort_flag, prm.err, budget));
+                        ok = warp_all(mbar_wait(smem_u32(&e_full[(it - 1) & 3]), ((it - 1) >> 2) & 1, abort_flag, prm.err, budget) &&
+                                      mbar_wait(smem_u32(&acc_full[b]), nth & 1, abort_flag, prm.err, budget));
                         if (!ok) break;
                         tc_fence_after();
                         const int row = 32 * q4 + lane;
@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                     for (int s0 = 0; s0 < kDrainAt; ++s0) load_step(src, lim, s0, v[s0]);
                 }
                 if (s < steps) {
-                    ok = ok && warp_all(mbar_wait_tested(smem_u32(&a_empty[ra.idx]), ra.phase ^ 1, abort_flag, prm.err, budget));
+                    ok = ok && warp_all(mbar_wait(smem_u32(&a_empty[ra.idx]), ra.phase ^ 1, abort_flag, prm.err, budget));
                     if (!ok) break;
                     uint8_t *dst = sA + (size_t)ra.idx * kSlotA1 + a_off;
                     uint32_t wl[4], wh[4], d0[kDig], d1[kDig];
@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                     if (nb >= nbs) continue;
                     const uint8_t *from = src + (size_t)(g + nb) * un.steps * kSlotB;
                     for (int s = 0; s < un.steps; ++s, rb.next(prm.ns_b)) {
-                        ok = mbar_wait_tested(smem_u32(&my_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
+                        ok = mbar_wait(smem_u32(&my_empty[rb.idx]), rb.phase ^ 1, abort_flag, prm.err, budget);
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&my_full[rb.idx]);
                         mbar_arrive_expect_tx(bar, kSlotB);
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                 const int nbs = min(2, un.blk1 - un.pair(gi));
                 for (int ch = 0; ch < un.n_chunks && ok; ++ch) {
                     if (un.n_chunks > 1 || gi == 0) {
-                        ok = warp_all(mbar_wait_tested(smem_u32(a_full), conv & 1, abort_flag, prm.err, budget));
+                        ok = warp_all(mbar_wait(smem_u32(a_full), conv & 1, abort_flag, prm.err, budget));
                         if (!ok) break;
                         ++conv;
                     }
@@ -979,19 +979,19 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                     for (int nb = 0; nb < nbs && ok; ++nb) {
                         if (((blk + nb) & 1) != mine) continue;
                         if (ch == 0) {
-                            ok = warp_all(mbar_wait_tested(smem_u32(&acc_empty[mine]), (((blk + nb) >> 1) & 1) ^ 1, abort_flag,
+                            ok = warp_all(mbar_wait(smem_u32(&acc_empty[mine]), (((blk + nb) >> 1) & 1) ^ 1, abort_flag,
                                                            prm.err, budget));
                             if (!ok) break;
                             tc_fence_after();
                         }
                         uint32_t a_lo = a_lo0;
                         for (int s = s0; s < s1; ++s, rb.next(prm.ns_b), a_lo += kStepA2 / 16) {
-                            ok = warp_all(mbar_wait_tested(smem_u32(&my_full[rb.idx]), rb.phase, abort_flag, prm.err, budget));
+                            ok = warp_all(mbar_wait(smem_u32(&my_full[rb.idx]), rb.phase, abort_flag, prm.err, budget));
                             if (!ok) break;
                             const uint32_t b_lo = b_lo0 + (uint32_t)rb.idx * (kSlotB / 16);
 #pragma unroll
                             for (int i = 0; i < kDig; ++i)
-                                umma_f16_warp(d0 + (uint32_t)(i * kNtX), a_lo + i * (kDigA2 / 16), a_hi, b_lo, b_hi,
+                                umma_warp(d0 + (uint32_t)(i * kNtX), a_lo + i * (kDigA2 / 16), a_hi, b_lo, b_hi,
                                               idesc_f16_f32(128, (kDig - i) * kNtX), (s | i) != 0, leader);
                             umma_commit_warp(smem_u32(&my_empty[rb.idx]), leader);
                         }
@@ -1065,7 +1065,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
             row_max[cg * 128] = mx;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(m_full));
-            ok = warp_all(mbar_wait_tested(smem_u32(m_full), lu & 1, abort_flag, prm.err, budget));
+            ok = warp_all(mbar_wait(smem_u32(m_full), lu & 1, abort_flag, prm.err, budget));
             if (!ok) break;
             mx = max(max(row_max[0], row_max[128]), max(row_max[256], row_max[384]));
             int E = (int)(mx >> 20), E0 = 0;
@@ -1110,7 +1110,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
             // A for the K steps of piece ch, once the MMAs of the piece before have read theirs
             auto split = [&](int ch) -> bool {
                 if (splits > 0 &&
-                    !warp_all(mbar_wait_tested(smem_u32(a_free), (splits - 1) & 1, abort_flag, prm.err, budget)))
+                    !warp_all(mbar_wait(smem_u32(a_free), (splits - 1) & 1, abort_flag, prm.err, budget)))
                     return false;
                 ++splits;
                 const int s0 = ch * un.chunk_steps, s1 = min(un.steps, s0 + un.chunk_steps);
@@ -1140,7 +1140,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                     for (int ch = 0; ch < un.n_chunks && ok; ++ch) ok = split(ch);
                 for (int nb = 0; nb < nbs && ok; ++nb, ++blk) {
                     const int b = blk & 1;
-                    ok = warp_all(mbar_wait_tested(smem_u32(&acc_full[b]), (blk >> 1) & 1, abort_flag, prm.err, budget));
+                    ok = warp_all(mbar_wait(smem_u32(&acc_full[b]), (blk >> 1) & 1, abort_flag, prm.err, budget));
                     if (!ok) break;
                     tc_fence_after();
                     uint32_t t[kDig][8];

@@ -37,8 +37,8 @@ constexpr int kBM = 128;      // rows per tile (UMMA M)
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // bf16 product terms (a_term, b_term) accumulated per K step.
-__constant__ int c_prod_a[6] = {0, 0, 1, 0, 1, 2};
-__constant__ int c_prod_b[6] = {0, 1, 0, 2, 1, 0};
+__host__ __device__ constexpr int prod_a(int i) { return i == 2 || i == 4 ? 1 : i == 5 ? 2 : 0; }
+__host__ __device__ constexpr int prod_b(int i) { return i == 1 || i == 4 ? 1 : i == 3 ? 2 : 0; }
 
 
 // ----------------------------------------------------------------------------
@@ -207,52 +207,53 @@ __global__ void __launch_bounds__(kProjThreads, 1) k_proj_tc(const __grid_consta
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32(kBM, Npad);
-            const uint32_t b_term = (uint32_t)Npad * (BK * 2);
-            Ring ro, rb;
-            int lt = 0;
-            bool ok = true;
-            if (prm.b_resident && (int)blockIdx.x < prm.n_tiles) ok = mbar_wait(smem_u32(&b_full[0]), 0, abort_flag, prm.err);
-            for (int tile = blockIdx.x; tile < prm.n_tiles && ok; tile += gridDim.x, ++lt) {
-                const int b = lt & 1;
-                ok = mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err);
+        const uint32_t leader = elect_one();
+        const uint32_t idesc = idesc_bf16_f32(kBM, Npad);
+        const uint32_t b_term = (uint32_t)Npad * (BK * 2);
+        Ring ro, rb;
+        int lt = 0;
+        bool ok = true;
+        const uint64_t ad0 = sdesc_noswizzle(smem_u32(sA), 128, SBO), bd0 = sdesc_noswizzle(smem_u32(sB), 128, SBO);
+        const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32), b_lo0 = (uint32_t)bd0, b_hi = (uint32_t)(bd0 >> 32);
+        if (prm.b_resident && (int)blockIdx.x < prm.n_tiles)
+            ok = warp_all(mbar_wait(smem_u32(&b_full[0]), 0, abort_flag, prm.err));
+        for (int tile = blockIdx.x; tile < prm.n_tiles && ok; tile += gridDim.x, ++lt) {
+            const int b = lt & 1;
+            ok = warp_all(mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d_buf = tmem_base + (uint32_t)b * acc_stride;
+            for (int it = 0; it < prm.n_kc; ++it, ro.next(NS_O)) {
+                const uint32_t d_tmem = d_buf + (uint32_t)((it % nacc) * Npad);
+                ok = warp_all(mbar_wait(smem_u32(&o_full[ro.idx]), ro.phase, abort_flag, prm.err) &&
+                              (prm.b_resident || mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err)));
                 if (!ok) break;
-                tc_fence_after();
-                const uint32_t d_buf = tmem_base + (uint32_t)b * acc_stride;
-                for (int it = 0; it < prm.n_kc; ++it, ro.next(NS_O)) {
-                    const uint32_t d_tmem = d_buf + (uint32_t)((it % nacc) * Npad);
-                    ok = mbar_wait(smem_u32(&o_full[ro.idx]), ro.phase, abort_flag, prm.err) &&
-                         (prm.b_resident || mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err));
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t a_base = smem_u32(sA + (size_t)ro.idx * A_TERMS * A_TERM_BYTES);
-                    const int bslot = prm.b_resident ? rotated_chunk(it, tile, prm.n_kc) : rb.idx;
-                    const uint32_t b_base = smem_u32(sB + (size_t)bslot * prm.bload);
+                const uint32_t a_lo = a_lo0 + (uint32_t)(ro.idx * (A_TERMS * A_TERM_BYTES / 16));
+                const int bslot = prm.b_resident ? rotated_chunk(it, tile, prm.n_kc) : rb.idx;
+                const uint32_t b_lo = b_lo0 + (uint32_t)bslot * (uint32_t)(prm.bload / 16);
 #pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks) {
+                for (int ks = 0; ks < BK / 16; ++ks) {
 #pragma unroll
-                        for (int pi = 0; pi < NPROD; ++pi) {
-                            const uint64_t ad =
-                                sdesc_noswizzle(a_base + c_prod_a[pi] * A_TERM_BYTES + ks * 256, 128, SBO);
-                            const uint64_t bd = sdesc_noswizzle(b_base + c_prod_b[pi] * b_term + ks * 256, 128, SBO);
-                            umma_bf16(d_tmem, ad, bd, idesc, (it >= nacc) || ((ks | pi) != 0));
-                        }
-                    }
-                    umma_commit(smem_u32(&o_empty[ro.idx]));
-                    if (!prm.b_resident) {
-                        umma_commit(smem_u32(&b_empty[rb.idx]));
-                        rb.next(NS_B);
+                    for (int pi = 0; pi < NPROD; ++pi) {
+                        umma_warp(d_tmem, a_lo + (prod_a(pi) * A_TERM_BYTES + ks * 256) / 16, a_hi,
+                                       b_lo + (prod_b(pi) * b_term + ks * 256) / 16, b_hi, idesc,
+                                       (it >= nacc) || ((ks | pi) != 0), leader);
                     }
                 }
-                if (!ok) break;
-                umma_commit(smem_u32(&acc_full[b]));
+                umma_commit_warp(smem_u32(&o_empty[ro.idx]), leader);
+                if (!prm.b_resident) {
+                    umma_commit_warp(smem_u32(&b_empty[rb.idx]), leader);
+                    rb.next(NS_B);
+                }
             }
-            umma_commit(smem_u32(drain));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
-            }
+            if (!ok) break;
+            umma_commit_warp(smem_u32(&acc_full[b]), leader);
         }
+        umma_commit_warp(smem_u32(drain), leader);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+        }
+        __syncwarp();
     } else {
         // ---------------- converters + epilogue
         const int cw = warp - 3, grp = cw / kGroupWarps, qd = warp & 3, half = (cw >> 2) & 1;
@@ -930,60 +931,59 @@ __global__ void __launch_bounds__(synth::THREADS, 1)
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32(kBM, NC);
-            const uint32_t sbo_a = (uint32_t)Kpad * 16;
-            const uint32_t a_term_bytes = (uint32_t)kBM * Kpad * 2;
-            Ring ra, rb;
-            uint32_t u = 0;
-            bool ok = true;
-            if (prm.b_resident && blockIdx.x < n_units) ok = mbar_wait(smem_u32(&b_full[0]), 0, abort_flag, prm.err);
-            for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x, ra.next(NS_A)) {
-                const int nc = unit % prm.n_nc;
-                ok = mbar_wait(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err);
+        const uint32_t leader = elect_one();
+        const uint32_t idesc = idesc_bf16_f32(kBM, NC);
+        const uint32_t sbo_a = (uint32_t)Kpad * 16;
+        const uint32_t a_term_bytes = (uint32_t)kBM * Kpad * 2;
+        Ring ra, rb;
+        uint32_t u = 0;
+        bool ok = true;
+        const uint64_t ad0 = sdesc_noswizzle(smem_u32(sA), 128, sbo_a), bd0 = sdesc_noswizzle(smem_u32(sB), 128, 256);
+        const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32), b_lo0 = (uint32_t)bd0, b_hi = (uint32_t)(bd0 >> 32);
+        if (prm.b_resident && blockIdx.x < n_units)
+            ok = warp_all(mbar_wait(smem_u32(&b_full[0]), 0, abort_flag, prm.err));
+        for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x, ra.next(NS_A)) {
+            const int nc = unit % prm.n_nc;
+            ok = warp_all(mbar_wait(smem_u32(&a_full[ra.idx]), ra.phase, abort_flag, prm.err));
+            if (!ok) break;
+            const uint32_t a_lo1 = a_lo0 + (uint32_t)ra.idx * (uint32_t)(a_stage / 16);
+            {
+                const int buf = u & 1;
+                ok = warp_all(mbar_wait(smem_u32(&acc_empty[buf]), ((u >> 1) & 1) ^ 1, abort_flag, prm.err));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a_base0 = smem_u32(sA + (size_t)ra.idx * a_stage);
-                {
-                    const int buf = u & 1;
-                    ok = mbar_wait(smem_u32(&acc_empty[buf]), ((u >> 1) & 1) ^ 1, abort_flag, prm.err);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_stride;
-                    for (int kk = 0; kk < nkk; ++kk) {
-                        uint32_t b_base;
-                        if (prm.b_resident) {
-                            b_base = smem_u32(sB + (size_t)(nc * nkk + kk) * prm.bload);
-                        } else {
-                            ok = mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err);
-                            if (!ok) break;
-                            tc_fence_after();
-                            b_base = smem_u32(sB + (size_t)rb.idx * prm.bload);
-                        }
-                        const uint32_t a_base = a_base0 + (uint32_t)(kk * 256);
-#pragma unroll
-                        for (int pi = 0; pi < NPROD; ++pi) {
-                            const uint64_t ad = sdesc_noswizzle(a_base + c_prod_a[pi] * a_term_bytes, 128, sbo_a);
-                            const uint64_t bd = sdesc_noswizzle(b_base + (uint32_t)(c_prod_b[pi] * NC * 32), 128, 256);
-                            umma_bf16(d_tmem, ad, bd, idesc, (kk | pi) != 0);
-                        }
-                        if (!prm.b_resident) {
-                            umma_commit(smem_u32(&b_empty[rb.idx]));
-                            rb.next(NS_B);
-                        }
+                const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_stride;
+                for (int kk = 0; kk < nkk; ++kk) {
+                    int bslot = nc * nkk + kk;
+                    if (!prm.b_resident) {
+                        ok = warp_all(mbar_wait(smem_u32(&b_full[rb.idx]), rb.phase, abort_flag, prm.err));
+                        if (!ok) break;
+                        bslot = rb.idx;
                     }
-                    if (!ok) break;
-                    umma_commit(smem_u32(&acc_full[buf]));
-                    ++u;
+                    const uint32_t a_lo = a_lo1 + (uint32_t)(kk * 16);
+                    const uint32_t b_lo = b_lo0 + (uint32_t)bslot * (uint32_t)(prm.bload / 16);
+#pragma unroll
+                    for (int pi = 0; pi < NPROD; ++pi) {
+                        umma_warp(d_tmem, a_lo + prod_a(pi) * (a_term_bytes / 16), a_hi,
+                                       b_lo + (uint32_t)(prod_b(pi) * NC * 2), b_hi, idesc, (kk | pi) != 0, leader);
+                    }
+                    if (!prm.b_resident) {
+                        umma_commit_warp(smem_u32(&b_empty[rb.idx]), leader);
+                        rb.next(NS_B);
+                    }
                 }
                 if (!ok) break;
-                umma_commit(smem_u32(&a_empty[ra.idx]));
+                umma_commit_warp(smem_u32(&acc_full[buf]), leader);
+                ++u;
             }
-            umma_commit(smem_u32(drain));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
-            }
+            if (!ok) break;
+            umma_commit_warp(smem_u32(&a_empty[ra.idx]), leader);
         }
+        umma_commit_warp(smem_u32(drain), leader);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+        }
+        __syncwarp();
     } else {
         // ---------------- epilogue: accumulators -> Phi
         const int cw = warp - 2, qd = warp & 3, quarter = cw >> 2;

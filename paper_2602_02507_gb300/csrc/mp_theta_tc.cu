@@ -35,8 +35,8 @@ namespace mp {
 namespace {
 
 // bf16 products accumulated per K step: (dynamic-operand term, table term)
-__constant__ int c_pa[6] = {0, 0, 1, 0, 1, 2};
-__constant__ int c_pb[6] = {0, 1, 0, 2, 1, 0};
+__host__ __device__ constexpr int prod_a(int i) { return i == 2 || i == 4 ? 1 : i == 5 ? 2 : 0; }
+__host__ __device__ constexpr int prod_b(int i) { return i == 1 || i == 4 ? 1 : i == 3 ? 2 : 0; }
 
 __host__ __device__ inline int round16(int x) { return (x + 15) / 16 * 16; }
 
@@ -144,48 +144,49 @@ __global__ void __launch_bounds__(thc::THREADS, 1) k_theta_tc(const __grid_const
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            Ring rs, ro;
-            int lt = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x, ++lt) {
-                const int m = 1 + u / prm.n_groups;
-                const int Nm = round16(prm.L + 1 - m);
-                const uint32_t idesc = idesc_bf16_f32(128, Nm);
-                const uint32_t b_term = (uint32_t)Nm * 64;
-                const int b = lt & 1;
-                ok = mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err);
+        const uint32_t leader = elect_one();
+        const uint64_t ad0 = sdesc_noswizzle(smem_u32(sA), 128, SBO), td0 = sdesc_noswizzle(smem_u32(sS) + F_BYTES, 128, SBO);
+        const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32), t_lo0 = (uint32_t)td0, t_hi = (uint32_t)(td0 >> 32);
+        Ring rs, ro;
+        int lt = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x, ++lt) {
+            const int m = 1 + u / prm.n_groups;
+            const int Nm = round16(prm.L + 1 - m);
+            const uint32_t idesc = idesc_bf16_f32(128, Nm);
+            const uint32_t b_term = (uint32_t)Nm * 64;
+            const int b = lt & 1;
+            ok = warp_all(mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d_buf = tmem_base + (uint32_t)b * acc_stride;
+            for (int c = 0; c < prm.n_kc; ++c, rs.next(NS_S), ro.next(NS_O)) {
+                ok = warp_all(mbar_wait(smem_u32(&o_full[ro.idx]), ro.phase, abort_flag, prm.err) &&
+                              mbar_wait(smem_u32(&s_full[rs.idx]), rs.phase, abort_flag, prm.err));
                 if (!ok) break;
-                tc_fence_after();
-                const uint32_t d_buf = tmem_base + (uint32_t)b * acc_stride;
-                for (int c = 0; c < prm.n_kc; ++c, rs.next(NS_S), ro.next(NS_O)) {
-                    ok = mbar_wait(smem_u32(&o_full[ro.idx]), ro.phase, abort_flag, prm.err) &&
-                         mbar_wait(smem_u32(&s_full[rs.idx]), rs.phase, abort_flag, prm.err);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t a_base = smem_u32(sA + (size_t)ro.idx * A_TERMS * A_TERM_BYTES);
-                    const uint32_t t_base = smem_u32(sS + (size_t)rs.idx * prm.stage_bytes + F_BYTES);
-                    const uint32_t d_tmem = d_buf + (uint32_t)((c % nacc) * Nmax);
+                const uint32_t a_lo = a_lo0 + (uint32_t)(ro.idx * (A_TERMS * A_TERM_BYTES / 16));
+                const uint32_t t_lo = t_lo0 + (uint32_t)rs.idx * (prm.stage_bytes / 16);
+                const uint32_t d_tmem = d_buf + (uint32_t)((c % nacc) * Nmax);
 #pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks) {
+                for (int ks = 0; ks < BK / 16; ++ks) {
 #pragma unroll
-                        for (int pi = 0; pi < NPROD; ++pi) {
-                            const uint64_t ad = sdesc_noswizzle(a_base + c_pa[pi] * A_TERM_BYTES + ks * 256, 128, SBO);
-                            const uint64_t bd = sdesc_noswizzle(t_base + c_pb[pi] * b_term + ks * 256, 128, SBO);
-                            umma_bf16(d_tmem, ad, bd, idesc, (c >= nacc) || ((ks | pi) != 0));
-                        }
+                    for (int pi = 0; pi < NPROD; ++pi) {
+                        umma_warp(d_tmem, a_lo + (prod_a(pi) * A_TERM_BYTES + ks * 256) / 16, a_hi,
+                                       t_lo + (prod_b(pi) * b_term + ks * 256) / 16, t_hi, idesc,
+                                       (c >= nacc) || ((ks | pi) != 0), leader);
                     }
-                    umma_commit(smem_u32(&o_empty[ro.idx]));
-                    umma_commit(smem_u32(&s_empty[rs.idx]));
                 }
-                if (!ok) break;
-                umma_commit(smem_u32(&acc_full[b]));
+                umma_commit_warp(smem_u32(&o_empty[ro.idx]), leader);
+                umma_commit_warp(smem_u32(&s_empty[rs.idx]), leader);
             }
-            umma_commit(smem_u32(drain));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
-            }
+            if (!ok) break;
+            umma_commit_warp(smem_u32(&acc_full[b]), leader);
         }
+        umma_commit_warp(smem_u32(drain), leader);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+        }
+        __syncwarp();
     } else {
         // ---------------- converters (F -> bf16 terms) + epilogue (accumulators -> moments)
         const int cw = warp - 2, grp = cw / GROUP_WARPS, qd = warp & 3, half = (cw >> 2) & 1;
@@ -398,48 +399,49 @@ __global__ void __launch_bounds__(gsc::THREADS, 1) k_gsynth_tc(const GsynthTcPar
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32(128, N);
-            Ring rs;
-            int lt = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x, ++lt) {
-                const int mg = u / prm.n_jb / prm.n_sg;
-                const int b = lt & 1;
-                ok = mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err);
-                if (!ok) break;
-                tc_fence_after();
-                for (int ml = 0; ml < ORDERS && ok; ++ml) {
-                    const int m = ORDERS * mg + 1 + ml;
-                    if (m > prm.L) break;
-                    const int n_kcm = (prm.L + 1 - m + BK - 1) / BK;
-                    const uint32_t d_tmem = tmem_base + (uint32_t)b * acc_stride + (uint32_t)(ml * N);
-                    for (int kc = 0; kc < n_kcm; ++kc, rs.next(NS_S)) {
-                        ok = mbar_wait(smem_u32(&s_full[rs.idx]), rs.phase, abort_flag, prm.err);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t t_base = smem_u32(sS + (size_t)rs.idx * prm.stage_bytes);
-                        const uint32_t c_base = t_base + tbytes;
+        const uint32_t leader = elect_one();
+        const uint32_t idesc = idesc_bf16_f32(128, N);
+        const uint64_t td0 = sdesc_noswizzle(smem_u32(sS), 128, SBO);
+        const uint32_t t_lo0 = (uint32_t)td0, d_hi = (uint32_t)(td0 >> 32);
+        Ring rs;
+        int lt = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x, ++lt) {
+            const int mg = u / prm.n_jb / prm.n_sg;
+            const int b = lt & 1;
+            ok = warp_all(mbar_wait(smem_u32(&acc_empty[b]), ((lt >> 1) & 1) ^ 1, abort_flag, prm.err));
+            if (!ok) break;
+            tc_fence_after();
+            for (int ml = 0; ml < ORDERS && ok; ++ml) {
+                const int m = ORDERS * mg + 1 + ml;
+                if (m > prm.L) break;
+                const int n_kcm = (prm.L + 1 - m + BK - 1) / BK;
+                const uint32_t d_tmem = tmem_base + (uint32_t)b * acc_stride + (uint32_t)(ml * N);
+                for (int kc = 0; kc < n_kcm; ++kc, rs.next(NS_S)) {
+                    ok = warp_all(mbar_wait(smem_u32(&s_full[rs.idx]), rs.phase, abort_flag, prm.err));
+                    if (!ok) break;
+                    const uint32_t t_lo = t_lo0 + (uint32_t)rs.idx * (prm.stage_bytes / 16);
+                    const uint32_t c_lo = t_lo + tbytes / 16;
 #pragma unroll
-                        for (int ks = 0; ks < BK / 16; ++ks) {
+                    for (int ks = 0; ks < BK / 16; ++ks) {
 #pragma unroll
-                            for (int pi = 0; pi < NPROD; ++pi) {
-                                const uint64_t ad = sdesc_noswizzle(t_base + c_pb[pi] * T_TERM_BYTES + ks * 256, 128, SBO);
-                                const uint64_t bd = sdesc_noswizzle(c_base + c_pa[pi] * c_term + ks * 256, 128, SBO);
-                                umma_bf16(d_tmem, ad, bd, idesc, ((kc | ks | pi) != 0));
-                            }
+                        for (int pi = 0; pi < NPROD; ++pi) {
+                            umma_warp(d_tmem, t_lo + (prod_b(pi) * T_TERM_BYTES + ks * 256) / 16, d_hi,
+                                           c_lo + (prod_a(pi) * c_term + ks * 256) / 16, d_hi, idesc,
+                                           (kc | ks | pi) != 0, leader);
                         }
-                        umma_commit(smem_u32(&s_empty[rs.idx]));
                     }
+                    umma_commit_warp(smem_u32(&s_empty[rs.idx]), leader);
                 }
-                if (!ok) break;
-                umma_commit(smem_u32(&acc_full[b]));
             }
-            umma_commit(smem_u32(drain));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
-            }
+            if (!ok) break;
+            umma_commit_warp(smem_u32(&acc_full[b]), leader);
         }
+        umma_commit_warp(smem_u32(drain), leader);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(drain), 0) && clock64() - t0 < MP_WAIT_BUDGET_CYCLES) {
+        }
+        __syncwarp();
     } else {
         // ---------------- epilogue: accumulators -> bf16 terms of the phi-synthesis A operand
         const int ew = warp - 2, qd = warp & 3, sh = ew >> 2;

@@ -74,37 +74,27 @@ __device__ __forceinline__ long long wait_budget(const int *err)
     return b > 0 ? b : MP_WAIT_BUDGET_CYCLES;
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err)
+//
+// The first test does not suspend the thread, and the budget is looked at before every
+// suspended one: a budget of a few cycles runs out on any phase that is not complete at the
+// first test, however fast the pipeline is.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    const long long budget = wait_budget(err);
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > budget) {
-            *abort_flag = 1;
-            atomicOr(err, DEV_ERR_TIMEOUT);
-            return false;
-        }
-    }
-}
-
-// The same, with a first test that does not suspend the thread and the budget looked at before
-// every suspended one (`budget`: wait_budget, read once a kernel): a budget of a few cycles runs out on any phase that is not complete at
-// the first test, however fast the pipeline is.
-__device__ __forceinline__ bool mbar_wait_tested(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
-                                                 long long budget)
-{
-    uint32_t done;
+    uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
+        : "=r"(ok)
         : "r"(bar), "r"(parity)
         : "memory");
-    if (done) return true;
+    return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
+                                          long long budget)
+{
+    if (mbar_test_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
         if (*abort_flag) return false;
@@ -115,6 +105,13 @@ __device__ __forceinline__ bool mbar_wait_tested(uint32_t bar, uint32_t parity, 
         }
         if (mbar_try_wait(bar, parity)) return true;
     }
+}
+
+// The same with the budget read when a wait needs it.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err)
+{
+    if (mbar_test_wait(bar, parity)) return true;
+    return mbar_wait(bar, parity, abort_flag, err, wait_budget(err));
 }
 
 // Position in a ring of mbarrier-guarded stages: index and phase advance together.
@@ -307,26 +304,6 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 or fp16 inputs (as idesc says), fp32 accumulate, one
-// thread issues.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// Arrive once on the mbarrier when every tcgen05 op issued so far by this thread is done.
-__device__ __forceinline__ void umma_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
-}
-
 // One lane of a converged warp (always the same one), as 0 / 1.
 __device__ __forceinline__ uint32_t elect_one()
 {
@@ -335,12 +312,13 @@ __device__ __forceinline__ uint32_t elect_one()
     return v;
 }
 
-// The two above for a converged warp whose `leader` lane (elect_one) issues: the operands are
-// then warp-uniform and go to the tensor core from uniform registers; under a lane test each
-// MMA first moved its operands there from the one lane's, about 100 cycles an MMA.  The
-// descriptors come as (low word, high word): only the low words change from one MMA to the next,
-// and a lone warp's instructions are what bounds a stream of small MMAs.
-__device__ __forceinline__ void umma_f16_warp(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 or fp16 inputs (as idesc says), fp32 accumulate, issued
+// by the `leader` lane (elect_one) of a converged warp: the operands are then warp-uniform and go
+// to the tensor core from uniform registers; under a lane test each MMA first moved its operands
+// there from the one lane's, about 100 cycles an MMA.  The descriptors come as (low word, high
+// word): only the low words change from one MMA to the next, and a lone warp's instructions are
+// what bounds a stream of small MMAs.
+__device__ __forceinline__ void umma_warp(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                               uint32_t idesc, uint32_t accumulate, uint32_t leader)
 {
     asm volatile(
@@ -353,6 +331,7 @@ __device__ __forceinline__ void umma_f16_warp(uint32_t d_tmem, uint32_t alo, uin
         : "memory");
 }
 
+// Arrive once on the mbarrier when every tcgen05 op issued so far by this lane is done.
 __device__ __forceinline__ void umma_commit_warp(uint32_t bar, uint32_t leader)
 {
     asm volatile(
