@@ -94,36 +94,50 @@ __global__ void __launch_bounds__(256) k64_synth_phi(const double *__restrict__ 
 }
 
 // (a1) and (d2) for a few azimuthal cells, beside the tensor-core theta stages: F and G as
-// [n_r][P][ldJ], neighbouring threads on neighbouring polar cells.
-__global__ void __launch_bounds__(256) k64_project_few(const double *__restrict__ rho, const double *__restrict__ Iph,
+// [n_r][P][ldJ], neighbouring threads on neighbouring polar cells.  Each thread of the projection
+// takes kFewCols columns of its cell row (a block for each column made 19,000 blocks of one product
+// a thread at 471 x 128 x 1 cells, l_max = 20), and the synthesis sums in four chains: latency
+// bounds both (the projection 16.5 -> 12.7 us there).
+constexpr int kFewCols = 8;
+
+__global__ void __launch_bounds__(128) k64_project_few(const double *__restrict__ rho, const double *__restrict__ Iph,
                                                        double *__restrict__ F, int n_t, int n_p, int P, int ldJ,
                                                        int *err)
 {
-    const int i = blockIdx.x, p = blockIdx.y;
-    for (int j = threadIdx.x; j < n_t; j += blockDim.x) {
+    const int i = blockIdx.x, p0 = blockIdx.y * kFewCols, np = min(kFewCols, P - p0);
+    for (int j = threadIdx.x + blockIdx.z * blockDim.x; j < n_t; j += blockDim.x * gridDim.z) {
         const double *s = rho + ((size_t)i * n_t + j) * n_p;
-        double acc = 0.0;
+        double acc[kFewCols] = {};
         bool bad = false;
         for (int k = 0; k < n_p; ++k) {
             const double v = __ldg(s + k);
             bad |= !isfinite(v);
-            acc = fma(__ldg(Iph + (size_t)p * n_p + k), v, acc);
+#pragma unroll
+            for (int q = 0; q < kFewCols; ++q)
+                if (q < np) acc[q] = fma(__ldg(Iph + (size_t)(p0 + q) * n_p + k), v, acc[q]);
         }
-        if (bad && p == 0) atomicOr(err, DEV_ERR_NONFINITE);
-        F[((size_t)i * P + p) * ldJ + j] = acc;
+        if (bad && p0 == 0) atomicOr(err, DEV_ERR_NONFINITE);
+#pragma unroll
+        for (int q = 0; q < kFewCols; ++q)
+            if (q < np) F[((size_t)i * P + p0 + q) * ldJ + j] = acc[q];
     }
 }
 
-__global__ void __launch_bounds__(256) k64_synth_phi_few(const double *__restrict__ Gm, const double *__restrict__ Iphc,
+__global__ void __launch_bounds__(128) k64_synth_phi_few(const double *__restrict__ Gm, const double *__restrict__ Iphc,
                                                          double *__restrict__ phi, int n_t, int n_p, int P, int ldJ)
 {
     const int i = blockIdx.x;
     for (int c = threadIdx.x + blockIdx.y * blockDim.x; c < n_t * n_p; c += blockDim.x * gridDim.y) {
         const int k = c / n_t, j = c - k * n_t;
         const double *g = Gm + (size_t)i * P * ldJ + j;
-        double acc = 0.0;
-        for (int p = 0; p < P; ++p) acc = fma(__ldg(g + (size_t)p * ldJ), __ldg(Iphc + (size_t)p * n_p + k), acc);
-        phi[((size_t)i * n_t + j) * n_p + k] = acc;
+        double acc[4] = {};
+        int p = 0;
+        for (; p + 4 <= P; p += 4)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                acc[q] = fma(__ldg(g + (size_t)(p + q) * ldJ), __ldg(Iphc + (size_t)(p + q) * n_p + k), acc[q]);
+        for (; p < P; ++p) acc[0] = fma(__ldg(g + (size_t)p * ldJ), __ldg(Iphc + (size_t)p * n_p + k), acc[0]);
+        phi[((size_t)i * n_t + j) * n_p + k] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     }
 }
 
@@ -135,8 +149,9 @@ cudaError_t launch_fp64_project(mp_mesh *m, const double *rho)
     if (m->fp.on) {
         cudaEvent_t ev;
         prof_begin(m, "fp64_phi_project", &ev);
-        k64_project_few<<<dim3(m->n_r, m->P), std::min(256, round_up(m->n_t, 32)), 0, m->stream>>>(
-            rho, m->d_Iph, m->d_F64, m->n_t, m->n_p, m->P, m->fp.ldJ, m->d_err);
+        const int threads = std::min(128, round_up(m->n_t, 32));
+        k64_project_few<<<dim3(m->n_r, (m->P + kFewCols - 1) / kFewCols, (m->n_t + threads - 1) / threads), threads, 0,
+                          m->stream>>>(rho, m->d_Iph, m->d_F64, m->n_t, m->n_p, m->P, m->fp.ldJ, m->d_err);
         prof_end(m, "fp64_phi_project", ev);
         return cudaGetLastError();
     }
@@ -186,7 +201,8 @@ cudaError_t launch_fp64_synth(mp_mesh *m, double *phi)
         if (m->fp.phi_on) return launch_fp64_tc_synth_phi(m, phi);
         prof_begin(m, "fp64_phi_synth", &ev);
         const int cells = m->n_t * m->n_p;
-        k64_synth_phi_few<<<dim3(m->n_r, (cells + 255) / 256), std::min(256, round_up(cells, 32)), 0, m->stream>>>(
+        const int threads = std::min(128, round_up(cells, 32));
+        k64_synth_phi_few<<<dim3(m->n_r, (cells + threads - 1) / threads), threads, 0, m->stream>>>(
             m->d_G64, m->d_Iphc, phi, m->n_t, m->n_p, m->P, m->fp.ldJ);
         prof_end(m, "fp64_phi_synth", ev);
         return cudaGetLastError();

@@ -36,7 +36,7 @@
 // What bounds them: not the tensor core (about 40 % of the time at 1024 x 256 x 512 cells,
 // l_max = 32) nor HBM, but the integer instructions that split and rejoin the operands (half the
 // rate of float32's) and the hand-offs between the warps that issue them.  Measured there against
-// float64 on CUDA cores: (a1) 29.5 ms -> 724 us, (a2) 688 -> 98 us, (d1) 2143 -> 66 us, (d2)
+// float64 on CUDA cores: (a1) 29.5 ms -> 649 us, (a2) 688 -> 90 us, (d1) 2143 -> 66 us, (d2)
 // 13.9 ms -> 423 us; at 512 x 128 x 256, l_max = 16: 1918 -> 102, 76 -> 21, 200 -> 17, 891 -> 69 us.
 #include <algorithm>
 
@@ -240,6 +240,26 @@ __device__ __forceinline__ void acc_sum_small(const float (&t)[kDig], uint32_t &
     hi = (uint32_t)(v >> 32);
 }
 
+// One chain of several (DS >= 2) whose first three accumulators stay below 2^22 (the next two may
+// not, and are converted): the integers keep their offsets as in acc_sum_small, kChainOff in all.
+template <int DS>
+__device__ __forceinline__ unsigned long long acc_sum_chain(const float (&t)[kDig])
+{
+    constexpr float w5 = 1.0f / (1 << DS), w6 = w5 / 256.0f;
+    uint32_t a[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) a[i] = (uint32_t)__float_as_int(t[i] + 12582912.0f);
+    const uint32_t a5 = (uint32_t)__float_as_int(fmaf(t[6], w6, t[5] * w5) + 12582912.0f);
+    const uint32_t a3 = (uint32_t)__float2int_rn(t[3]), a4 = (uint32_t)__float2int_rn(t[4]);
+    return (unsigned long long)(a[2] * 256u + a3) * (65536u >> DS) + (a4 * (256u >> DS) + a5) +
+           (unsigned long long)(a[0] * 256u + a[1]) * ((1ull << 32) >> DS);
+}
+template <int DS>
+struct ChainOff {
+    static constexpr unsigned long long pair = 0x4B400000u * 257u, one = 0x4B400000u * 256u;  // modulo 2^32
+    static constexpr unsigned long long value = one * (65536u >> DS) + 0x4B400000u + pair * ((1ull << 32) >> DS);
+};
+
 // Eight results of one row at once: hi:lo 2^(e0 + et) as in scaled_i64, for integers of 33 bits or
 // more (the common case); false when one is smaller.
 template <int N>
@@ -272,7 +292,7 @@ struct TabParams {
     const unsigned long long *off;  // byte offset per set (pass, or order m)
     int *et;                        // column exponents, [set][et_ld]
     int kind, n_t, n_p, L, P, pass_cols, m0, et_ld;
-    int *bound;  // largest sum an accumulator can reach: expand, the sixth; contract, the fourth
+    int *bound;  // largest sum an accumulator can reach: expand, the sixth; contract, the third
 };
 
 // Sets of the theta contraction: order m = s, columns l = m .. m + 63, for s = 0 .. L; the
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n
             for (int i = 0; i < kDig; ++i) {
                 const int v = abs(__half2int_rn(__ushort_as_half((unsigned short)(d[i] & 0xFFFFu))));
                 (i < 6 ? s5 : s6) += v;
-                if (i < 4) s3 += v;
+                if (i < 3) s3 += v;
             }
             uint8_t *dst = base + (size_t)(k >> 4) * step + (k & 7) * 2;
             const int oct = (k >> 3) & 1;
@@ -615,19 +635,24 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
 
         // K step s of a chunk: `p` at the thread's first k of the chunk, `lim` terms left from it
         // (none or fewer past the last row)
+        bool whole = false;  // a whole chunk of a whole warp's rows: no bounds to look at
         auto load_step = [&](const double *p, int lim, int s, double (&x)[4]) {
-            if (VEC && lim > 16 * s + 3) {
+            if (VEC && whole) {
                 ldg_f64x4(p + 16 * s, x);
+            } else if (VEC) {  // (lim is a multiple of four)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[e] = 0.0;
+                if (lim > 16 * s) ldg_f64x4(p + 16 * s, x);
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) x[e] = lim > 16 * s + e ? __ldg(p + 16 * s + e) : 0.0;
             }
         };
-        auto chunk_at = [&](int u, int c, const double *&p, int &lim) {
+        // the thread's place in the first chunk of unit u
+        auto unit_at = [&](int u, const double *&p, int &lim) {
             p = u < prm.n_units ? contract_row<THETA>(prm, contract_unit<THETA>(prm, u), crow) : nullptr;
-            const int k = c * (16 * kChunkSteps) + 4 * quad;
-            lim = p ? prm.K - k : 0;
-            p += k;
+            lim = p ? (THETA ? prm.ldJ : prm.K) - 4 * quad : 0;  // (the cells past n_theta in a row of F are zeros)
+            p += 4 * quad;
         };
 
         Ring ra;
@@ -635,7 +660,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
         int u = blockIdx.x, c = 0, pu = -1, pc = 0;  // this item, the one before (not yet drained)
         const double *src;
         int lim;
-        chunk_at(u, c, src, lim);
+        unit_at(u, src, lim);
 #pragma unroll
         for (int s = 0; s < kChunkSteps; ++s) load_step(src, lim, s, v[s]);
         while (ok && (u < prm.n_units || pu >= 0)) {
@@ -658,7 +683,20 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
             __syncwarp();
             if (lane == 0 && steps) mbar_arrive(smem_u32(&e_full[it & 3]));
             const int e9 = E + 9;
-            chunk_at(u2, c2, src, lim);
+            if (c2) {
+                src += 16 * kChunkSteps;
+                lim -= 16 * kChunkSteps;
+            } else {
+                unit_at(u2, src, lim);
+            }
+            whole = VEC && warp_all(lim > 16 * (kChunkSteps - 1) + 3);
+            // the last step's loads of the next item are needed as soon as they are issued: they
+            // come from L2 then, where this has brought the item by that time
+            if (lim > 0) {
+                const double *pf = src + 28 * quad;
+                if (lim > 28 * quad) prefetch_l2(pf);
+                if (lim > 28 * quad + 16) prefetch_l2(pf + 16);
+            }
 #pragma unroll
             for (int s = 0; s < kChunkSteps; ++s) {
                 if (s == kDrainAt) {
@@ -688,10 +726,11 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                         }
                         const bool shifts = DS != 0 && !warp_all((sh_old | sh_new) == 0);
                         double *dst = nullptr;  // column n of the unit: dst + n ldJ, or dst + (col0 + n)^2
-                        if (!THETA) {
+                        if (!last) {
+                        } else if (!THETA) {
                             const long long r = un.row0 + row;
                             if (r < prm.R) {
-                                const int i = (int)(r / prm.n_t), j = (int)(r - (long long)i * prm.n_t);
+                                const int i = (int)((unsigned)r / (unsigned)prm.n_t), j = (int)r - i * prm.n_t;
                                 dst = prm.dst + ((size_t)i * prm.P + un.col0) * prm.ldJ + j;
                             }
                         } else {
@@ -705,13 +744,22 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                         // the last chunk, to `out`
                         auto result = [&](const float (&a)[kDig], long long *pa, int et, double *out, bool in) {
                             uint32_t lo, hi;
-                            acc_sum<NM, (DS > 0 ? DS : 0)>(a, lo, hi);
                             if (DS != 0) {
-                                long long x = (long long)(((unsigned long long)hi << 32) | lo);
-                                if (shifts) x >>= sh_new;
+                                long long x, o = 0;
                                 if (pc > 0) {
-                                    long long o = *pa;
+                                    o = *pa;
                                     if (shifts) o >>= sh_old;
+                                }
+                                if (DS > 0 && NM >= 3) {
+                                    x = (long long)acc_sum_chain<(DS > 0 ? DS : 2)>(a);
+                                    if (shifts)
+                                        x = ((x - (long long)ChainOff<(DS > 0 ? DS : 2)>::value) >> sh_new) + o;
+                                    else
+                                        x = x + o - (long long)ChainOff<(DS > 0 ? DS : 2)>::value;
+                                } else {
+                                    acc_sum<NM, (DS > 0 ? DS : 0)>(a, lo, hi);
+                                    x = (long long)(((unsigned long long)hi << 32) | lo);
+                                    if (shifts) x >>= sh_new;
                                     x += o;
                                 }
                                 if (!last) {
@@ -720,6 +768,8 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                                 }
                                 lo = (uint32_t)x;
                                 hi = (uint32_t)(x >> 32);
+                            } else {
+                                acc_sum<NM, 0>(a, lo, hi);
                             }
                             bool odd = Er >= kExpNan;
                             double x = scaled_i64(lo, hi, e_base + et, odd);
@@ -730,7 +780,33 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                         // groups of four columns, dealt to the four warps of a lane quarter (the
                         // padding up to Nt holds zeros); the column m = 0 of its own block, with its
                         // weights side by side, goes to the last of them
-                        for (int n = 4 * grp; n < un.N; n += 16) {
+                        const int n_first = 4 * grp;
+                        if (DS > 0 && NM >= 3 && !last && !shifts) {
+                            // the usual chain before the last, rows whose exponents agree: read all
+                            // seven sums and the integer so far at once, no result to look at
+                            for (int n = n_first; n < un.N; n += 16) {
+                                uint32_t t[kDig][4];
+                                const int hf = n >> 5, nt = un.Nt[hf];
+                                const uint32_t c0 = col + (uint32_t)(hf * 256 + (n & 31));
+#pragma unroll
+                                for (int i = 0; i < kDig; ++i) tmem_ld4(c0 + (uint32_t)(i * nt), t[i]);
+                                unsigned long long *pa = reinterpret_cast<unsigned long long *>(sAcc) + (size_t)n * 128 + row;
+                                unsigned long long o[4] = {0, 0, 0, 0};
+                                if (pc > 0) {
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) o[e] = pa[e * 128];
+                                }
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    float a[kDig];
+#pragma unroll
+                                    for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(t[i][e]);
+                                    pa[e * 128] = acc_sum_chain<(DS > 0 ? DS : 2)>(a) + o[e] - ChainOff<(DS > 0 ? DS : 2)>::value;
+                                }
+                            }
+                        } else
+                        for (int n = n_first; n < un.N; n += 16) {
                             uint32_t t[kDig][4];
                             const int hf = n >> 5, nt = un.Nt[hf];
                             const uint32_t c0 = col + (uint32_t)(hf * 256 + (n & 31));
@@ -1299,7 +1375,8 @@ bool plan_fp64_tc(mp_mesh *m)
     f.npass = (cols + kNtMax - 1) / kNtMax;
     f.pass_cols = (cols + f.npass - 1) / f.npass;
     if (f.npass > 1) f.pass_cols = std::min(kNtMax, ceil16(f.pass_cols));
-    if (m->L > 71 || !plan_contract(m->n_t, std::min(m->L + 1, kNtMax), 0, f.th_c) || !plan_expand(m->L + 1, f.th_x)) {
+    if (m->L > 71 || m->R >= (1LL << 31) || !plan_contract(m->n_t, std::min(m->L + 1, kNtMax), 0, f.th_c) ||
+        !plan_expand(m->L + 1, f.th_x)) {
         f = Fp64Plan();  // the CUDA-core path and its layouts
         return false;
     }
@@ -1356,7 +1433,7 @@ static const unsigned long long *fp64_off(const mp_mesh *m, int which)
 
 // The contraction's variants: theta or phi step, 32-byte loads, the bits dropped from a chain's sum
 // (none for one chain; 2 for up to 4, 4 for up to 16, the number of bits at run time beyond) and,
-// for several chains, whether the table keeps the first four accumulators below 2^22.
+// for several chains, whether the table keeps the first three accumulators below 2^22.
 template <int NM>
 static void (*contract_kernel_nm(int theta, int vec, int ds, int n_chunks))(ContractParams)
 {
@@ -1373,7 +1450,7 @@ static void (*contract_kernel_nm(int theta, int vec, int ds, int n_chunks))(Cont
 }
 static void (*contract_kernel(int theta, int vec, int ds, int n_chunks, int small))(ContractParams)
 {
-    return small ? contract_kernel_nm<4>(theta, vec, ds, n_chunks) : contract_kernel_nm<2>(theta, vec, ds, n_chunks);
+    return small ? contract_kernel_nm<3>(theta, vec, ds, n_chunks) : contract_kernel_nm<2>(theta, vec, ds, n_chunks);
 }
 
 static void (*expand_kernel(int theta, int nm))(const CUtensorMap, ExpandParams)

@@ -350,6 +350,8 @@ __device__ __forceinline__ void ldg_f64x4(const double *p, double (&x)[4])
                  : "l"(p));
 }
 
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Moves registers of the block's launch allocation between its warpgroups (all four warps of a
 // warpgroup call it; the shares stay within the launch total).
 template <int R>
