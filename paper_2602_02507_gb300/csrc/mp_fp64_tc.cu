@@ -533,7 +533,6 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
     const uint32_t acc_stride = prm.nacc == 2 ? 256 : 0;
-    pdl_trigger();
     pdl_wait();  // the source comes from the previous kernels
     const long long budget = wait_budget(prm.err);
 
@@ -990,7 +989,6 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
-    pdl_trigger();
     pdl_wait();  // the source comes from the previous kernels
     const long long budget = wait_budget(prm.err);
 

@@ -86,8 +86,7 @@ __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const
                                              const CbOut cbo, const double *__restrict__ off, size_t ldC)
 {
     __shared__ double wt[2][NT / 32];
-    // the next kernel's blocks may start (and copy their tables) while this one runs
-    pdl_trigger();
+    if (!cbo.cb) pdl_trigger();  // (the tensor-core synthesis is preceded by k_gsynth_m0: many blocks an SM)
     pdl_wait();  // A comes from the previous kernel
     const int q = blockIdx.x;
     int l = (int)sqrtf((float)q);
@@ -150,8 +149,7 @@ __global__ void __launch_bounds__(NT) k_scan_reg(const double *__restrict__ A, c
                                                  const CbOut cbo, const double *__restrict__ off, size_t ldC)
 {
     __shared__ double wt[2][NT / 32];
-    // the next kernel's blocks may start (and copy their tables) while this one runs
-    pdl_trigger();
+    if (!cbo.cb) pdl_trigger();  // (the tensor-core synthesis is preceded by k_gsynth_m0: many blocks an SM)
     pdl_wait();  // A comes from the previous kernel
     const int q = blockIdx.x;
     int l = (int)sqrtf((float)q);
@@ -235,7 +233,7 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
 {
     constexpr int NW = 4 * NT / 32;
     __shared__ double wt[2][NW][4];
-    pdl_trigger();
+    if (!cbo.cb) pdl_trigger();
     pdl_wait();  // A comes from the previous kernel
     const int sub = threadIdx.x & 3, c = threadIdx.x >> 2, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int q = 4 * blockIdx.x + sub;
@@ -397,8 +395,8 @@ __global__ void __launch_bounds__(1024, 1) k32_theta_pipe(const float *__restric
         mbar_arrive_expect_tx(smem_u32(&bars[0]), tab_bytes);
         bulk_load(smem_u32(sT), Ith, tab_bytes, smem_u32(&bars[0]));
     }
-    // the table copy overlaps the previous kernel's tail; F rows only after it completed
-    pdl_trigger();
+    // the table copy overlaps the previous kernel's tail; F rows only after it completed (no
+    // trigger: the radial scan has many blocks an SM)
     pdl_wait();
     if (tid == 0)
         for (int b = 0; b < 2; ++b)
@@ -691,8 +689,8 @@ bool theta_pipe_fits(const mp_mesh *m) { return theta_pipe_smem(m) <= 200 * 1024
 
 // Four columns per block when there are at least four such blocks per SM; 128 chunk
 // threads per column (512 per block), CH shells each.  Not beside the persistent theta
-// contraction of the split path: its blocks leave room for the small one-column scan
-// blocks to start early, not for these (that early start is worth more than coalescing).
+// contraction of the split path, whose moments are few: no gain there (eight meshes of up to
+// 768 x 192 x 384 solved together: 874 us with one column a block, 877 with four).
 static bool scan_q4_dispatch(mp_mesh *m, int want_f32)
 {
     if (m->KL < 4 * m->num_sms) return false;

@@ -70,6 +70,7 @@ struct ProjParams {
     long long R;
     int n_p, n_kc, Npad, n_tiles, ns_s, ns_o;
     int n_t, P, ldF;
+    int early_next;        // 1: the next kernel has one block per SM and may start early
     int nacc;              // tensor-memory accumulators per tile (K chunks dealt round-robin)
     int b_resident;        // 1: every table chunk stays in shared memory for the whole launch
     int ns_b;              // table ring slots (when not resident)
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kProjThreads, 1) k_proj_tc(const __grid_consta
     const uint32_t tmem_base = *tmem_holder;
     // barrier set-up, tensor memory and the table copy overlap the previous kernel's tail;
     // the density and the outputs are touched only after the previous kernel has completed
-    pdl_trigger();
+    if (prm.early_next) pdl_trigger();
     pdl_wait();
 
     if (warp == 0) {
@@ -1383,6 +1384,7 @@ cudaError_t launch_split_project(mp_mesh *m, const double *rho)
     prm.nacc = std::max(1, std::min(pl.proj_nacc, pl.proj_nacc_max));
     prm.b_resident = pl.proj_b_resident;
     prm.ns_b = pl.proj_ns_b;
+    prm.early_next = !pl.use_theta_tc && theta_pipe_fits(m);  // k32_theta_pipe; the others have many blocks an SM
     const int grid = std::min(prm.n_tiles, pl.proj_ctas);
     cudaEvent_t ev;
     prof_begin(m, "split_phi_project_tc", &ev);

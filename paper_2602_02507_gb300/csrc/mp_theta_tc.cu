@@ -113,7 +113,6 @@ __global__ void __launch_bounds__(thc::THREADS, 1) k_theta_tc(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
-    pdl_trigger();
     pdl_wait();  // F comes from the previous kernels
 
     if (warp == 0) {

@@ -167,7 +167,14 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Lets the next kernel on the stream start its blocks once every block of this
 // grid has issued the trigger or exited (so a block of this grid never waits
 // for resources held by waiting dependents); they still wait in pdl_wait for
-// this grid to complete.
+// this grid to complete.  Only before a kernel with one block per SM: blocks of a
+// kernel that fits several on an SM pile up on the SMs that this grid leaves free,
+// and run there one after another while the others idle.  Measured, a solve with the
+// trigger -> without: theta contraction before the radial scan 91.3 -> 82.4 us (301 x 99
+// x 180, l_max = 21, bf16x6), 3410 -> 3352 us (2048 x 512 x 1024, l_max = 64); scan and projection before the m = 0 kernels 470 -> 458 us (1024 x 256 x
+// 512, l_max = 32).  The other way round, projection before k32_theta_pipe: 85.1 without,
+// 84.2 with (512 x 128 x 256, l_max = 16).  The float64 tensor-core kernels do not
+// trigger either: 225 -> 204 us at 512 x 128 x 256 with moments, 130 -> 117 at 353 x 96 x 192.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
 // ---------------------------------------------------------------- TMA / bulk copies
