@@ -21,7 +21,7 @@
 //
 // The m = 0 column of both stages, the bulk of Phi, stays on CUDA cores in small kernels
 // of their own launched just before the tensor-core kernels: compensated float32 sums for
-// the contraction (a warp per shell), double-float for the synthesis (a thread per row).
+// the contraction, double-float for the synthesis.
 // The tensor core accumulates in float32 with truncation, which the monopole cannot afford.
 //
 // Roles per CTA of the tensor-core kernels (persistent, one CTA per SM): warp 0 issues the
@@ -510,62 +510,71 @@ __global__ void __launch_bounds__(gsc::THREADS, 1) k_gsynth_tc(const GsynthTcPar
 // ---------------------------------------------------------------------------- m = 0 columns
 // (a2) m = 0 as a register-tiled float32 GEMM with compensated sums:
 //   A[i][l^2] = scale sum_j Ith[t(l,0)][j] F[i][0][j]
-// Block (64 degrees, 16 shells) stages K chunks of 32 polar cells of both operands in
-// shared memory; thread (rg, cg) owns degrees rg + 16 a (a < 4) and shell cg; products are
-// summed over blocks of eight cells, block sums with Kahan compensation.
-constexpr int kM0Deg = 64, kM0Shells = 16, kM0K = 32, kM0Ld = kM0K + 4;
+// Block (16 NA degrees, 8 shells) brings K chunks of 32 polar cells of both operands to shared
+// memory; thread (rg, cg) owns degrees rg + 16 a (a < NA) and shell cg; products are summed over
+// blocks of eight cells, block sums with Kahan compensation.  Latency bounds it (a few MB of F):
+// two chunks ahead by cp.async, small blocks, so that nearly every SM has one at 1024 shells.
+// Measured with the launch: 12.0 -> 10.6 us at 1024 x 256 x 512 cells, l_max = 32, 25.0 -> 20.3
+// at 2048 x 512 x 1024, l_max = 64 (before: 64 degrees x 16 shells, one chunk ahead in registers).
+constexpr int kM0Shells = 8, kM0K = 32, kM0Ld = kM0K + 4, kM0Stages = 3, kM0Threads = 16 * kM0Shells;
 
 __device__ __forceinline__ float dot4f(float4 a, float4 b, float acc)
 {
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
 
-__global__ void __launch_bounds__(256) k_theta_m0(const ThetaTcParams prm)
+template <int NA>
+__global__ void __launch_bounds__(kM0Threads) k_theta_m0(const ThetaTcParams prm)
 {
-    __shared__ __align__(16) float sT[kM0Deg][kM0Ld];
-    __shared__ __align__(16) float sF[kM0Shells][kM0Ld];
-    // no early trigger: the tensor-core kernel that follows holds one CTA of shared memory
-    // per SM, which would leave this kernel's later blocks no room
-    pdl_wait();  // F comes from the previous kernel
-    const int tid = threadIdx.x, rg = tid >> 4, cg = tid & 15;
-    const int i0 = blockIdx.x * kM0Shells, l0 = blockIdx.y * kM0Deg;
-    float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
-    // the next chunk's table and F values are loaded into registers while this chunk is
-    // summed (two table float4s and, for the first 128 threads, one F float4 a thread)
-    float4 tv[2], fv = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto load = [&](int j0) {
+    __shared__ __align__(16) float sT[kM0Stages][16 * NA][kM0Ld];
+    __shared__ __align__(16) float sF[kM0Stages][kM0Shells][kM0Ld];
+    const int tid = threadIdx.x, rg = tid / kM0Shells, cg = tid % kM0Shells;
+    const int i0 = blockIdx.x * kM0Shells, l0 = blockIdx.y * (16 * NA);
+    const int n_c = (prm.n_t + kM0K - 1) / kM0K;
+    float s[NA], c[NA];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int e = tid + 256 * k, r = e >> 3, q = e & 7, l = l0 + r, j = j0 + 4 * q;
-            tv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (l <= prm.L && j < prm.ldF)
-                tv[k] = __ldg(reinterpret_cast<const float4 *>(prm.Ith32 + (size_t)tri(l, 0) * prm.ldF + j));
-        }
-        if (tid < kM0Shells * (kM0K / 4)) {
-            const int r = tid >> 3, q = tid & 7, i = i0 + r, j = j0 + 4 * q;
-            fv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i < prm.n_r && j < prm.ldF) fv = __ldg(reinterpret_cast<const float4 *>(prm.F + (size_t)i * prm.P * prm.ldF + j));
+    for (int a = 0; a < NA; ++a) s[a] = c[a] = 0.f;
+    // float4 q = tid % 8 of rows tid / 8 + 16 k of the table and of row tid / 8 (< 8) of F
+    const int r = tid >> 3, q = tid & 7;
+    auto load_table = [&](int ch) {
+        const int st = ch % kM0Stages, j = ch * kM0K + 4 * q;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) {
+            const int l = l0 + r + 16 * k;
+            const bool in = ch < n_c && l <= prm.L && j < prm.ldF;
+            cp_async16_zfill(smem_u32(&sT[st][r + 16 * k][4 * q]), in ? prm.Ith32 + (size_t)tri(l, 0) * prm.ldF + j : prm.Ith32,
+                             in ? 16u : 0u);
         }
     };
-    load(0);
-    for (int j0 = 0; j0 < prm.n_t; j0 += kM0K) {
-        __syncthreads();  // the previous chunk is consumed
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int e = tid + 256 * k;
-            *reinterpret_cast<float4 *>(&sT[e >> 3][4 * (e & 7)]) = tv[k];
-        }
-        if (tid < kM0Shells * (kM0K / 4)) *reinterpret_cast<float4 *>(&sF[tid >> 3][4 * (tid & 7)]) = fv;
-        __syncthreads();
-        if (j0 + kM0K < prm.n_t) load(j0 + kM0K);
+    auto load_source = [&](int ch) {
+        const int st = ch % kM0Stages, j = ch * kM0K + 4 * q, i = i0 + r;
+        if (r >= kM0Shells) return;
+        const bool in = ch < n_c && i < prm.n_r && j < prm.ldF;
+        cp_async16_zfill(smem_u32(&sF[st][r][4 * q]), in ? prm.F + (size_t)i * prm.P * prm.ldF + j : prm.F, in ? 16u : 0u);
+    };
+    load_table(0);
+    load_table(1);
+    pdl_trigger();
+    pdl_wait();  // F comes from the previous kernel
+    load_source(0);
+    cp_async_commit();
+    load_source(1);
+    cp_async_commit();
+    for (int ch = 0; ch < n_c; ++ch) {
+        cp_async_wait<1>();
+        __syncthreads();  // this chunk is there, the one before is consumed
+        load_table(ch + 2);
+        load_source(ch + 2);
+        cp_async_commit();
+        const int st = ch % kM0Stages;
 #pragma unroll
         for (int jb = 0; jb < kM0K; jb += 8) {
-            const float4 f0 = *reinterpret_cast<const float4 *>(&sF[cg][jb]);
-            const float4 f1 = *reinterpret_cast<const float4 *>(&sF[cg][jb + 4]);
+            const float4 f0 = *reinterpret_cast<const float4 *>(&sF[st][cg][jb]);
+            const float4 f1 = *reinterpret_cast<const float4 *>(&sF[st][cg][jb + 4]);
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const float4 t0 = *reinterpret_cast<const float4 *>(&sT[rg + 16 * a][jb]);
-                const float4 t1 = *reinterpret_cast<const float4 *>(&sT[rg + 16 * a][jb + 4]);
+            for (int a = 0; a < NA; ++a) {
+                const float4 t0 = *reinterpret_cast<const float4 *>(&sT[st][rg + 16 * a][jb]);
+                const float4 t1 = *reinterpret_cast<const float4 *>(&sT[st][rg + 16 * a][jb + 4]);
                 const float blk = dot4f(t1, f1, dot4f(t0, f0, 0.f));
                 const float y = blk - c[a];
                 const float t = s[a] + y;
@@ -574,48 +583,66 @@ __global__ void __launch_bounds__(256) k_theta_m0(const ThetaTcParams prm)
             }
         }
     }
+    cp_async_wait<0>();
     const int i = i0 + cg;
     if (i >= prm.n_r) return;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+    for (int a = 0; a < NA; ++a) {
         const int l = l0 + rg + 16 * a;
         if (l <= prm.L) prm.A[(size_t)i * prm.KL + (size_t)l * l] = prm.scale * f32_to_f64_alu(s[a] - c[a]);
     }
 }
 
 // (d1) m = 0 in double-float: G0[row] = (hi, lo) of sum_l (Ith[t(l,0)][j] / dmu_j) C[i][l^2]
-// for the rows (i, j) of a block of 128 polar cells and SB shells; the block's table slice
-// and coefficients sit in shared memory, thread (j, half) forms SB / 2 shells of cell j.
-__global__ void __launch_bounds__(256) k_gsynth_m0(const float2 *__restrict__ C0, const float2 *__restrict__ Itc0,
-                                                   float *__restrict__ G0, int n_r, int n_t, int L, int SB)
+// for the rows (i, j) of a block of 128 polar cells and SH shells, a cell a thread: the
+// coefficients sit in shared memory, the table is read once for the SH shells, a group of
+// kM0Ahead degrees ahead of the sums.  The float32 instructions of the sums bound it (12 for each
+// row and degree; 24 us at 2048 x 512 rows, l_max = 64), and at 1024 shells the latency of one
+// group after the other.  Measured with the launch: 14.3 -> 12.6 us at 1024 x 256 x 512 cells, l_max
+// = 32, 45.5 -> 40.2 at the larger size (before: the table in shared memory as well).
+constexpr int kM0Ahead = 8, kM0LMax = 128;
+
+template <int SH>
+__global__ void __launch_bounds__(128) k_gsynth_m0(const float2 *__restrict__ C0, const float2 *__restrict__ Itc0,
+                                                   float *__restrict__ G0, int n_r, int n_t, int L)
 {
-    extern __shared__ __align__(16) float2 sm0[];
-    float2 *sT = sm0;                          // [L + 1][128]
-    float2 *sC = sm0 + (size_t)(L + 1) * 128;  // [SB][L + 1]
-    const int tid = threadIdx.x;
-    const int j0 = blockIdx.x * 128, i0 = blockIdx.y * SB;
-    for (int e = tid; e < (L + 1) * 128; e += 256) {  // the static table, ahead of the wait
-        const int l = e >> 7, j = j0 + (e & 127);
-        sT[e] = j < n_t ? Itc0[(size_t)l * n_t + j] : make_float2(0.f, 0.f);
-    }
-    pdl_wait();  // C0 comes from the previous kernel (no early trigger: see k_theta_m0)
-    for (int e = tid; e < SB * (L + 1); e += 256) {
-        const int i = i0 + e / (L + 1);
-        sC[e] = i < n_r ? C0[(size_t)i0 * (L + 1) + e] : make_float2(0.f, 0.f);
+    __shared__ __align__(16) float2 sC[kM0LMax + 1][SH];
+    const int tid = threadIdx.x, j = blockIdx.y * blockDim.x + tid, i0 = blockIdx.x * SH;
+    const float2 *T = Itc0 + min(j, n_t - 1);
+    float2 t[kM0Ahead];
+#pragma unroll
+    for (int k = 0; k < kM0Ahead; ++k) t[k] = __ldg(T + (size_t)min(k, L) * n_t);  // static, ahead of the wait
+    pdl_trigger();
+    pdl_wait();  // C0 comes from the previous kernel
+    for (int e = tid; e < SH * (L + 1); e += blockDim.x) {
+        const int sh = e / (L + 1), l = e - sh * (L + 1);
+        sC[l][sh] = i0 + sh < n_r ? C0[(size_t)i0 * (L + 1) + e] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    const int jj = tid & 127, half = tid >> 7, j = j0 + jj;
-    if (j >= n_t) return;
-    // this thread's shells in groups of four (SB is a multiple of 8): four chains in flight
-    for (int s0 = 4 * half; s0 < SB; s0 += 8) {
-        float2 g[4];
-        g0_double_float_n<4>(sT + jj, 128, sC + (size_t)s0 * (L + 1), L + 1, L, g);
+    float s[SH], er[SH];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = i0 + s0 + k;
-            if (i < n_r) *reinterpret_cast<float2 *>(G0 + 2 * ((size_t)i * n_t + j)) = g[k];
-        }
+    for (int k = 0; k < SH; ++k) s[k] = er[k] = 0.0f;
+    auto term = [&](const float2 tt, int l) {
+#pragma unroll
+        for (int k = 0; k < SH; ++k) double_float_term(tt, sC[l][k], s[k], er[k]);
+    };
+    int l0 = 0;
+    for (; l0 + kM0Ahead <= L + 1; l0 += kM0Ahead) {
+        float2 nx[kM0Ahead];
+#pragma unroll
+        for (int k = 0; k < kM0Ahead; ++k) nx[k] = __ldg(T + (size_t)min(l0 + kM0Ahead + k, L) * n_t);
+#pragma unroll
+        for (int k = 0; k < kM0Ahead; ++k) term(t[k], l0 + k);
+#pragma unroll
+        for (int k = 0; k < kM0Ahead; ++k) t[k] = nx[k];
     }
+#pragma unroll
+    for (int k = 0; k < kM0Ahead - 1; ++k)
+        if (l0 + k <= L) term(t[k], l0 + k);
+    if (j >= n_t) return;
+#pragma unroll
+    for (int k = 0; k < SH; ++k)
+        if (i0 + k < n_r) *reinterpret_cast<float2 *>(G0 + 2 * ((size_t)(i0 + k) * n_t + j)) = double_float_sum(s[k], er[k]);
 }
 
 // ---------------------------------------------------------------------------- tables
@@ -816,8 +843,7 @@ cudaError_t launch_theta_tc_tables(mp_mesh *m)
         for (cudaError_t r : {cudaFuncSetAttribute(k_theta_tc<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit),
                               cudaFuncSetAttribute(k_theta_tc<3, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit),
                               cudaFuncSetAttribute(k_gsynth_tc<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit),
-                              cudaFuncSetAttribute(k_gsynth_tc<3, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit),
-                              cudaFuncSetAttribute(k_gsynth_m0, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit)})
+                              cudaFuncSetAttribute(k_gsynth_tc<3, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit)})
             if (r != cudaSuccess) return r;
         attr_set = true;
     }
@@ -854,8 +880,11 @@ cudaError_t launch_theta_tc(mp_mesh *m)
     // the m = 0 column first (CUDA cores), then the orders m >= 1
     cudaEvent_t ev;
     prof_begin(m, "split_theta_contract_m0", &ev);
-    cudaError_t e = launch_pdl(k_theta_m0, dim3((m->n_r + kM0Shells - 1) / kM0Shells, (m->L + kM0Deg) / kM0Deg),
-                               dim3(256), 0, m->stream, prm);
+    const int n_lb = (m->L + 80) / 80, na = ((m->L + n_lb) / n_lb + 15) / 16;  // at most 80 degrees a block
+    const dim3 grid0((m->n_r + kM0Shells - 1) / kM0Shells, n_lb);
+    auto go = [&](void (*kern)(const ThetaTcParams)) { return launch_pdl(kern, grid0, dim3(kM0Threads), 0, m->stream, prm); };
+    cudaError_t e = na == 1 ? go(k_theta_m0<1>) : na == 2 ? go(k_theta_m0<2>) : na == 3 ? go(k_theta_m0<3>)
+                  : na == 4 ? go(k_theta_m0<4>) : go(k_theta_m0<5>);
     prof_end(m, "split_theta_contract_m0", ev);
     if (e != cudaSuccess) return e;
     const int grid = std::min(pl.th_units, m->num_sms);
@@ -888,15 +917,14 @@ cudaError_t launch_gsynth_tc(mp_mesh *m)
     prm.ns_s = pl.gs_ns_s;
     prm.bterms = pl.n_products == 3 ? 2 : 3;
     prm.stage_bytes = (uint32_t)(prm.bterms * gsc::T_TERM_BYTES + pl.a_terms * 2 * pl.gs_NS * 64);
-    // the m = 0 column first (double-float on CUDA cores): 32 shells per block, or 8 when that
+    // the m = 0 column first (double-float on CUDA cores): eight shells a thread, or four when that
     // leaves fewer than two blocks per SM
-    const int n_jb = (m->n_t + 127) / 128;
-    const int SB = (long long)n_jb * ((m->n_r + 31) / 32) >= 2LL * m->num_sms ? 32 : 8;
-    const size_t smem0 = ((size_t)(m->L + 1) * 128 + (size_t)SB * (m->L + 1)) * sizeof(float2);
+    const int t0 = std::min(128, (m->n_t + 31) / 32 * 32), n_j0 = (m->n_t + t0 - 1) / t0;
+    const int sh = (long long)n_j0 * ((m->n_r + 7) / 8) >= 2LL * m->num_sms ? 8 : 4;
     cudaEvent_t ev;
     prof_begin(m, "split_theta_synth_m0", &ev);
-    cudaError_t e = launch_pdl(k_gsynth_m0, dim3(n_jb, (m->n_r + SB - 1) / SB), dim3(256), smem0, m->stream,
-                               (const float2 *)m->d_C0, (const float2 *)m->d_Itc0, m->d_G0, m->n_r, m->n_t, m->L, SB);
+    cudaError_t e = launch_pdl(sh == 8 ? k_gsynth_m0<8> : k_gsynth_m0<4>, dim3((m->n_r + sh - 1) / sh, n_j0), dim3(t0), 0,
+                               m->stream, (const float2 *)m->d_C0, (const float2 *)m->d_Itc0, m->d_G0, m->n_r, m->n_t, m->L);
     prof_end(m, "split_theta_synth_m0", ev);
     if (e != cudaSuccess) return e;
     const int grid = std::min(pl.gs_units, m->num_sms);

@@ -556,6 +556,25 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float x, float y)
 __device__ __forceinline__ float bf16lo_to_f32(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi_to_f32(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
+// One term of a double-float sum: (s, e) += t c, for t and c as (hi, lo) pairs.
+__device__ __forceinline__ void double_float_term(const float2 t, const float2 c, float &s, float &e)
+{
+    const float p = __fmul_rn(t.x, c.x);
+    const float pe = fmaf(t.x, c.x, -p);            // exact error of the leading product
+    const float cross = fmaf(t.x, c.y, __fmul_rn(t.y, c.x));
+    const float s2 = __fadd_rn(s, p);               // TwoSum of the running sum and p
+    const float bv = __fsub_rn(s2, s);
+    const float se = __fadd_rn(__fsub_rn(s, __fsub_rn(s2, bv)), __fsub_rn(p, bv));
+    s = s2;
+    e = __fadd_rn(e, __fadd_rn(se, __fadd_rn(pe, cross)));
+}
+
+__device__ __forceinline__ float2 double_float_sum(float s, float e)
+{
+    const float hi = __fadd_rn(s, e);
+    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+}
+
 // The m = 0 column is the bulk of Phi and its Legendre sum can cancel: it is formed in
 // double-float arithmetic on the float32 pipe from (hi, lo) pairs of the table T[l] and
 // the coefficients c[l] -- products split exactly by fmaf, the running sum kept as a
@@ -563,51 +582,8 @@ __device__ __forceinline__ float bf16hi_to_f32(uint32_t w) { return __uint_as_fl
 __device__ __forceinline__ float2 g0_double_float(const float2 *T, int t_stride, const float2 *c, int L)
 {
     float s = 0.0f, e = 0.0f;
-    for (int l = 0; l <= L; ++l) {
-        const float2 t = T[(size_t)l * t_stride], k = c[l];
-        const float p = __fmul_rn(t.x, k.x);
-        const float pe = fmaf(t.x, k.x, -p);            // exact error of the leading product
-        const float cross = fmaf(t.x, k.y, __fmul_rn(t.y, k.x));
-        const float s2 = __fadd_rn(s, p);                 // TwoSum of the running sum and p
-        const float bv = __fsub_rn(s2, s);
-        const float se = __fadd_rn(__fsub_rn(s, __fsub_rn(s2, bv)), __fsub_rn(p, bv));
-        s = s2;
-        e = __fadd_rn(e, __fadd_rn(se, __fadd_rn(pe, cross)));
-    }
-    const float hi = __fadd_rn(s, e);
-    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
-}
-
-// The same sum for NS coefficient rows c + k c_stride (k < NS) sharing the table column T:
-// NS independent accumulation chains in flight (a single chain is bound by the latency of
-// its dependent float32 operations).
-template <int NS>
-__device__ __forceinline__ void g0_double_float_n(const float2 *T, int t_stride, const float2 *c, int c_stride, int L,
-                                                  float2 (&out)[NS])
-{
-    float s[NS], e[NS];
-#pragma unroll
-    for (int k = 0; k < NS; ++k) s[k] = e[k] = 0.0f;
-    for (int l = 0; l <= L; ++l) {
-        const float2 t = T[(size_t)l * t_stride];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) {
-            const float2 kk = c[(size_t)k * c_stride + l];
-            const float p = __fmul_rn(t.x, kk.x);
-            const float pe = fmaf(t.x, kk.x, -p);
-            const float cross = fmaf(t.x, kk.y, __fmul_rn(t.y, kk.x));
-            const float s2 = __fadd_rn(s[k], p);
-            const float bv = __fsub_rn(s2, s[k]);
-            const float se = __fadd_rn(__fsub_rn(s[k], __fsub_rn(s2, bv)), __fsub_rn(p, bv));
-            s[k] = s2;
-            e[k] = __fadd_rn(e[k], __fadd_rn(se, __fadd_rn(pe, cross)));
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        const float hi = __fadd_rn(s[k], e[k]);
-        out[k] = make_float2(hi, __fsub_rn(e[k], __fsub_rn(hi, s[k])));
-    }
+    for (int l = 0; l <= L; ++l) double_float_term(T[(size_t)l * t_stride], c[l], s, e);
+    return double_float_sum(s, e);
 }
 
 }  // namespace mp
