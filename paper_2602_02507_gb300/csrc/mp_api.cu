@@ -504,8 +504,8 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
     ALLOC(m->d_Iphc, (size_t)m->P * n_phi);
     ALLOC(m->d_WR, (size_t)(l_max + 1) * n_r);
     ALLOC(m->d_WI, (size_t)(l_max + 1) * n_r);
-    ALLOC(m->d_GR, (size_t)(l_max + 1) * n_r);
-    ALLOC(m->d_GI, (size_t)(l_max + 1) * n_r);
+    ALLOC(m->d_GR, (size_t)2 * (l_max + 1) * n_r);
+    ALLOC(m->d_GI, (size_t)2 * (l_max + 1) * n_r);
     ALLOC(m->d_V, n_r);
     ALLOC(m->d_A, (size_t)n_r * m->KL);
     ALLOC(m->d_MR, (size_t)(n_r + 1) * m->KL);

@@ -125,7 +125,7 @@ struct mp_mesh {
     double *d_Iph = nullptr;   // [P][n_p]  int cos|sin(m phi) over azimuthal cells
     double *d_Iphc = nullptr;  // [P][n_p]  Iph / dphi (cell mean)
     double *d_WR = nullptr, *d_WI = nullptr;  // [L+1][n_r]
-    double *d_GR = nullptr, *d_GI = nullptr;  // [L+1][n_r]  -(R^R, R^I) / (2 (2l+1))
+    double *d_GR = nullptr, *d_GI = nullptr;  // [2][L+1][n_r]  -(R^R, R^I) / (2 (2l+1)) for m = 0, twice that for m > 0
     double *d_V = nullptr;     // [n_r]
 
     // moments (both paths)

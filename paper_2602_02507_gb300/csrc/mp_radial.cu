@@ -99,6 +99,8 @@ __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const
     const int i0 = min(n_r, (int)threadIdx.x * chunk), i1 = min(n_r, i0 + chunk);
     const double *wr = WR + (size_t)l * n_r;
     const double *wi = WI + (size_t)l * n_r;
+    const double *gr = GR + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
+    const double *gi = GI + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
     double sR = 0.0, sI = 0.0;
     for (int i = i0; i < i1; ++i) {
         const double a = A[(size_t)i * KL + q];
@@ -128,8 +130,7 @@ __global__ void __launch_bounds__(NT) k_scan(const double *__restrict__ A, const
         MI[(size_t)i * KL + q] = mi;
         const double mr_lo = MR[(size_t)i * KL + q];
         const double mr_hi = fma(wr[i], a, mr_lo);
-        double c = fma(GI[(size_t)l * n_r + i], mr_lo + mr_hi, GR[(size_t)l * n_r + i] * (mi + mi_hi));
-        if (m > 0) c += c;
+        const double c = fma(gi[i], mr_lo + mr_hi, gr[i] * (mi + mi_hi));
         if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = c;
         const float c32 = f64_to_f32_alu(c);
         if (C32) C32[(size_t)i * KL + q] = c32;
@@ -161,8 +162,8 @@ __global__ void __launch_bounds__(NT) k_scan_reg(const double *__restrict__ A, c
     const int i0 = (int)threadIdx.x * CH;
     const double *wr = WR + (size_t)l * n_r;
     const double *wi = WI + (size_t)l * n_r;
-    const double *gr = GR + (size_t)l * n_r;
-    const double *gi = GI + (size_t)l * n_r;
+    const double *gr = GR + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
+    const double *gi = GI + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
     double a[CH], w1[CH], w2[CH], g1[CH], g2[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
@@ -199,8 +200,7 @@ __global__ void __launch_bounds__(NT) k_scan_reg(const double *__restrict__ A, c
         if (i < n_r) {
             MR[(size_t)i * KL + q] = er[k];
             MI[(size_t)i * KL + q] = ei[k];
-            double c = fma(g2[k], er[k] + er[k + 1], g1[k] * (ei[k] + ei[k + 1]));
-            if (m > 0) c += c;
+            const double c = fma(g2[k], er[k] + er[k + 1], g1[k] * (ei[k] + ei[k + 1]));
             if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = c;
             const float c32 = f64_to_f32_alu(c);
             if (C32) C32[(size_t)i * KL + q] = c32;
@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
     const int i0 = c * CH;
     const double *wr = WR + (size_t)l * n_r;
     const double *wi = WI + (size_t)l * n_r;
-    const double *gr = GR + (size_t)l * n_r;
-    const double *gi = GI + (size_t)l * n_r;
+    const double *gr = GR + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
+    const double *gi = GI + (size_t)(m > 0 ? Lp1 + l : l) * n_r;
     // registers hold the column's values and its inward edge moments; the small weight
     // tables are read again where needed (cache hits), which keeps 512 threads resident
     double a[CH];
@@ -280,9 +280,32 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
     if (lane >= 28) wt[0][w][sub] = inf;
     if (lane < 4) wt[1][w][sub] = inb;
     __syncthreads();
+    // The sums of the warps before (and after) each warp, in that order: by one warp for all, since
+    // by every warp for itself they are 15 of the float64 instructions that bound a launch of one
+    // wave (1024 shells, 1089 columns: 38 -> 33 us).  With
+    // 16 shells a thread the launch has several waves, other blocks fill the pipe meanwhile, and
+    // the serial part of one warp costs more than it saves (2048 shells, 4225 columns: 214 us with
+    // it, 206 without).
     double of = 0.0, ob = 0.0;
-    for (int w2_ = 0; w2_ < w; ++w2_) of += wt[0][w2_][sub];
-    for (int w2_ = NW - 1; w2_ > w; --w2_) ob += wt[1][w2_][sub];
+    if constexpr (CH < 16) {
+        if (threadIdx.x < 8) {
+            const int dir = threadIdx.x >> 2;
+            double acc = 0.0;
+#pragma unroll 1
+            for (int k = 0; k < NW; ++k) {
+                double *at = &wt[dir][dir ? NW - 1 - k : k][sub];
+                const double v = *at;
+                *at = acc;
+                acc += v;
+            }
+        }
+        __syncthreads();
+        of = wt[0][w][sub];
+        ob = wt[1][w][sub];
+    } else {
+        for (int w2_ = 0; w2_ < w; ++w2_) of += wt[0][w2_][sub];
+        for (int w2_ = NW - 1; w2_ > w; --w2_) ob += wt[1][w2_][sub];
+    }
     if (!valid) return;
     if (off) {  // the sums of the slabs below (regular) and above (irregular) this one
         of += off[q];
@@ -303,8 +326,7 @@ __global__ void __launch_bounds__(4 * NT, 2) k_scan_q4(const double *__restrict_
             const double er1 = fma(__ldg(wr + i), a[k], er);
             MR[(size_t)i * KL + q] = er;
             MI[(size_t)i * KL + q] = ei[k];
-            double cv = fma(__ldg(gi + i), er + er1, __ldg(gr + i) * (ei[k] + ei[k + 1]));
-            if (m > 0) cv += cv;
+            const double cv = fma(__ldg(gi + i), er + er1, __ldg(gr + i) * (ei[k] + ei[k + 1]));
             if (C) C[ldC ? (size_t)q * ldC + i : (size_t)i * KL + q] = cv;
             const float c32 = f64_to_f32_alu(cv);
             if (C32) C32[(size_t)i * KL + q] = c32;

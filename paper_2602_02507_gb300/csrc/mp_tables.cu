@@ -190,6 +190,10 @@ __global__ void k_radial_tables(int L, int n_r, const double *__restrict__ r, do
         GI[(size_t)l * n_r + i] = hp * (wi / vol);
     else
         GI[(size_t)l * n_r + i] = 2.0 * hp * (6.0 * r1 * r1 / (5.0 * (l + 3.0))) / wr;
+    // the orders m > 0 carry Delta_m = 2 (Phi sums m >= 0 only): exact, and no multiplication a coefficient
+    const size_t second = (size_t)(L + 1) * n_r;
+    GR[second + (size_t)l * n_r + i] = 2.0 * GR[(size_t)l * n_r + i];
+    GI[second + (size_t)l * n_r + i] = 2.0 * GI[(size_t)l * n_r + i];
     if (l == 0) V[i] = vol;
 }
 
