@@ -66,7 +66,7 @@ SPLIT_PRECISION = "bf16x3"
 # those two counters alone (one pass, as on a 128-shell cut first): 8.60 GB of density read
 # and 0.49 GB of F written back (F, 545 MB, outgrows L2 at this size; on the cut it stays).
 NCU_TRAFFIC = {
-    ("large", "split_phi_project_tc"): (8.60e9 + 489.97e6, "mp_split.cu", "db667758754e9e99133af3c6f11f0db47869fecb"),
+    ("large", "split_phi_project_tc"): (8.603e9 + 487.8e6, "mp_split.cu", "b39e7ee298fb1997bd290f7c46aadda95b9b1c26"),
 }
 KERNEL_HEADERS = ("ptx.cuh", "mp_internal.h", "mp_errors.h")
 
@@ -593,8 +593,8 @@ def beside_solve(stream, hbm_peak, rates, steps):
     gravity = {"kernel": "gravity_sources", "workload": WORKLOADS["presn"], "launches": kg, "avg_launch_us": g_us,
                "algorithmic_bytes_per_cell": 72, "hbm_gbs": 72 * cells / g_us / 1e3,
                "hbm_frac": 72 * cells / g_us / 1e3 / hbm_peak,
-               "fp64_instr_per_cell": 12, "fp64_instr_per_s": 12 * cells / (g_us * 1e-6),
-               "fp64_frac": 12 * cells / (g_us * 1e-6) / fp64_instr_peak, "bound": "fp64",
+               "fp64_instr_per_cell": 6, "fp64_instr_per_s": 6 * cells / (g_us * 1e-6),
+               "fp64_frac": 6 * cells / (g_us * 1e-6) / fp64_instr_peak, "bound": "issue",
                "note": "S [3] and E from Phi, rho, v [3]: 9 float64 reads + 4 writes per cell"}
     mesh.close()
     del gvel, gS, gE, rho

@@ -33,11 +33,12 @@
 // right, so a K step of 16 takes seven MMAs for its 28 products and reads A seven times
 // instead of 28 (with one MMA per pair the shared-memory reads of A would bound it).
 //
-// What bounds them: not the tensor core (about 40 % of the time at 1024 x 256 x 512 cells,
-// l_max = 32) nor HBM, but the integer instructions that split and rejoin the operands (half the
-// rate of float32's) and the hand-offs between the warps that issue them.  Measured there against
-// float64 on CUDA cores: (a1) 29.5 ms -> 649 us, (a2) 688 -> 90 us, (d1) 2143 -> 66 us, (d2)
-// 13.9 ms -> 423 us; at 512 x 128 x 256, l_max = 16: 1918 -> 102, 76 -> 21, 200 -> 17, 891 -> 69 us.
+// What bounds them: not the tensor core (35 % of the time in the long contraction, 49 % in the
+// long expansion at 1024 x 256 x 512 cells, l_max = 32) nor HBM (24 and 34 %), but the integer
+// instructions that split and rejoin the operands (half the rate of float32's: their pipe is 50 and
+// 58 % busy) and the hand-offs between the warps that issue them.  Measured there against float64
+// on CUDA cores: (a1) 29.5 ms -> 649 us, (a2) 688 -> 90 us, (d1) 2143 -> 65 us, (d2) 13.9 ms -> 425
+// us; at 512 x 128 x 256, l_max = 16: 1918 -> 89, 76 -> 20, 200 -> 17, 891 -> 69 us.
 #include <algorithm>
 
 #include <cuda_fp16.h>
