@@ -1,8 +1,8 @@
 // mp_fp64.cu -- the float64 path: its contractions on CUDA cores in float64 (GB300's float64
 // rate bounds them), used beyond the range of the tensor-core form (l_max > 71), for a few
 // azimuthal cells, and by mp_moments_noalloc, whose scratch is fixed; and the dispatch to the
-// tensor-core form (mp_fp64_tc.cu), which is 13 to 34 times faster per solve (1024 x 256 x 512
-// cells at l_max = 32: 46.3 -> 1.34 ms; 512 x 128 x 256 at 16: 3.10 -> 0.24 ms).
+// tensor-core form (mp_fp64_tc.cu), which is 13 to 37 times faster per solve (1024 x 256 x 512
+// cells at l_max = 32: 46.3 -> 1.24 ms; 512 x 128 x 256 at 16: 3.10 -> 0.20 ms).
 // Steps of GenASiS II Sec. 2.2:
 //   (a1) F[row][p]  = sum_k Iph[p][k] rho[row][k]                 (phi part of Eq. AngularMomentsDiscrete)
 //   (a2) A[i][q]    = 4 pi G sum_j Ith[t][j] F[i n_t + j][p]      (theta part)
