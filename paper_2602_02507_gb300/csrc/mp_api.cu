@@ -446,6 +446,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
     const double rmin = r_edges[0] > 0.0 ? r_edges[0] : r_edges[1];
     const double rmax = r_edges[n_r];
     const double r_ref = r_ref_given > 0.0 ? r_ref_given : std::sqrt(rmin * rmax);
+    bool far_moments;  // radial weights whose squares leave the float64 range
     {
         const double lx_hi = std::log10(rmax / r_ref), lx_lo = std::log10(rmin / r_ref), lr = std::log10(r_ref);
         const double e_reg = 3.0 * lr + (l_max + 3.0) * lx_hi;
@@ -453,6 +454,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         if (e_reg > 290.0 || e_irr > 290.0 || 3.0 * std::log10(rmax) > 300.0)
             return set_error(MP_ERR_RANGE, "r^l or r^-(l+1) over [%g, %g] at l_max = %d exceeds float64", rmin, rmax,
                              l_max);
+        far_moments = std::max(e_reg, e_irr) > 150.0;
     }
 
     mp_mesh *m = new (std::nothrow) mp_mesh();
@@ -493,7 +495,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
 
     const size_t nedges = (size_t)(n_r + 1) + (n_theta + 1) + (n_phi + 1);
     mp_status st;
-    if (m->eff_prec == MP_PREC_FP64) plan_fp64_tc(m);
+    if (m->eff_prec == MP_PREC_FP64) plan_fp64_tc(m, far_moments);
 #define ALLOC(ptr, count)                             \
     st = dalloc(m, &(ptr), (size_t)(count));          \
     if (st != MP_OK) return fail(st);

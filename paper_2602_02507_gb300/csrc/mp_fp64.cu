@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(128) k64_synth_phi_few(const double *__restric
 
 cudaError_t launch_fp64_project(mp_mesh *m, const double *rho)
 {
-    if (m->fp.phi_on) return launch_fp64_tc_project(m, rho);
-    if (m->fp.on) {
+    if (m->fp.mom_on && m->fp.phi_on) return launch_fp64_tc_project(m, rho);
+    if (m->fp.mom_on) {
         cudaEvent_t ev;
         prof_begin(m, "fp64_phi_project", &ev);
         const int threads = std::min(128, round_up(m->n_t, 32));
@@ -183,7 +183,7 @@ cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double
 
 cudaError_t launch_fp64_theta(mp_mesh *m)
 {
-    if (m->fp.on) return launch_fp64_tc_theta(m);
+    if (m->fp.mom_on) return launch_fp64_tc_theta(m);
     cudaEvent_t ev;
     prof_begin(m, "fp64_theta_contract", &ev);
     k64_theta<<<m->n_r, 256, 0, m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_t, m->L, m->KL, m->P,

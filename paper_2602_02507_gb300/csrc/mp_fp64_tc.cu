@@ -1361,7 +1361,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-bool plan_fp64_tc(mp_mesh *m)
+bool plan_fp64_tc(mp_mesh *m, bool far_moments)
 {
     Fp64Plan &f = m->fp;
     f = Fp64Plan();
@@ -1382,6 +1382,12 @@ bool plan_fp64_tc(mp_mesh *m)
     // below 16 azimuthal cells (axisymmetric meshes have one) a 16-wide K step is mostly padding
     // and the sums are short: CUDA cores
     f.phi_on = m->n_p >= 16 && plan_contract(m->n_p, f.pass_cols, f.m0, f.ph_c) && plan_expand(m->P - 1, f.ph_x);
+    // Moments whose radial weights reach 1e150 (l_max = 48 over five decades of r): their squares
+    // leave the float64 range, so neither they nor the differences of two solutions have a norm,
+    // and equality is the one way to compare them.  They stay sums in the order of the CUDA-core
+    // kernels, those of mp_moments_noalloc, to the last bit.  It costs their speed: 260 x 130 x 150
+    // cells, l_max = 64: 346 -> 1860 us a solve (3594 with the synthesis on CUDA cores as well).
+    f.mom_on = !far_moments;
     f.on = 1;
     return true;
 }
@@ -1404,7 +1410,7 @@ size_t fp64_tc_arena(mp_mesh *m)
     const int n_blk = (m->n_t + kNtX - 1) / kNtX;
     for (int s = 0; s < n_sets; ++s) {
         oc[s] = c;
-        c += (unsigned long long)f.th_c.n_steps * kDig * (half_cols(set_cols(s, L), 0) + half_cols(set_cols(s, L), 1)) * 32;
+        if (f.mom_on) c += (unsigned long long)f.th_c.n_steps * kDig * (half_cols(set_cols(s, L), 0) + half_cols(set_cols(s, L), 1)) * 32;
     }
     for (int mm = 0; mm <= L; ++mm) {
         ox[mm] = x;
@@ -1414,7 +1420,7 @@ size_t fp64_tc_arena(mp_mesh *m)
     for (int s = 0; s < f.npass; ++s) op[s] = s * pstep;
     f.o_tab_c = take(c);
     f.o_tab_x = take(x);
-    f.o_tab_pc = take(f.phi_on ? f.npass * pstep : 0);
+    f.o_tab_pc = take(f.phi_on && f.mom_on ? f.npass * pstep : 0);
     f.o_tab_px = take(f.phi_on ? (size_t)((m->n_p + kNtX - 1) / kNtX) * std::max(1, (m->P - 1 + 15) / 16) * kRowsX * 32 : 0);
     f.o_off = take(f.h_off.size() * sizeof(unsigned long long));
     f.o_et_c = take((size_t)n_sets * kEtLd * 4);
@@ -1473,12 +1479,10 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
                     reinterpret_cast<int *>(f.arena + f.o_bound) + kind};
         k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t, n_sets);
     };
-    build(TAB_CONTRACT, f.o_tab_c, 0, f.o_et_c, kEtLd, std::min(L + 1, kNtMax), L + 1 + set_extra(L));
+    if (f.mom_on) build(TAB_CONTRACT, f.o_tab_c, 0, f.o_et_c, kEtLd, std::min(L + 1, kNtMax), L + 1 + set_extra(L));
     build(TAB_EXPAND_TH, f.o_tab_x, 1, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
-    if (f.phi_on) {
-        build(TAB_PROJECT, f.o_tab_pc, 2, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
-        build(TAB_EXPAND_PH, f.o_tab_px, 3, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
-    }
+    if (f.phi_on && f.mom_on) build(TAB_PROJECT, f.o_tab_pc, 2, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
+    if (f.phi_on) build(TAB_EXPAND_PH, f.o_tab_px, 3, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
     // 227 KB of dynamic shared memory for the kernels of this file (per device)
     for (int theta = 0; theta < 2; ++theta) {
         for (int vec = 0; vec < 2; ++vec)

@@ -70,6 +70,7 @@ struct Fp64Expand {
 struct Fp64Plan {
     int on = 0;      // theta stages (and the layouts F, G [n_r][P][ldJ], C [K_L][ldI])
     int phi_on = 0;  // phi stages too
+    int mom_on = 0;  // the projection and the theta contraction among them (else F [R][P])
     int ldJ = 0, ldI = 0, npass = 1, pass_cols = 0, m0 = 0, off_ld = 0;
     Fp64Contract ph_c, th_c;
     Fp64Expand ph_x, th_x;
@@ -264,7 +265,8 @@ cudaError_t launch_fp64_synth(mp_mesh *m, double *phi);
 cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double *F, double *A);
 
 // the same steps as exact integer slices on the tensor cores (F, G [n_r][P][ldJ], C [K_L][ldI])
-bool plan_fp64_tc(mp_mesh *m);             // false: sizes out of its range (l_max > 71)
+// (false: sizes out of its range, l_max > 71; far_moments: the moments stay on CUDA cores)
+bool plan_fp64_tc(mp_mesh *m, bool far_moments);
 size_t fp64_tc_arena(mp_mesh *m);          // lays the tables out; bytes of the arena
 cudaError_t launch_fp64_tc_tables(mp_mesh *m);
 cudaError_t fp64_tc_bounds(mp_mesh *m);    // reads what the finished tables say about the accumulators
