@@ -519,8 +519,6 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         if (m->fp.on) {
             ALLOC(m->d_F64, (size_t)n_r * m->P * m->fp.ldJ);
             ALLOC(m->d_G64, (size_t)n_r * m->P * m->fp.ldJ);
-            // padding cells of the polar rows stay zero: the theta contraction reads them
-            cudaMemsetAsync(m->d_F64, 0, (size_t)n_r * m->P * m->fp.ldJ * sizeof(double), m->stream);
             m->fp.arena_bytes = fp64_tc_arena(m);
             ALLOC(m->fp.arena, m->fp.arena_bytes);
             st = make_map_f64_G(&m->tm_G64, m->d_G64, n_r, m->P, n_theta, m->fp.ldJ);

@@ -1,8 +1,10 @@
 // mp_fp64.cu -- the float64 path: its contractions on CUDA cores in float64 (GB300's float64
-// rate bounds them), used beyond the range of the tensor-core form (l_max > 71), for a few
-// azimuthal cells, and by mp_moments_noalloc, whose scratch is fixed; and the dispatch to the
-// tensor-core form (mp_fp64_tc.cu), which is 13 to 37 times faster per solve (1024 x 256 x 512
-// cells at l_max = 32: 46.3 -> 1.24 ms; 512 x 128 x 256 at 16: 3.10 -> 0.20 ms).
+// rate bounds them) and the dispatch to their tensor-core form (mp_fp64_tc.cu).  The theta
+// contraction always runs here; the other steps do beyond the range of the tensor-core form (l_max >
+// 71), for a few azimuthal cells, for moments whose squares overflow, and in mp_moments_noalloc,
+// whose scratch is fixed.  A solve with the tensor-core steps against one without: 46.3 -> 1.63 ms at
+// 1024 x 256 x 512 cells, l_max = 32; 3.10 -> 0.22 ms at 512 x 128 x 256, 16; 1.53 -> 0.15 ms at 353 x
+// 96 x 192, 20; 340 -> 117 us at 471 x 128 x 1, 20.
 // Steps of GenASiS II Sec. 2.2:
 //   (a1) F[row][p]  = sum_k Iph[p][k] rho[row][k]                 (phi part of Eq. AngularMomentsDiscrete)
 //   (a2) A[i][q]    = 4 pi G sum_j Ith[t][j] F[i n_t + j][p]      (theta part)
@@ -59,6 +61,91 @@ __global__ void __launch_bounds__(256) k64_theta(const double *__restrict__ F, c
         double acc = 0.0;
         for (int j = 0; j < n_t; ++j) acc = fma(w[j], f[(size_t)j * P], acc);
         A[(size_t)i * KL + q] = scale * acc;
+    }
+}
+
+// (a2) with F as [n_r][P][ldJ]: in float64 whatever the other steps do.  The table (sin^m theta
+// near the poles) and a row of F may be large at different cells, and a product of fixed-point
+// operands, scaled by the maxima of both, then loses what a float64 sum keeps: a clump near the pole
+// left moments of order 16 with errors of 1e-5 of their own terms.  A block takes 32 rows (shells,
+// or cos and sin of 16 shells) of one order and 32 of its degrees; chunks of 32 polar cells of both
+// operands pass through shared memory, a lane sums its row for up to four degrees, in the
+// order of k64_theta.  The float64 pipe bounds it, so lanes are rows (always full) and not degrees,
+// and the degrees are dealt to the warps one by one (to the SM's four quarters evenly).
+// 512 x 128 x 256 cells, l_max = 16: 76 us as k64_theta, 53 so; 1024 x 256 x 512, 32: 688 -> 479 (0.6 T
+// products a second, all the pipe does); fixed-point slices on the tensor cores took 20 and 92.
+constexpr int kThRows = 32, kThDeg = 32, kThCells = 32, kThWarps = 8, kThWarpDeg = kThDeg / kThWarps;
+
+// One chunk: ND degrees (rows kThWarps apart of sT) of the lane's row.
+template <int ND>
+__device__ __forceinline__ void theta_chunk(const double (*sF)[kThRows + 1], const double (*sT)[kThCells], int lane,
+                                            int cells, double (&acc)[kThWarpDeg])
+{
+    if (cells == kThCells) {
+#pragma unroll 4
+        for (int j = 0; j < kThCells; j += 2) {
+            const double f0 = sF[j][lane], f1 = sF[j + 1][lane];
+#pragma unroll
+            for (int c = 0; c < ND; ++c) {
+                const double2 w = *reinterpret_cast<const double2 *>(&sT[kThWarps * c][j]);
+                acc[c] = fma(w.y, f1, fma(w.x, f0, acc[c]));
+            }
+        }
+    } else {
+        for (int j = 0; j < cells; ++j)
+#pragma unroll
+            for (int c = 0; c < ND; ++c) acc[c] = fma(sT[kThWarps * c][j], sF[j][lane], acc[c]);
+    }
+}
+
+__global__ void __launch_bounds__(32 * kThWarps) k64_theta_rows(const double *__restrict__ F, const double *__restrict__ Ith,
+                                                      double *__restrict__ A, int n_r, int n_t, int L, int KL, int P,
+                                                      int ldJ, double scale)
+{
+    __shared__ double sF[kThCells][kThRows + 1];
+    __shared__ __align__(16) double sT[kThDeg][kThCells];
+    const int n_dg = (L + kThDeg) / kThDeg, m = blockIdx.y / n_dg, d0 = (blockIdx.y - m * n_dg) * kThDeg;
+    const int N = min(kThDeg, L + 1 - m - d0);  // degrees m + d0 ... of this block
+    const int i0 = blockIdx.x * (m ? kThRows / 2 : kThRows);
+    if (N <= 0 || i0 >= n_r) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // loads: cell `lane` of rows (and degrees) warp, warp + kThWarps, ...
+    double f[kThWarpDeg], t[kThWarpDeg];
+    auto load = [&](int j0) {
+        const int j = j0 + lane;
+#pragma unroll
+        for (int k = 0; k < kThWarpDeg; ++k) {
+            const int r = warp + kThWarps * k, i = i0 + (m ? r >> 1 : r), p = m ? 2 * m - 1 + (r & 1) : 0;
+            f[k] = j < n_t && i < n_r ? __ldg(F + ((size_t)i * P + p) * ldJ + j) : 0.0;
+            t[k] = j < n_t && r < N ? __ldg(Ith + (size_t)tri(m + d0 + r, m) * n_t + j) : 0.0;
+        }
+    };
+    double acc[kThWarpDeg] = {};
+    const int nd = (N - warp + kThWarps - 1) / kThWarps;  // degrees of this warp
+    load(0);
+    for (int j0 = 0; j0 < n_t; j0 += kThCells) {
+        __syncthreads();  // the chunk before has been read
+#pragma unroll
+        for (int k = 0; k < kThWarpDeg; ++k) {
+            sF[lane][warp + kThWarps * k] = f[k];
+            sT[warp + kThWarps * k][lane] = t[k];
+        }
+        __syncthreads();
+        if (j0 + kThCells < n_t) load(j0 + kThCells);
+        const int cells = min(kThCells, n_t - j0);
+        switch (nd) {
+        case 4: theta_chunk<4>(sF, sT + warp, lane, cells, acc); break;
+        case 3: theta_chunk<3>(sF, sT + warp, lane, cells, acc); break;
+        case 2: theta_chunk<2>(sF, sT + warp, lane, cells, acc); break;
+        case 1: theta_chunk<1>(sF, sT + warp, lane, cells, acc); break;
+        }
+    }
+    const int i = i0 + (m ? lane >> 1 : lane), p = m ? 2 * m - 1 + (lane & 1) : 0;
+    if (i >= n_r) return;
+#pragma unroll
+    for (int c = 0; c < kThWarpDeg; ++c) {
+        const int d = warp + kThWarps * c, l = m + d0 + d;
+        if (d < N) A[(size_t)i * KL + l * l + p] = scale * acc[c];
     }
 }
 
@@ -183,11 +270,15 @@ cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double
 
 cudaError_t launch_fp64_theta(mp_mesh *m)
 {
-    if (m->fp.mom_on) return launch_fp64_tc_theta(m);
     cudaEvent_t ev;
     prof_begin(m, "fp64_theta_contract", &ev);
-    k64_theta<<<m->n_r, 256, 0, m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_t, m->L, m->KL, m->P,
-                                            kFourPi * m->G);
+    if (m->fp.mom_on)
+        k64_theta_rows<<<dim3((m->n_r + kThRows / 2 - 1) / (kThRows / 2), (m->L + 1) * ((m->L + kThDeg) / kThDeg)), 32 * kThWarps, 0,
+                         m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_r, m->n_t, m->L, m->KL, m->P, m->fp.ldJ,
+                                      kFourPi * m->G);
+    else
+        k64_theta<<<m->n_r, 256, 0, m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_t, m->L, m->KL, m->P,
+                                                kFourPi * m->G);
     prof_end(m, "fp64_theta_contract", ev);
     return cudaGetLastError();
 }

@@ -1,8 +1,8 @@
-// mp_fp64_tc.cu -- the float64 path's four contractions on the tensor cores, to float64
-// accuracy, by exact integer slices.
+// mp_fp64_tc.cu -- three of the float64 path's four contractions on the tensor cores, by exact
+// integer slices.
 //
-// GB300 does about 0.5 T float64 operations a second, 1/1700 of its 16-bit tensor rate, so
-// the contractions of GenASiS II Sec. 2.2 (both factors of Eq. (AngularMomentsDiscrete) and
+// GB300 does about 0.6 T float64 operations a second, 1/1700 of its 16-bit tensor rate, so
+// contractions of GenASiS II Sec. 2.2 (the azimuthal factor of Eq. (AngularMomentsDiscrete) and both
 // of Eq. (Solution)) run here as sums of exact 16-bit products: every float64 operand row
 // is scaled by a power of two of its own to a 55-bit fixed-point magnitude, cut into seven
 // 8-bit balanced digits (integers of magnitude <= 128, exact in float16), and the products
@@ -14,15 +14,23 @@
 // the tensor core's truncating addition never truncates.  Pairs with a + b >= 7 are left
 // out: they weigh at most 2^-56 of (row maximum x column maximum) each.  The seven
 // accumulators are put together as a 64-bit integer and leave as float64 by integer
-// instructions; no step uses the float64 pipe.  A value 2^k below its row's maximum keeps
-// 55 - k bits; float64 sums of such rows carry a rounding error of that size as well.
+// instructions (ldexp, on the float64 pipe, for results outside the normal range).
 //
-// Two kernels serve the four steps.  A is always the data (split on the fly), B a table
-// (split once per mesh), D = A B^T:
+// Accuracy.  The operands are fixed-point: a value 2^k below its row's (or table column's) maximum
+// keeps 55 - k bits.  A result of K terms is off by at most about K 2^-54 x (row maximum) x (column
+// maximum), whether or not the two maxima meet at one index, where a float64 sum is off by a
+// multiple of 2^-53 of the sum of its terms' magnitudes.  The steps below can afford that: the
+// azimuthal tables are of one size along a row of cells and themselves off by the rounding of
+// m phi, 2^-53 m phi of their maximum; and the synthesis delivers Phi alone, whose sum over the
+// orders is of the size of the row maxima (errors stay at 2^-53 of the largest |Phi| of the
+// shell; G of an order m near the poles, a small part of it there, is less accurate by itself).
+// The theta part of the moments cannot (sin^m theta against a clump near the pole): it is summed
+// in float64, k64_theta_rows in mp_fp64.cu.
+//
+// Two kernels.  A is always the data (split on the fly), B a table (split once per mesh),
+// D = A B^T:
 //   k64_contract_tc  long K, few columns (K streamed):
 //       (a1) F[i][p][j] = sum_k rho[i][j][k] Iph[p][k]      rows (i, j), K = n_phi
-//       (a2) A[i][q]    = 4 pi G sum_j F[i][p][j] Ith[t][j]  rows (i, cos | sin) of one order m,
-//                                                            columns l = m .. L, K = n_theta
 //   k64_expand_tc    short K, many columns (A kept, columns streamed):
 //       (d1) G[i][p][j] = sum_l C[q][i] Ith[t][j] / dmu_j    rows (i, cos | sin) of one order m,
 //                                                            columns j, K = L + 1 - m
@@ -37,8 +45,8 @@
 // long expansion at 1024 x 256 x 512 cells, l_max = 32) nor HBM (24 and 34 %), but the integer
 // instructions that split and rejoin the operands (half the rate of float32's: their pipe is 50 and
 // 58 % busy) and the hand-offs between the warps that issue them.  Measured there against float64
-// on CUDA cores: (a1) 29.5 ms -> 649 us, (a2) 688 -> 90 us, (d1) 2143 -> 65 us, (d2) 13.9 ms -> 425
-// us; at 512 x 128 x 256, l_max = 16: 1918 -> 89, 76 -> 20, 200 -> 17, 891 -> 69 us.
+// on CUDA cores: (a1) 29.5 ms -> 653 us, (d1) 2143 -> 66 us, (d2) 13.9 ms -> 427 us; at 512 x 128 x
+// 256, l_max = 16: 1918 -> 87, 200 -> 16, 891 -> 69 us.
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -77,7 +85,7 @@ constexpr int kStepA2 = kDig * kDigA2;
 
 __host__ __device__ inline int ceil16(int x) { return (x + 15) & ~15; }
 
-// Contract: the columns of a set (a pass over the density, or the degrees of one order), 64 at
+// Contract: the columns of a set (a pass over the density), 64 at
 // most, in halves of up to 32, each padded to a multiple of 16 (accumulator blocks start on such
 // columns) and stacked by itself: 7 * 32 of the half's 256 columns of tensor memory.  A
 // projection of P = 2 L + 1 columns with L a multiple of 8 would pay a block of 16 for its one
@@ -285,7 +293,7 @@ __device__ __forceinline__ bool scaled_row(const uint32_t (&lo)[N], const uint32
 }
 
 // ---------------------------------------------------------------------------- tables
-enum { TAB_PROJECT = 0, TAB_CONTRACT = 1, TAB_EXPAND_TH = 2, TAB_EXPAND_PH = 3 };
+enum { TAB_PROJECT = 0, TAB_EXPAND_TH = 1, TAB_EXPAND_PH = 2 };
 
 struct TabParams {
     const double *Ith, *Iph, *Iphc, *dmu;
@@ -295,17 +303,6 @@ struct TabParams {
     int kind, n_t, n_p, L, P, pass_cols, m0, et_ld;
     int *bound;  // largest sum an accumulator can reach: expand, the sixth; contract, the third
 };
-
-// Sets of the theta contraction: order m = s, columns l = m .. m + 63, for s = 0 .. L; the
-// columns past 64 of the orders that have them as sets L + 1 + m.
-__host__ __device__ inline int set_order(int s, int L) { return s <= L ? s : s - L - 1; }
-__host__ __device__ inline int set_col0(int s, int L) { return s <= L ? 0 : kNtMax; }
-__host__ __device__ inline int set_cols(int s, int L)
-{
-    const int n = L + 1 - set_order(s, L) - set_col0(s, L);
-    return n < kNtMax ? n : kNtMax;
-}
-__host__ __device__ inline int set_extra(int L) { return L + 1 > kNtMax ? L + 1 - kNtMax : 0; }
 
 // First column of a projection pass; m0: the column m = 0 rides on pass 0 in a block of its own.
 __host__ __device__ inline int pass_col0(int s, int pass_cols, int m0) { return s * pass_cols + m0; }
@@ -320,16 +317,12 @@ __device__ __forceinline__ double tab_value(const TabParams &t, int set, int n, 
     switch (t.kind) {
     case TAB_PROJECT:  // n = -1: the column m = 0 in its own block
         return t.Iph[(size_t)(n < 0 ? 0 : pass_col0(set, t.pass_cols, t.m0) + n) * t.n_p + k];
-    case TAB_CONTRACT: {
-        const int m = set_order(set, t.L);
-        return t.Ith[(size_t)tri(m + set_col0(set, t.L) + n, m) * t.n_t + k];
-    }
     case TAB_EXPAND_TH: return t.Ith[(size_t)tri(set + k, set) * t.n_t + n] / t.dmu[n];
     default: return t.Iphc[(size_t)(k + 1) * t.n_p + n];  // m >= 1: the column m = 0 is 1 everywhere
     }
 }
 
-// One warp per table column n of one set: its exponent, then its digits.  Contract tables are
+// One warp per table column n of one set: its exponent, then its digits.  The contract table is
 // [K step]{per half [octet][7 Nt rows][8], row = digit Nt + n; for a column m = 0 of its own
 // then [digit of A][octet][16 rows][8]}; expand tables are blocks of 32
 // columns, [block][K step][octet][7 x 32][8].  Cells past K are never written (the tables
@@ -342,7 +335,6 @@ __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n
     int N, K;
     switch (t.kind) {
     case TAB_PROJECT: N = pass_ncols(set, t.pass_cols, t.m0, t.P), K = t.n_p; break;
-    case TAB_CONTRACT: N = set_cols(set, t.L), K = t.n_t; break;
     case TAB_EXPAND_TH: N = t.n_t, K = t.L + 1 - set; break;
     default: N = t.n_p, K = t.P - 1; break;
     }
@@ -354,7 +346,7 @@ __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n
     const int E = t.kind == TAB_EXPAND_PH ? 1023 : (int)(mx >> 20);
     if (lane == 0) t.et[(size_t)set * t.et_ld + (n < 0 ? kNtMax : n)] = E;
     if (E == 0) return;  // zeros
-    const bool stacked = t.kind == TAB_PROJECT || t.kind == TAB_CONTRACT;
+    const bool stacked = t.kind == TAB_PROJECT;
     const int hf = stacked && n >= kHalf, h0 = half_cols(N, 0), h1 = half_cols(N, 1);
     const int nd = !stacked ? kNtX : hf ? h1 : h0, rows = kDig * nd;
     const int main_rows = stacked ? kDig * (h0 + h1) : rows;
@@ -422,77 +414,53 @@ struct ContractParams {
     const int *et;
     int *err;
     long long R;
-    int n_r, n_t, n_p, L, KL, P, ldJ;
-    int K, n_steps, n_chunks, ds;  // ds: low bits of a chain's 62-bit sum dropped, so that n_chunks of them fit
+    int n_t, n_p, P, ldJ;
+    int n_steps, n_chunks, ds;  // ds: low bits of a chain's 62-bit sum dropped, so that n_chunks of them fit
                                    // (the template's DS, or where that is negative at run time)
-    int n_units, npass, pass_cols, m0, n_groups, n_groups0, et_ld;
+    int n_units, npass, pass_cols, m0;
     int ns_a, ns_b, nacc, slot_b, cols_max;
-    double scale;                  // (a2) 4 pi G
 };
 
 struct ContractUnit {
-    int set, order, col0;  // pass or theta set; its order (theta) and first column
+    int set, col0;         // pass and its first column
     int N, Nt[2], own0;    // columns, those of its halves padded; the column m = 0 in a block of its own
-    long long row0;        // (a1) first row; (a2) first shell
+    long long row0;
     __device__ __forceinline__ uint32_t step_bytes() const
     {
         return (uint32_t)(kDig * (Nt[0] + Nt[1]) + (own0 ? kRows0 : 0)) * 32;
     }
 };
 
-template <bool THETA>
 __device__ __forceinline__ ContractUnit contract_unit(const ContractParams &p, int u)
 {
     ContractUnit r;
-    if (!THETA) {
-        const int tile = u / p.npass;
-        r.set = u - tile * p.npass;
-        r.order = 0;
-        r.row0 = (long long)tile * 128;
-        r.col0 = pass_col0(r.set, p.pass_cols, p.m0);
-        r.N = pass_ncols(r.set, p.pass_cols, p.m0, p.P);
-        r.own0 = p.m0 && r.set == 0;
-    } else {
-        // order 0 (rows are 128 shells), then the orders with cos and sin rows of 64 shells
-        const int extra = set_extra(p.L), v0 = p.n_groups0 * (extra ? 2 : 1);
-        if (u < v0) {
-            r.set = u < p.n_groups0 ? 0 : p.L + 1;
-            r.row0 = (long long)(u < p.n_groups0 ? u : u - p.n_groups0) * 128;
-        } else {
-            const int v = (u - v0) / p.n_groups;
-            r.set = v < p.L ? 1 + v : p.L + 2 + (v - p.L);
-            r.row0 = (long long)(u - v0 - v * p.n_groups) * 64;
-        }
-        r.order = set_order(r.set, p.L);
-        r.col0 = r.order + set_col0(r.set, p.L);
-        r.N = set_cols(r.set, p.L);
-        r.own0 = 0;
-    }
+    const int tile = u / p.npass;
+    r.set = u - tile * p.npass;
+    r.row0 = (long long)tile * 128;
+    r.col0 = pass_col0(r.set, p.pass_cols, p.m0);
+    r.N = pass_ncols(r.set, p.pass_cols, p.m0, p.P);
+    r.own0 = p.m0 && r.set == 0;
     r.Nt[0] = half_cols(r.N, 0);
     r.Nt[1] = half_cols(r.N, 1);
     return r;
 }
 
-// Start of row `r` of a unit in the source (K contiguous values), or nullptr past the last row.
-template <bool THETA>
+// Start of row `r` of a unit in the source (n_phi contiguous values), or nullptr past the last row.
 __device__ __forceinline__ const double *contract_row(const ContractParams &p, const ContractUnit &u, int r)
 {
-    if (!THETA) {
-        const long long row = u.row0 + r;
-        return row < p.R ? p.src + row * p.n_p : nullptr;
-    }
-    const int i = (int)u.row0 + (u.order ? r >> 1 : r);
-    const int col = u.order ? 2 * u.order - 1 + (r & 1) : 0;
-    return i < p.n_r ? p.src + ((size_t)i * p.P + col) * p.ldJ : nullptr;
+    const long long row = u.row0 + r;
+    return row < p.R ? p.src + row * p.n_p : nullptr;
 }
 
 // Roles: warps 0-15 split A (each thread four neighbouring k of one row per K step, the whole
 // chunk of 128 k in registers: its row maxima come from a shuffle over the row's four threads,
 // and a step's registers take the next chunk's loads as soon as it is split, so 128 KB are in
 // flight a CTA) and drain the accumulators between their steps; warp 16 owns tensor memory;
-// warps 16-18 issue the MMAs, warp 19 copies the table.
-template <bool THETA, bool VEC, int DS, int NM>
-__global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractParams prm)
+// warps 16-18 issue the MMAs, warp 19 copies the table.  (The parameters stay in constant memory:
+// copied to registers, as the compiler does with up to 128 bytes of them, they cost 20 bytes of
+// spills and 89 -> 118 us at 512 x 128 x 256 cells, l_max = 16.)
+template <bool VEC, int DS, int NM>
+__global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_constant__ ContractParams prm)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -546,7 +514,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                 int issued = 0;
                 bool ok = true;
                 for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                    const ContractUnit un = contract_unit<THETA>(prm, u);
+                    const ContractUnit un = contract_unit(prm, u);
                     const uint8_t *src = prm.tab + prm.off[un.set];
                     const uint32_t bytes = un.step_bytes();
                     for (int s = 0; s < prm.n_steps; ++s, rb.next(prm.ns_b)) {
@@ -573,7 +541,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
             int it = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
-                const ContractUnit un = contract_unit<THETA>(prm, u);
+                const ContractUnit un = contract_unit(prm, u);
                 const int n = mine < 2 ? un.Nt[mine] : 0;          // this issuer's columns
                 const bool own = mine == 2 && un.own0;
                 // its table rows and accumulators
@@ -650,8 +618,8 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
         };
         // the thread's place in the first chunk of unit u
         auto unit_at = [&](int u, const double *&p, int &lim) {
-            p = u < prm.n_units ? contract_row<THETA>(prm, contract_unit<THETA>(prm, u), crow) : nullptr;
-            lim = p ? (THETA ? prm.ldJ : prm.K) - 4 * quad : 0;  // (the cells past n_theta in a row of F are zeros)
+            p = u < prm.n_units ? contract_row(prm, contract_unit(prm, u), crow) : nullptr;
+            lim = p ? prm.n_p - 4 * quad : 0;
             p += 4 * quad;
         };
 
@@ -704,7 +672,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                     // sums, after its last chunk to memory (two steps of this item are split by
                     // now, so the MMAs have work as soon as the accumulators are free)
                     if (pu >= 0 && ok) {
-                        const ContractUnit un = contract_unit<THETA>(prm, pu);
+                        const ContractUnit un = contract_unit(prm, pu);
                         const int b = prm.nacc == 2 ? (it - 1) & 1 : 0, nth = prm.nacc == 2 ? (it - 1) >> 1 : it - 1;
                         ok = warp_all(mbar_wait(smem_u32(&e_full[(it - 1) & 3]), ((it - 1) >> 2) & 1, abort_flag, prm.err, budget) &&
                                       mbar_wait(smem_u32(&acc_full[b]), nth & 1, abort_flag, prm.err, budget));
@@ -725,18 +693,11 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                             Er = En;
                         }
                         const bool shifts = DS != 0 && !warp_all((sh_old | sh_new) == 0);
-                        double *dst = nullptr;  // column n of the unit: dst + n ldJ, or dst + (col0 + n)^2
-                        if (!last) {
-                        } else if (!THETA) {
-                            const long long r = un.row0 + row;
-                            if (r < prm.R) {
-                                const int i = (int)((unsigned)r / (unsigned)prm.n_t), j = (int)r - i * prm.n_t;
-                                dst = prm.dst + ((size_t)i * prm.P + un.col0) * prm.ldJ + j;
-                            }
-                        } else {
-                            const int i = (int)un.row0 + (un.order ? row >> 1 : row);
-                            if (i < prm.n_r)
-                                dst = prm.dst + (size_t)i * prm.KL + (un.order ? 2 * un.order - 1 + (row & 1) : 0);
+                        double *dst = nullptr;  // column n of the unit: dst + n ldJ
+                        const long long r = un.row0 + row;
+                        if (last && r < prm.R) {
+                            const int i = (int)((unsigned)r / (unsigned)prm.n_t), j = (int)r - i * prm.n_t;
+                            dst = prm.dst + ((size_t)i * prm.P + un.col0) * prm.ldJ + j;
                         }
                         const uint32_t col = tmem_base + (uint32_t)b * acc_stride + ((uint32_t)(q4 * 32) << 16);
                         const int e_base = 56 + (DS < 0 ? prm.ds : DS) + Er - 2154;
@@ -774,9 +735,9 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                             bool odd = Er >= kExpNan;
                             double x = scaled_i64(lo, hi, e_base + et, odd);
                             if (odd) x = scaled_i64_slow(lo, hi, e_base + et, Er);
-                            if (in) *out = THETA ? prm.scale * x : x;
+                            if (in) *out = x;
                         };
-                        const int *et = prm.et + (size_t)un.set * prm.et_ld;
+                        const int *et = prm.et + (size_t)un.set * kEtLd;
                         // groups of four columns, dealt to the four warps of a lane quarter (the
                         // padding up to Nt holds zeros); the column m = 0 of its own block, with its
                         // weights side by side, goes to the last of them
@@ -821,13 +782,11 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
                                 float a[kDig];
 #pragma unroll
                                 for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(t[i][e]);
-                                const int l = un.col0 + n + e;
-                                result(a, sAcc + (size_t)(n + e) * 128 + row, ee[e],
-                                       THETA ? dst + (size_t)l * l : dst + (size_t)(n + e) * prm.ldJ,
+                                result(a, sAcc + (size_t)(n + e) * 128 + row, ee[e], dst + (size_t)(n + e) * prm.ldJ,
                                        dst && n + e < un.N);
                             }
                         }
-                        if (!THETA && un.own0 && grp == 3) {
+                        if (un.own0 && grp == 3) {
                             uint32_t w[8];
                             tmem_ld8(col + (uint32_t)(kDig * un.Nt[0]), w);
                             tmem_ld_wait();
@@ -873,7 +832,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const ContractPa
             c = c2;
             ++it;
         }
-        if (bad && !THETA) atomicOr(prm.err, DEV_ERR_NONFINITE);
+        if (bad) atomicOr(prm.err, DEV_ERR_NONFINITE);
     }
     tc_fence_before();
     __syncthreads();
@@ -1374,8 +1333,7 @@ bool plan_fp64_tc(mp_mesh *m, bool far_moments)
     f.npass = (cols + kNtMax - 1) / kNtMax;
     f.pass_cols = (cols + f.npass - 1) / f.npass;
     if (f.npass > 1) f.pass_cols = std::min(kNtMax, ceil16(f.pass_cols));
-    if (m->L > 71 || m->R >= (1LL << 31) || !plan_contract(m->n_t, std::min(m->L + 1, kNtMax), 0, f.th_c) ||
-        !plan_expand(m->L + 1, f.th_x)) {
+    if (m->L > 71 || m->R >= (1LL << 31) || !plan_expand(m->L + 1, f.th_x)) {
         f = Fp64Plan();  // the CUDA-core path and its layouts
         return false;
     }
@@ -1402,28 +1360,21 @@ size_t fp64_tc_arena(mp_mesh *m)
         at = align256(at + bytes);
         return o;
     };
-    const int n_sets = L + 1 + set_extra(L);
-    f.off_ld = n_sets + 1;
-    f.h_off.assign((size_t)4 * f.off_ld, 0);
-    unsigned long long *oc = f.h_off.data(), *ox = oc + f.off_ld, *op = ox + f.off_ld;
-    unsigned long long c = 0, x = 0;
+    f.off_ld = std::max(L + 1, f.npass);
+    f.h_off.assign((size_t)3 * f.off_ld, 0);
+    unsigned long long *ox = f.h_off.data(), *op = ox + f.off_ld;
+    unsigned long long x = 0;
     const int n_blk = (m->n_t + kNtX - 1) / kNtX;
-    for (int s = 0; s < n_sets; ++s) {
-        oc[s] = c;
-        if (f.mom_on) c += (unsigned long long)f.th_c.n_steps * kDig * (half_cols(set_cols(s, L), 0) + half_cols(set_cols(s, L), 1)) * 32;
-    }
     for (int mm = 0; mm <= L; ++mm) {
         ox[mm] = x;
         x += (unsigned long long)n_blk * ((L + 1 - mm + 15) / 16) * kRowsX * 32;
     }
     const unsigned long long pstep = (unsigned long long)f.ph_c.n_steps * f.ph_c.slot_b;
     for (int s = 0; s < f.npass; ++s) op[s] = s * pstep;
-    f.o_tab_c = take(c);
     f.o_tab_x = take(x);
     f.o_tab_pc = take(f.phi_on && f.mom_on ? f.npass * pstep : 0);
     f.o_tab_px = take(f.phi_on ? (size_t)((m->n_p + kNtX - 1) / kNtX) * std::max(1, (m->P - 1 + 15) / 16) * kRowsX * 32 : 0);
     f.o_off = take(f.h_off.size() * sizeof(unsigned long long));
-    f.o_et_c = take((size_t)n_sets * kEtLd * 4);
     f.o_et_x = take((size_t)(L + 1) * round_up(m->n_t, kNtX) * 4);
     f.o_et_pc = take((size_t)f.npass * kEtLd * 4);
     f.o_bound = take(4 * sizeof(int));
@@ -1436,26 +1387,23 @@ static const unsigned long long *fp64_off(const mp_mesh *m, int which)
     return reinterpret_cast<const unsigned long long *>(m->fp.arena + m->fp.o_off) + (size_t)which * m->fp.off_ld;
 }
 
-// The contraction's variants: theta or phi step, 32-byte loads, the bits dropped from a chain's sum
+// The contraction's variants: 32-byte loads, the bits dropped from a chain's sum
 // (none for one chain; 2 for up to 4, 4 for up to 16, the number of bits at run time beyond) and,
 // for several chains, whether the table keeps the first three accumulators below 2^22.
 template <int NM>
-static void (*contract_kernel_nm(int theta, int vec, int ds, int n_chunks))(ContractParams)
+static void (*contract_kernel_nm(int vec, int ds, int n_chunks))(ContractParams)
 {
     auto pick = [&](auto k0, auto k2, auto k4, auto kr) {
         return n_chunks == 1 ? k0 : ds == 2 ? k2 : ds == 4 ? k4 : kr;
     };
-    if (theta)
-        return pick(k64_contract_tc<true, true, 0, 2>, k64_contract_tc<true, true, 2, NM>,
-                    k64_contract_tc<true, true, 4, NM>, k64_contract_tc<true, true, -1, 2>);
-    return vec ? pick(k64_contract_tc<false, true, 0, 2>, k64_contract_tc<false, true, 2, NM>,
-                      k64_contract_tc<false, true, 4, NM>, k64_contract_tc<false, true, -1, 2>)
-               : pick(k64_contract_tc<false, false, 0, 2>, k64_contract_tc<false, false, 2, NM>,
-                      k64_contract_tc<false, false, 4, NM>, k64_contract_tc<false, false, -1, 2>);
+    return vec ? pick(k64_contract_tc<true, 0, 2>, k64_contract_tc<true, 2, NM>, k64_contract_tc<true, 4, NM>,
+                      k64_contract_tc<true, -1, 2>)
+               : pick(k64_contract_tc<false, 0, 2>, k64_contract_tc<false, 2, NM>, k64_contract_tc<false, 4, NM>,
+                      k64_contract_tc<false, -1, 2>);
 }
-static void (*contract_kernel(int theta, int vec, int ds, int n_chunks, int small))(ContractParams)
+static void (*contract_kernel(int vec, int ds, int n_chunks, int small))(ContractParams)
 {
-    return small ? contract_kernel_nm<3>(theta, vec, ds, n_chunks) : contract_kernel_nm<2>(theta, vec, ds, n_chunks);
+    return small ? contract_kernel_nm<3>(vec, ds, n_chunks) : contract_kernel_nm<2>(vec, ds, n_chunks);
 }
 
 static void (*expand_kernel(int theta, int nm))(const CUtensorMap, ExpandParams)
@@ -1479,19 +1427,18 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
                     reinterpret_cast<int *>(f.arena + f.o_bound) + kind};
         k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t, n_sets);
     };
-    if (f.mom_on) build(TAB_CONTRACT, f.o_tab_c, 0, f.o_et_c, kEtLd, std::min(L + 1, kNtMax), L + 1 + set_extra(L));
-    build(TAB_EXPAND_TH, f.o_tab_x, 1, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
-    if (f.phi_on && f.mom_on) build(TAB_PROJECT, f.o_tab_pc, 2, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
-    if (f.phi_on) build(TAB_EXPAND_PH, f.o_tab_px, 3, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
+    build(TAB_EXPAND_TH, f.o_tab_x, 0, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
+    if (f.phi_on && f.mom_on) build(TAB_PROJECT, f.o_tab_pc, 1, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
+    if (f.phi_on) build(TAB_EXPAND_PH, f.o_tab_px, 2, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
     // 227 KB of dynamic shared memory for the kernels of this file (per device)
+    for (int vec = 0; vec < 2; ++vec)
+        for (int v = 0; v < 8; ++v) {
+            const int ds = v < 6 ? (v >> 1) * 2 : 5;
+            e = cudaFuncSetAttribute((const void *)contract_kernel(vec, ds, ds ? 2 : 1, v & 1),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+            if (e != cudaSuccess) return e;
+        }
     for (int theta = 0; theta < 2; ++theta) {
-        for (int vec = 0; vec < 2; ++vec)
-            for (int v = 0; v < 8; ++v) {
-                const int ds = v < 6 ? (v >> 1) * 2 : 5;
-                e = cudaFuncSetAttribute((const void *)contract_kernel(theta, theta || vec, ds, ds ? 2 : 1, v & 1),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-                if (e != cudaSuccess) return e;
-            }
         for (int nm : {1, 3, 6}) {
             e = cudaFuncSetAttribute((const void *)expand_kernel(theta, nm), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kSmemMax);
@@ -1503,46 +1450,12 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
 
 cudaError_t fp64_tc_bounds(mp_mesh *m)
 {
-    int b[4] = {0, 0, 0, 0};
+    int b[3] = {0, 0, 0};
     cudaError_t e = cudaMemcpy(b, m->fp.arena + m->fp.o_bound, sizeof(b), cudaMemcpyDeviceToHost);
     m->fp.ph_c.small = b[TAB_PROJECT] < (1 << 22);
-    m->fp.th_c.small = b[TAB_CONTRACT] < (1 << 22);
     m->fp.th_x.small = b[TAB_EXPAND_TH] < (1 << 22);
     m->fp.ph_x.small = b[TAB_EXPAND_PH] < (1 << 22);
     return e;
-}
-
-static cudaError_t launch_contract(mp_mesh *m, int theta, const double *src, double *dst, const char *name)
-{
-    const Fp64Plan &f = m->fp;
-    const Fp64Contract &c = theta ? f.th_c : f.ph_c;
-    ContractParams p{};
-    p.src = src;
-    p.dst = dst;
-    p.tab = f.arena + (theta ? f.o_tab_c : f.o_tab_pc);
-    p.off = fp64_off(m, theta ? 0 : 2);
-    p.et = reinterpret_cast<const int *>(f.arena + (theta ? f.o_et_c : f.o_et_pc));
-    p.err = m->d_err;
-    p.R = m->R;
-    p.n_r = m->n_r, p.n_t = m->n_t, p.n_p = m->n_p, p.L = m->L, p.KL = m->KL, p.P = m->P, p.ldJ = f.ldJ;
-    p.K = theta ? m->n_t : m->n_p;
-    p.n_steps = c.n_steps, p.n_chunks = c.n_chunks, p.ds = c.ds;
-    p.npass = f.npass, p.pass_cols = f.pass_cols, p.m0 = f.m0;
-    p.n_groups = (m->n_r + 63) / 64, p.n_groups0 = (m->n_r + 127) / 128;
-    const int extra = set_extra(m->L);
-    p.n_units = theta ? p.n_groups0 * (extra ? 2 : 1) + (m->L + std::max(0, extra - 1)) * p.n_groups : (int)((m->R + 127) / 128) * f.npass;
-    p.et_ld = kEtLd;
-    p.ns_a = c.ns_a, p.ns_b = c.ns_b, p.nacc = c.nacc, p.slot_b = c.slot_b, p.cols_max = c.cols_max;
-    p.scale = 12.566370614359172954 * m->G;
-    // 32-byte loads where every row starts on a 32-byte boundary
-    const bool vec = theta || (m->n_p % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 31) == 0);
-    auto kern = contract_kernel(theta, vec, c.ds, c.n_chunks, c.small);
-    cudaEvent_t ev;
-    prof_begin(m, name, &ev);
-    cudaError_t e = launch_pdl(kern, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreadsC), c.smem,
-                               m->stream, p);
-    prof_end(m, name, ev);
-    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 static cudaError_t launch_expand(mp_mesh *m, int theta, const double *src, double *dst, const char *name)
@@ -1553,7 +1466,7 @@ static cudaError_t launch_expand(mp_mesh *m, int theta, const double *src, doubl
     p.src = src;
     p.dst = dst;
     p.tab = f.arena + (theta ? f.o_tab_x : f.o_tab_px);
-    p.off = fp64_off(m, theta ? 1 : 3);
+    p.off = fp64_off(m, theta ? 0 : 2);
     p.et = reinterpret_cast<const int *>(f.arena + (theta ? f.o_et_x : f.o_et_px));
     p.err = m->d_err;
     p.R = m->R;
@@ -1590,11 +1503,30 @@ static cudaError_t launch_expand(mp_mesh *m, int theta, const double *src, doubl
 
 cudaError_t launch_fp64_tc_project(mp_mesh *m, const double *rho)
 {
-    return launch_contract(m, 0, rho, m->d_F64, "fp64_phi_project");
-}
-cudaError_t launch_fp64_tc_theta(mp_mesh *m)
-{
-    return launch_contract(m, 1, m->d_F64, m->d_A, "fp64_theta_contract");
+    const Fp64Plan &f = m->fp;
+    const Fp64Contract &c = f.ph_c;
+    ContractParams p{};
+    p.src = rho;
+    p.dst = m->d_F64;
+    p.tab = f.arena + f.o_tab_pc;
+    p.off = fp64_off(m, 1);
+    p.et = reinterpret_cast<const int *>(f.arena + f.o_et_pc);
+    p.err = m->d_err;
+    p.R = m->R;
+    p.n_t = m->n_t, p.n_p = m->n_p, p.P = m->P, p.ldJ = f.ldJ;
+    p.n_steps = c.n_steps, p.n_chunks = c.n_chunks, p.ds = c.ds;
+    p.npass = f.npass, p.pass_cols = f.pass_cols, p.m0 = f.m0;
+    p.n_units = (int)((m->R + 127) / 128) * f.npass;
+    p.ns_a = c.ns_a, p.ns_b = c.ns_b, p.nacc = c.nacc, p.slot_b = c.slot_b, p.cols_max = c.cols_max;
+    // 32-byte loads where every row starts on a 32-byte boundary
+    const bool vec = m->n_p % 4 == 0 && (reinterpret_cast<uintptr_t>(rho) & 31) == 0;
+    auto kern = contract_kernel(vec, c.ds, c.n_chunks, c.small);
+    cudaEvent_t ev;
+    prof_begin(m, "fp64_phi_project", &ev);
+    cudaError_t e = launch_pdl(kern, dim3(std::min(p.n_units, m->num_sms)), dim3(kThreadsC), c.smem,
+                               m->stream, p);
+    prof_end(m, "fp64_phi_project", ev);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 cudaError_t launch_fp64_tc_synth_theta(mp_mesh *m)
 {

@@ -68,16 +68,15 @@ struct Fp64Expand {
     int a_steps = 0, ns_b = 0, smem = 0, small = 0;
 };
 struct Fp64Plan {
-    int on = 0;      // theta stages (and the layouts F, G [n_r][P][ldJ], C [K_L][ldI])
+    int on = 0;      // theta synthesis (and the layouts G [n_r][P][ldJ], C [K_L][ldI])
     int phi_on = 0;  // phi stages too
-    int mom_on = 0;  // the projection and the theta contraction among them (else F [R][P])
+    int mom_on = 0;  // the projection among them, and F as [n_r][P][ldJ] (else [R][P])
     int ldJ = 0, ldI = 0, npass = 1, pass_cols = 0, m0 = 0, off_ld = 0;
-    Fp64Contract ph_c, th_c;
+    Fp64Contract ph_c;
     Fp64Expand ph_x, th_x;
-    size_t o_tab_c = 0, o_tab_x = 0, o_tab_pc = 0, o_tab_px = 0, o_off = 0, o_et_c = 0, o_et_x = 0, o_et_pc = 0,
-           o_et_px = 0, o_bound = 0, arena_bytes = 0;
+    size_t o_tab_x = 0, o_tab_pc = 0, o_tab_px = 0, o_off = 0, o_et_x = 0, o_et_pc = 0, o_et_px = 0, o_bound = 0, arena_bytes = 0;
     uint8_t *arena = nullptr;
-    std::vector<unsigned long long> h_off;  // table offsets per order / pass, four lists of off_ld
+    std::vector<unsigned long long> h_off;  // table offsets per order / pass, three lists of off_ld
 };
 
 // Where the radial recurrences write the solution coefficients C[i][l^2 + p] (m >= 1) as
@@ -264,14 +263,13 @@ cudaError_t launch_fp64_synth(mp_mesh *m, double *phi);
 // step (a) in float64 with caller-provided workspace F [R][2L+1] and output A [n_r][K_L]
 cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double *F, double *A);
 
-// the same steps as exact integer slices on the tensor cores (F, G [n_r][P][ldJ], C [K_L][ldI])
+// steps (a1), (d1) and (d2) as exact integer slices on the tensor cores (F, G [n_r][P][ldJ], C [K_L][ldI])
 // (false: sizes out of its range, l_max > 71; far_moments: the moments stay on CUDA cores)
 bool plan_fp64_tc(mp_mesh *m, bool far_moments);
 size_t fp64_tc_arena(mp_mesh *m);          // lays the tables out; bytes of the arena
 cudaError_t launch_fp64_tc_tables(mp_mesh *m);
 cudaError_t fp64_tc_bounds(mp_mesh *m);    // reads what the finished tables say about the accumulators
 cudaError_t launch_fp64_tc_project(mp_mesh *m, const double *rho);
-cudaError_t launch_fp64_tc_theta(mp_mesh *m);
 cudaError_t launch_fp64_tc_synth_theta(mp_mesh *m);
 cudaError_t launch_fp64_tc_synth_phi(mp_mesh *m, double *phi);
 

@@ -3,7 +3,7 @@
 import numpy as np
 import pytest
 
-from gpu_helpers import gpu_solve
+from gpu_helpers import edge_term_errors, gpu_solve, moment_term_errors, oracle_solve, term_scales
 from paper_2602_02507_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -40,3 +40,26 @@ def test_moments_whose_squares_overflow_are_the_cuda_core_sums(shape, L):
     got = gpu_solve(w, "fp64")
     assert np.array_equal(got["A"], cuda_core_moments(w))
     assert np.all(np.isfinite(got["MR"])) and np.all(np.isfinite(got["MI"]))
+
+
+@pytest.mark.parametrize("L,center,width", [(8, 0.15, 0.05), (32, 0.15, 0.05), (32, 3.0, 0.02), (40, 0.4, 0.1), (71, 0.3, 0.1)])
+def test_every_moment_of_a_clump_near_the_pole(L, center, width):
+    """A clump beside the axis: its cells meet the smallest entries of the polar tables (sin^m
+    theta).  Every A_lm, M^R and M^I is within the float64 path's 1e-12 of the sum of the magnitudes
+    of its own terms; float64 sums of 128 + 256 terms stay below 400 * 2^-53 = 5e-14 of it."""
+    w = W.random_small((20, 128, 256), L, seed=L, r0=0.5, r1=1.0)
+    thc, phc = (0.5 * (e[1:] + e[:-1]) for e in (w.mesh.theta, w.mesh.phi))
+    w.rho *= np.exp(-((thc[:, None] - center) / width) ** 2 - ((phc[None, :] - 1.0) / 0.5) ** 2)[None]
+    ref, got = oracle_solve(w), gpu_solve(w, "fp64")
+    S = term_scales(w.rho, ref["tables"], w.mesh.G)
+    assert max(moment_term_errors(got["A"], ref["A"], S, L)) <= 1e-12
+    for key, errs in edge_term_errors(got, ref, S).items():
+        assert max(errs) <= 1e-12, key
+
+
+def test_theta_rows_are_summed_as_the_cuda_core_kernels_do():
+    """With few azimuthal cells both steps of the moments run on CUDA cores: blocks of 16 and 32
+    shells, 32 degrees and 32 polar cells, each with a remainder, equal k64_theta to the last bit."""
+    for shape, L in (((33, 33, 3), 33), ((17, 64, 2), 40), ((1, 1, 1), 0), ((40, 31, 15), 64), ((16, 70, 1), 31)):
+        w = W.random_small(shape, L, seed=5, r0=0.9, r1=1.0, uneven=True)
+        assert np.array_equal(gpu_solve(w, "fp64")["A"], cuda_core_moments(w)), (shape, L)
