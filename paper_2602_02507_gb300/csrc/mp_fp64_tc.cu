@@ -45,8 +45,9 @@
 // long expansion at 1024 x 256 x 512 cells, l_max = 32) nor HBM (24 and 34 %), but the integer
 // instructions that split and rejoin the operands (half the rate of float32's: their pipe is 50 and
 // 58 % busy) and the hand-offs between the warps that issue them.  Measured there against float64
-// on CUDA cores: (a1) 29.5 ms -> 653 us, (d1) 2143 -> 66 us, (d2) 13.9 ms -> 427 us; at 512 x 128 x
-// 256, l_max = 16: 1918 -> 87, 200 -> 16, 891 -> 69 us.
+// on CUDA cores: (a1) 29.5 ms -> 691 us, (d1) 2143 -> 66 us, (d2) 13.9 ms -> 427 us; at 512 x 128 x
+// 256, l_max = 16: 1918 -> 91, 200 -> 16, 891 -> 69 us.  (Rounding the operands instead of
+// truncating them is 38 and 3 us of (a1).)
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -105,18 +106,22 @@ __host__ __device__ inline int half_cols(int N, int h)
 }
 
 // ---------------------------------------------------------------------------- digits
-// |x| as a 55-bit integer relative to the row exponent (x = +- V 2^(E - 1077), V < 2^55,
-// truncated), with 0x80 added to its six low bytes: byte b of the sum less 128 is then a
-// balanced digit, and the seventh byte the leading one (0 .. 128).  e9 = E + 9.
-__device__ __forceinline__ void fix55(uint32_t lo, uint32_t hi, int e9, uint32_t &wl, uint32_t &wh)
+// |x| as a 55-bit integer relative to the row exponent (x = +- V 2^(E - 1077), V <= 2^55, rounded
+// to nearest: truncation takes up to one unit off every cell of a ring in the same direction), with
+// 0x80 added to its six low bytes: byte b of the sum less 128 is then a balanced digit, and the
+// seventh byte the leading one (0 .. 128).  e8 = E + 8.  The integer is formed with one bit more, so
+// that its rounding rides on the addition and costs the two shifts behind it.
+__device__ __forceinline__ void fix55(uint32_t lo, uint32_t hi, int e8, uint32_t &wl, uint32_t &wh)
 {
-    const int n = e9 - (int)((hi >> 20) & 0x7FFu);
+    const int n = e8 - (int)((hi >> 20) & 0x7FFu);
     const uint32_t th = __funnelshift_l(lo, hi, 11) | 0x80000000u, tl = lo << 11;
     uint32_t vl = __funnelshift_rc(tl, th, n), vh;
     asm("shr.u32 %0, %1, %2;" : "=r"(vh) : "r"(th), "r"(n));
     const int n2 = max(n - 32, 0);
     asm("shr.u32 %0, %1, %2;" : "=r"(vl) : "r"(vl), "r"(n2));
-    asm("add.cc.u32 %0, %2, 0x80808080;\n\taddc.u32 %1, %3, 0x00008080;" : "=r"(wl), "=r"(wh) : "r"(vl), "r"(vh));
+    asm("add.cc.u32 %0, %2, 0x01010101;\n\taddc.u32 %1, %3, 0x00010101;" : "=r"(wl), "=r"(wh) : "r"(vl), "r"(vh));
+    wl = __funnelshift_r(wl, wh, 1);
+    wh >>= 1;
 }
 
 // The digits of two neighbouring values as float16 pairs, d[0] the leading one: byte b becomes
@@ -292,6 +297,9 @@ __device__ __forceinline__ bool scaled_row(const uint32_t (&lo)[N], const uint32
     return least != 0;
 }
 
+// x 2^-n (n <= 62), rounded to nearest.
+__device__ __forceinline__ long long shift_round(long long x, int n) { return (x + ((1ll << n) >> 1)) >> n; }
+
 // ---------------------------------------------------------------------------- tables
 enum { TAB_PROJECT = 0, TAB_EXPAND_TH = 1, TAB_EXPAND_PH = 2 };
 
@@ -362,7 +370,7 @@ __global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n
             const double x = tab_value(t, set, n, k);
             const uint32_t hi = (uint32_t)__double2hiint(x);
             uint32_t wl, wh, d[kDig];
-            fix55((uint32_t)__double2loint(x), hi, E + 9, wl, wh);
+            fix55((uint32_t)__double2loint(x), hi, E + 8, wl, wh);
             if ((hi & 0x7FF00000u) == 0) wl = 0x80808080u, wh = 0x00008080u;  // zeros stay zeros
             digits2(wl, wh, hi, wl, wh, hi, d);
 #pragma unroll
@@ -650,7 +658,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
             if (quad == 0 && steps) sE[(it & 3) * 128 + crow] = tiny ? E - 300 : E;
             __syncwarp();
             if (lane == 0 && steps) mbar_arrive(smem_u32(&e_full[it & 3]));
-            const int e9 = E + 9;
+            const int e8 = E + 8;
             if (c2) {
                 src += 16 * kChunkSteps;
                 lim -= 16 * kChunkSteps;
@@ -688,8 +696,8 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
                             Er = Ec;
                         } else {
                             const int En = max(Er, Ec);
-                            sh_old = min(63, En - Er);
-                            sh_new = min(63, En - Ec + dsr);
+                            sh_old = min(62, En - Er);
+                            sh_new = min(62, En - Ec + dsr);
                             Er = En;
                         }
                         const bool shifts = DS != 0 && !warp_all((sh_old | sh_new) == 0);
@@ -709,18 +717,18 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
                                 long long x, o = 0;
                                 if (pc > 0) {
                                     o = *pa;
-                                    if (shifts) o >>= sh_old;
+                                    if (shifts) o = shift_round(o, sh_old);
                                 }
                                 if (DS > 0 && NM >= 3) {
                                     x = (long long)acc_sum_chain<(DS > 0 ? DS : 2)>(a);
                                     if (shifts)
-                                        x = ((x - (long long)ChainOff<(DS > 0 ? DS : 2)>::value) >> sh_new) + o;
+                                        x = shift_round(x - (long long)ChainOff<(DS > 0 ? DS : 2)>::value, sh_new) + o;
                                     else
                                         x = x + o - (long long)ChainOff<(DS > 0 ? DS : 2)>::value;
                                 } else {
                                     acc_sum<NM, (DS > 0 ? DS : 0)>(a, lo, hi);
                                     x = (long long)(((unsigned long long)hi << 32) | lo);
-                                    if (shifts) x >>= sh_new;
+                                    if (shifts) x = shift_round(x, sh_new);
                                     x += o;
                                 }
                                 if (!last) {
@@ -811,7 +819,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
                     if (tiny) scale_up(v[s]);
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        fix55((uint32_t)__double2loint(v[s][e]), (uint32_t)__double2hiint(v[s][e]), e9, wl[e], wh[e]);
+                        fix55((uint32_t)__double2loint(v[s][e]), (uint32_t)__double2hiint(v[s][e]), e8, wl[e], wh[e]);
                     digits2(wl[0], wh[0], (uint32_t)__double2hiint(v[s][0]), wl[1], wh[1],
                             (uint32_t)__double2hiint(v[s][1]), d0);
                     digits2(wl[2], wh[2], (uint32_t)__double2hiint(v[s][2]), wl[3], wh[3],
@@ -1108,7 +1116,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                 E0 = -300;
             }
             const int Erow = E + E0;
-            const int e9 = E + 9;
+            const int e8 = E + 8;
             // in units of 2^56: 1.0 in the table would be 2^54, so a quarter of its 55-bit integer
             uint32_t g0_lo = 0, g0_hi = 0;
             if (!THETA) {
@@ -1118,7 +1126,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                     g0 = t[0];
                 }
                 uint32_t wl, wh;
-                fix55((uint32_t)__double2loint(g0), (uint32_t)__double2hiint(g0), e9, wl, wh);
+                fix55((uint32_t)__double2loint(g0), (uint32_t)__double2hiint(g0), e8, wl, wh);
                 long long q = (long long)((((unsigned long long)wh << 32 | wl) - 0x0000808080808080ull + 2) >> 2);
                 if (g0 < 0.0) q = -q;
                 g0_lo = (uint32_t)q;
@@ -1132,8 +1140,8 @@ __global__ void __launch_bounds__(kThreadsX, 1) k64_expand_tc(const __grid_const
                 for (int e = 0; e < 8; e += 2) {
                     uint32_t wl0, wh0, wl1, wh1;
                     const uint32_t h0 = (uint32_t)__double2hiint(x[e]), h1 = (uint32_t)__double2hiint(x[e + 1]);
-                    fix55((uint32_t)__double2loint(x[e]), h0, e9, wl0, wh0);
-                    fix55((uint32_t)__double2loint(x[e + 1]), h1, e9, wl1, wh1);
+                    fix55((uint32_t)__double2loint(x[e]), h0, e8, wl0, wh0);
+                    fix55((uint32_t)__double2loint(x[e + 1]), h1, e8, wl1, wh1);
                     digits2(wl0, wh0, h0, wl1, wh1, h1, d[e >> 1]);
                 }
                 uint8_t *dst = sA + (size_t)((o >> 1) - s0) * kStepA2 + (o & 1) * kLboA2 + crow * 16;

@@ -63,3 +63,23 @@ def test_theta_rows_are_summed_as_the_cuda_core_kernels_do():
     for shape, L in (((33, 33, 3), 33), ((17, 64, 2), 40), ((1, 1, 1), 0), ((40, 31, 15), 64), ((16, 70, 1), 31)):
         w = W.random_small(shape, L, seed=5, r0=0.9, r1=1.0, uneven=True)
         assert np.array_equal(gpu_solve(w, "fp64")["A"], cuda_core_moments(w)), (shape, L)
+
+
+@pytest.mark.parametrize("n_phi", [128, 500, 2048])
+def test_small_cells_beside_a_large_one_are_rounded_both_ways(n_phi):
+    """One cell of each ring is 2^30 times the others: their last bits do not fit the ring's fixed
+    point.  Truncated, they would take n_phi 2^-56 off the monopole; rounded to nearest they leave
+    sqrt(n_phi) 2^-57, below the rounding of the 16 polar terms and their table (16 * 2^-53) and
+    of the sums of the chains of 128 cells (2^-50 of the hot cell for 2048): 5e-15 holds both."""
+    w = W.random_small((4, 16, n_phi), 2, seed=n_phi, r0=0.5, r1=1.0)
+    rng = np.random.default_rng(n_phi)
+    w.rho *= 2.0 ** -30
+    hot = rng.integers(0, n_phi, (4, 16))
+    np.put_along_axis(w.rho, hot[:, :, None], 1.0, axis=2)
+    m = w.mesh
+    LD = np.longdouble
+    polar = -np.diff(np.cos(m.theta.astype(LD)))
+    ring = (w.rho.astype(LD) * np.diff(m.phi.astype(LD))).sum(axis=2)
+    exact = (ring * polar).sum(axis=1) * np.sqrt(4 * np.arccos(LD(-1)))
+    got = gpu_solve(w, "fp64")["A"][:, 0]
+    assert np.max(np.abs(got - exact) / exact) <= 5e-15
