@@ -20,8 +20,8 @@
 // keeps 55 - k bits.  A result of K terms is off by at most about K 2^-54 x (row maximum) x (column
 // maximum), whether or not the two maxima meet at one index, where a float64 sum is off by a
 // multiple of 2^-53 of the sum of its terms' magnitudes.  The steps below can afford that: the
-// azimuthal tables are of one size along a row of cells and themselves off by the rounding of
-// m phi, 2^-53 m phi of their maximum; and the synthesis delivers Phi alone, whose sum over the
+// azimuthal tables are of one size along a row of cells (a factor of two in their widths is let in)
+// and themselves off by the rounding of m phi, 2^-53 m phi of their maximum; and the synthesis delivers Phi alone, whose sum over the
 // orders is of the size of the row maxima (errors stay at 2^-53 of the largest |Phi| of the
 // shell; G of an order m near the poles, a small part of it there, is less accurate by itself).
 // The theta part of the moments cannot (sin^m theta against a clump near the pole): it is summed
@@ -49,6 +49,7 @@
 // 256, l_max = 16: 1918 -> 91, 200 -> 16, 891 -> 69 us.  (Rounding the operands instead of
 // truncating them is 38 and 3 us of (a1).)
 #include <algorithm>
+#include <cmath>
 
 #include <cuda_fp16.h>
 
@@ -1353,7 +1354,18 @@ bool plan_fp64_tc(mp_mesh *m, bool far_moments)
     // and equality is the one way to compare them.  They stay sums in the order of the CUDA-core
     // kernels, those of mp_moments_noalloc, to the last bit.  It costs their speed: 260 x 130 x 150
     // cells, l_max = 64: 346 -> 1860 us a solve (3594 with the synthesis on CUDA cores as well).
-    f.mom_on = !far_moments;
+    //
+    // Azimuthal cells of widths more than a factor of two apart leave the projection there too: its
+    // fixed point is that of the widest cell, so the others of a ring whose largest cell is narrow
+    // are off by up to K 2^-56 x (widest / narrowest) of what the largest adds, K 2^-53 in a float64
+    // sum with two bits less for where the values lie between powers of two.  (One of 64 cells 1e-6
+    // as wide, and hot: 3e-11 of the moments' terms.)
+    double widest = 0.0, narrowest = HUGE_VAL;
+    for (int k = 0; k < m->n_p; ++k) {
+        widest = std::max(widest, m->h_ph[k + 1] - m->h_ph[k]);
+        narrowest = std::min(narrowest, m->h_ph[k + 1] - m->h_ph[k]);
+    }
+    f.mom_on = !far_moments && (!f.phi_on || widest <= 2.0 * narrowest);
     f.on = 1;
     return true;
 }

@@ -83,3 +83,21 @@ def test_small_cells_beside_a_large_one_are_rounded_both_ways(n_phi):
     exact = (ring * polar).sum(axis=1) * np.sqrt(4 * np.arccos(LD(-1)))
     got = gpu_solve(w, "fp64")["A"][:, 0]
     assert np.max(np.abs(got - exact) / exact) <= 5e-15
+
+
+@pytest.mark.parametrize("ratio", [1e-6, 0.04, 0.7])
+def test_a_large_density_in_a_narrow_azimuthal_cell(ratio):
+    """The other cells of the ring keep their bits beside a hot cell that is narrow: within 1e-13 of
+    the sum of the terms' magnitudes (float64 sums of 32 + 64 terms: 96 * 2^-53 = 1.1e-14, and
+    tables that agree to a few 1e-14)."""
+    w = W.random_small((8, 32, 64), 12, seed=3, r0=0.5, r1=1.0)
+    width = np.ones(64)
+    width[10] = ratio
+    edges = np.concatenate([[0.0], np.cumsum(width)])
+    w.mesh.phi[:] = edges / edges[-1] * 2.0 * np.pi
+    w.rho[:] = 1e-6
+    w.rho[:, :, 10] = np.exp(0.5 * (w.mesh.r[1:] + w.mesh.r[:-1]))[:, None]
+    ref, got = oracle_solve(w), gpu_solve(w, "fp64")
+    S = term_scales(w.rho, ref["tables"], w.mesh.G)
+    assert max(moment_term_errors(got["A"], ref["A"], S, 12)) <= 1e-13
+    assert np.max(np.abs(got["phi"] - ref["phi"]) / np.abs(ref["phi"])) <= 1e-12
