@@ -53,6 +53,7 @@
 
 #include <cuda_fp16.h>
 
+#include "mp_fp64_join.h"
 #include "mp_internal.h"
 #include "ptx.cuh"
 
@@ -256,7 +257,7 @@ __device__ __forceinline__ void acc_sum_small(const float (&t)[kDig], uint32_t &
 }
 
 // One chain of several (DS >= 2) whose first three accumulators stay below 2^22 (the next two may
-// not, and are converted): the integers keep their offsets as in acc_sum_small, kChainOff in all.
+// not, and are converted): the integers keep their offsets as in acc_sum_small, ChainJoin's in all.
 template <int DS>
 __device__ __forceinline__ unsigned long long acc_sum_chain(const float (&t)[kDig])
 {
@@ -265,15 +266,10 @@ __device__ __forceinline__ unsigned long long acc_sum_chain(const float (&t)[kDi
 #pragma unroll
     for (int i = 0; i < 3; ++i) a[i] = (uint32_t)__float_as_int(t[i] + 12582912.0f);
     const uint32_t a5 = (uint32_t)__float_as_int(fmaf(t[6], w6, t[5] * w5) + 12582912.0f);
-    const uint32_t a3 = (uint32_t)__float2int_rn(t[3]), a4 = (uint32_t)__float2int_rn(t[4]);
-    return (unsigned long long)(a[2] * 256u + a3) * (65536u >> DS) + (a4 * (256u >> DS) + a5) +
-           (unsigned long long)(a[0] * 256u + a[1]) * ((1ull << 32) >> DS);
+    // (the offset of a3 is exact: the sum is an integer up to 2^24)
+    const uint32_t a3 = (uint32_t)__float2int_rn(t[3] + 8388608.0f), a4 = (uint32_t)__float2int_rn(t[4]);
+    return ChainJoin<DS>::sum(a[0], a[1], a[2], a3, a4, a5);
 }
-template <int DS>
-struct ChainOff {
-    static constexpr unsigned long long pair = 0x4B400000u * 257u, one = 0x4B400000u * 256u;  // modulo 2^32
-    static constexpr unsigned long long value = one * (65536u >> DS) + 0x4B400000u + pair * ((1ull << 32) >> DS);
-};
 
 // Eight results of one row at once: hi:lo 2^(e0 + et) as in scaled_i64, for integers of 33 bits or
 // more (the common case); false when one is smaller.
@@ -723,9 +719,9 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
                                 if (DS > 0 && NM >= 3) {
                                     x = (long long)acc_sum_chain<(DS > 0 ? DS : 2)>(a);
                                     if (shifts)
-                                        x = shift_round(x - (long long)ChainOff<(DS > 0 ? DS : 2)>::value, sh_new) + o;
+                                        x = shift_round(x - (long long)ChainJoin<(DS > 0 ? DS : 2)>::offset, sh_new) + o;
                                     else
-                                        x = x + o - (long long)ChainOff<(DS > 0 ? DS : 2)>::value;
+                                        x = x + o - (long long)ChainJoin<(DS > 0 ? DS : 2)>::offset;
                                 } else {
                                     acc_sum<NM, (DS > 0 ? DS : 0)>(a, lo, hi);
                                     x = (long long)(((unsigned long long)hi << 32) | lo);
@@ -772,7 +768,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) k64_contract_tc(const __grid_con
                                     float a[kDig];
 #pragma unroll
                                     for (int i = 0; i < kDig; ++i) a[i] = __uint_as_float(t[i][e]);
-                                    pa[e * 128] = acc_sum_chain<(DS > 0 ? DS : 2)>(a) + o[e] - ChainOff<(DS > 0 ? DS : 2)>::value;
+                                    pa[e * 128] = acc_sum_chain<(DS > 0 ? DS : 2)>(a) + o[e] - ChainJoin<(DS > 0 ? DS : 2)>::offset;
                                 }
                             }
                         } else
