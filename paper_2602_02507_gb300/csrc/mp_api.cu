@@ -516,16 +516,16 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
     ALLOC(m->d_err, 4);
     ALLOC(m->d_slab_off, (size_t)2 * m->KL);  // radial sums of the other slabs (slab meshes)  // [0] error word, [2..3] budget of the pipeline waits (int64, 0: default)
     if (m->eff_prec == MP_PREC_FP64) {
-        if (m->fp.on) {
-            ALLOC(m->d_F64, (size_t)n_r * m->P * m->fp.ldJ);
-            ALLOC(m->d_G64, (size_t)n_r * m->P * m->fp.ldJ);
+        const Fp64Plan &f = m->fp;
+        ALLOC(m->d_F64, (size_t)n_r * m->P * (f.rows ? f.ldJ : n_theta));
+        ALLOC(m->d_G64, (size_t)n_r * m->P * (f.on ? f.ldJ : n_theta));
+        if (f.proj_on || f.on) {
             m->fp.arena_bytes = fp64_tc_arena(m);
             ALLOC(m->fp.arena, m->fp.arena_bytes);
-            st = make_map_f64_G(&m->tm_G64, m->d_G64, n_r, m->P, n_theta, m->fp.ldJ);
+        }
+        if (f.on) {
+            st = make_map_f64_G(&m->tm_G64, m->d_G64, n_r, m->P, n_theta, f.ldJ);
             if (st != MP_OK) return fail(st);
-        } else {
-            ALLOC(m->d_F64, (size_t)m->R * m->P);
-            ALLOC(m->d_G64, (size_t)m->R * m->P);
         }
     } else {
         st = plan_split(m);
@@ -599,7 +599,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         if (st != MP_OK) return fail(st);
         st = cuda_status(launch_tables(m), "build tables");
         if (st != MP_OK) return fail(st);
-        if (m->fp.on) {
+        if (m->fp.arena) {
             st = cuda_status(launch_fp64_tc_tables(m), "build float64 digit tables");
             if (st != MP_OK) return fail(st);
         }
@@ -611,7 +611,7 @@ static mp_status create_mesh(const double *r_edges, int n_r, const double *theta
         }
         st = cuda_status(cudaStreamSynchronize(m->stream), "table build");
         if (st != MP_OK) return fail(st);
-        if (m->fp.on) {
+        if (m->fp.arena) {
             st = cuda_status(fp64_tc_bounds(m), "float64 table bounds");
             if (st != MP_OK) return fail(st);
         }

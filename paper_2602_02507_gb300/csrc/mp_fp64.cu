@@ -1,8 +1,8 @@
 // mp_fp64.cu -- the float64 path: its contractions on CUDA cores in float64 (GB300's float64
 // rate bounds them) and the dispatch to their tensor-core form (mp_fp64_tc.cu).  The theta
 // contraction always runs here; the other steps do beyond the range of the tensor-core form (l_max >
-// 71), for a few azimuthal cells, for moments whose squares overflow, and in mp_moments_noalloc,
-// whose scratch is fixed.  A solve with the tensor-core steps against one without: 46.3 -> 1.63 ms at
+// 71), for small meshes and few azimuthal cells, for moments whose squares overflow, and in
+// mp_moments_noalloc, whose scratch is fixed.  A solve with the tensor-core steps against one without: 46.3 -> 1.63 ms at
 // 1024 x 256 x 512 cells, l_max = 32; 3.10 -> 0.22 ms at 512 x 128 x 256, 16; 1.53 -> 0.15 ms at 353 x
 // 96 x 192, 20; 340 -> 117 us at 471 x 128 x 1, 20.
 // Steps of GenASiS II Sec. 2.2:
@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(128) k64_synth_phi_few(const double *__restric
 
 cudaError_t launch_fp64_project(mp_mesh *m, const double *rho)
 {
-    if (m->fp.mom_on && m->fp.phi_on) return launch_fp64_tc_project(m, rho);
-    if (m->fp.mom_on) {
+    if (m->fp.proj_on) return launch_fp64_tc_project(m, rho);
+    if (m->fp.rows) {
         cudaEvent_t ev;
         prof_begin(m, "fp64_phi_project", &ev);
         const int threads = std::min(128, round_up(m->n_t, 32));
@@ -272,7 +272,7 @@ cudaError_t launch_fp64_theta(mp_mesh *m)
 {
     cudaEvent_t ev;
     prof_begin(m, "fp64_theta_contract", &ev);
-    if (m->fp.mom_on)
+    if (m->fp.rows)
         k64_theta_rows<<<dim3((m->n_r + kThRows / 2 - 1) / (kThRows / 2), (m->L + 1) * ((m->L + kThDeg) / kThDeg)), 32 * kThWarps, 0,
                          m->stream>>>(m->d_F64, m->d_Ith, m->d_A, m->n_r, m->n_t, m->L, m->KL, m->P, m->fp.ldJ,
                                       kFourPi * m->G);

@@ -1325,12 +1325,11 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-bool plan_fp64_tc(mp_mesh *m, bool far_moments)
+void plan_fp64_tc(mp_mesh *m, bool far_moments)
 {
     Fp64Plan &f = m->fp;
     f = Fp64Plan();
     f.ldJ = round_up(m->n_t, 4);
-    f.ldI = round_up(m->n_r, 4);
     // columns per pass over the density; the column m = 0 gets a block of its own where the
     // others fill blocks of 16 without it
     f.m0 = m->L > 0 && m->L % 8 == 0;
@@ -1338,13 +1337,12 @@ bool plan_fp64_tc(mp_mesh *m, bool far_moments)
     f.npass = (cols + kNtMax - 1) / kNtMax;
     f.pass_cols = (cols + f.npass - 1) / f.npass;
     if (f.npass > 1) f.pass_cols = std::min(kNtMax, ceil16(f.pass_cols));
-    if (m->L > 71 || m->R >= (1LL << 31) || !plan_expand(m->L + 1, f.th_x)) {
-        f = Fp64Plan();  // the CUDA-core path and its layouts
-        return false;
-    }
+    // 2 l_max terms in the chains of the phi synthesis, row indices in 32 bits
+    if (m->L > 71 || m->R >= (1LL << 31)) return;
     // below 16 azimuthal cells (axisymmetric meshes have one) a 16-wide K step is mostly padding
     // and the sums are short: CUDA cores
-    f.phi_on = m->n_p >= 16 && plan_contract(m->n_p, f.pass_cols, f.m0, f.ph_c) && plan_expand(m->P - 1, f.ph_x);
+    const bool few = m->n_p < 16;
+
     // Moments whose radial weights reach 1e150 (l_max = 48 over five decades of r): their squares
     // leave the float64 range, so neither they nor the differences of two solutions have a norm,
     // and equality is the one way to compare them.  They stay sums in the order of the CUDA-core
@@ -1361,9 +1359,21 @@ bool plan_fp64_tc(mp_mesh *m, bool far_moments)
         widest = std::max(widest, m->h_ph[k + 1] - m->h_ph[k]);
         narrowest = std::min(narrowest, m->h_ph[k + 1] - m->h_ph[k]);
     }
-    f.mom_on = !far_moments && (!f.phi_on || widest <= 2.0 * narrowest);
-    f.on = 1;
-    return true;
+    // Small meshes: a tensor-core kernel of this file takes 11 to 15 us for a single tile, where the
+    // CUDA-core ones take 6 and more by their products.  The two cross (both sides' times in
+    // us): projection with the theta contraction behind it at 0.6 M products (40 x 24 x 17 cells, l_max =
+    // 8: 21.5 against 19.6; 64 x 32 x 64, 2: 21.7 against 22.6), later where F's rows of polar cells
+    // are short (512 x 1 x 64, 16: 24.6 against 19.3); synthesis where the phi products and three
+    // times the theta products (uncoalesced) reach 6 M (64 x 32 x 64, 8: 24.1 against 20.1; 16: 26.6
+    // against 27.2); theta synthesis alone at 0.6 M (128 x 64 x 1, 2: 12.5 against 7.3; 8: 12.5
+    // against 15.8).
+    const double phi_products = (double)m->R * m->n_p * m->P, theta_products = (double)m->R * m->KL;
+    f.proj_on = !few && !far_moments && widest <= 2.0 * narrowest && phi_products >= (m->n_t >= 8 ? 0.6e6 : 4.8e6) &&
+                plan_contract(m->n_p, f.pass_cols, f.m0, f.ph_c);
+    f.rows = f.proj_on || (few && !far_moments);
+    f.on = (few ? theta_products >= 0.6e6 : phi_products + 3.0 * theta_products >= 6e6) && plan_expand(m->L + 1, f.th_x);
+    f.phi_on = f.on && !few && plan_expand(m->P - 1, f.ph_x);
+    if (f.on) f.ldI = round_up(m->n_r, 4);
 }
 
 size_t fp64_tc_arena(mp_mesh *m)
@@ -1381,14 +1391,14 @@ size_t fp64_tc_arena(mp_mesh *m)
     unsigned long long *ox = f.h_off.data(), *op = ox + f.off_ld;
     unsigned long long x = 0;
     const int n_blk = (m->n_t + kNtX - 1) / kNtX;
-    for (int mm = 0; mm <= L; ++mm) {
+    for (int mm = 0; mm <= L && f.on; ++mm) {
         ox[mm] = x;
         x += (unsigned long long)n_blk * ((L + 1 - mm + 15) / 16) * kRowsX * 32;
     }
     const unsigned long long pstep = (unsigned long long)f.ph_c.n_steps * f.ph_c.slot_b;
     for (int s = 0; s < f.npass; ++s) op[s] = s * pstep;
     f.o_tab_x = take(x);
-    f.o_tab_pc = take(f.phi_on && f.mom_on ? f.npass * pstep : 0);
+    f.o_tab_pc = take(f.proj_on ? f.npass * pstep : 0);
     f.o_tab_px = take(f.phi_on ? (size_t)((m->n_p + kNtX - 1) / kNtX) * std::max(1, (m->P - 1 + 15) / 16) * kRowsX * 32 : 0);
     f.o_off = take(f.h_off.size() * sizeof(unsigned long long));
     f.o_et_x = take((size_t)(L + 1) * round_up(m->n_t, kNtX) * 4);
@@ -1443,8 +1453,8 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
                     reinterpret_cast<int *>(f.arena + f.o_bound) + kind};
         k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t, n_sets);
     };
-    build(TAB_EXPAND_TH, f.o_tab_x, 0, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
-    if (f.phi_on && f.mom_on) build(TAB_PROJECT, f.o_tab_pc, 1, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
+    if (f.on) build(TAB_EXPAND_TH, f.o_tab_x, 0, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
+    if (f.proj_on) build(TAB_PROJECT, f.o_tab_pc, 1, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);
     if (f.phi_on) build(TAB_EXPAND_PH, f.o_tab_px, 2, f.o_et_px, round_up(m->n_p, kNtX), m->n_p, 1);
     // 227 KB of dynamic shared memory for the kernels of this file (per device)
     for (int vec = 0; vec < 2; ++vec)

@@ -68,9 +68,10 @@ struct Fp64Expand {
     int a_steps = 0, ns_b = 0, smem = 0, small = 0;
 };
 struct Fp64Plan {
-    int on = 0;      // theta synthesis (and the layouts G [n_r][P][ldJ], C [K_L][ldI])
-    int phi_on = 0;  // phi stages too
-    int mom_on = 0;  // the projection among them, and F as [n_r][P][ldJ] (else [R][P])
+    int proj_on = 0;  // the projection
+    int rows = 0;     // F as [n_r][P][ldJ], else [R][P]
+    int on = 0;       // the theta synthesis, and the layouts G [n_r][P][ldJ], C [K_L][ldI]
+    int phi_on = 0;   // the phi synthesis too
     int ldJ = 0, ldI = 0, npass = 1, pass_cols = 0, m0 = 0, off_ld = 0;
     Fp64Contract ph_c;
     Fp64Expand ph_x, th_x;
@@ -264,8 +265,7 @@ cudaError_t launch_fp64_synth(mp_mesh *m, double *phi);
 cudaError_t launch_fp64_moments_into(const mp_mesh *m, const double *rho, double *F, double *A);
 
 // steps (a1), (d1) and (d2) as exact integer slices on the tensor cores (F, G [n_r][P][ldJ], C [K_L][ldI])
-// (false: sizes out of its range, l_max > 71; far_moments: the moments stay on CUDA cores)
-bool plan_fp64_tc(mp_mesh *m, bool far_moments);
+void plan_fp64_tc(mp_mesh *m, bool far_moments);  // which steps run here (far_moments: not the projection)
 size_t fp64_tc_arena(mp_mesh *m);          // lays the tables out; bytes of the arena
 cudaError_t launch_fp64_tc_tables(mp_mesh *m);
 cudaError_t fp64_tc_bounds(mp_mesh *m);    // reads what the finished tables say about the accumulators
