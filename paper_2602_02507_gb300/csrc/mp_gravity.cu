@@ -33,8 +33,10 @@ namespace {
 
 // (a - b) w in integer instructions where that is exact work: a and b of one sign and within 2^9
 // of each other, as neighbouring cells of a potential are, subtract exactly as 62-bit integers;
-// the difference (33 bits or more of them) is normalised, multiplied by w's significand (64 x 64
-// -> the upper 64 bits) and rounded to nearest once.  False for anything else (zeros, denormals,
+// the difference is normalised, multiplied by w's significand (64 x 64 -> the upper 64 bits) and
+// rounded once, to nearest, ties away from zero (the float64 expression rounds the difference and
+// the product: the two agree within one unit in the last place).  No difference at all, everywhere
+// on an axis of symmetry, gives +0.  False for anything else (zero operands, denormals,
 // infinities, NaN, a sign change, results near the ends of the range), which takes the float64
 // pipe.  That pipe issues one warp's instruction every 64 cycles a scheduler here and bounded the
 // kernel with 12 a cell; three differences and their scalings on the integer pipe leave it 6.
@@ -53,8 +55,11 @@ __device__ __forceinline__ bool scaled_difference(double a, double b, const Grad
     const uint32_t sg = (uint32_t)((int)dh >> 31);
     uint32_t ul, uh;
     asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %4;" : "=r"(ul), "=r"(uh) : "r"(dl ^ sg), "r"(dh ^ sg), "r"(sg));
-    const int n = __clz((int)uh);
-    const uint32_t n1 = __funnelshift_l(ul, uh, n), n0 = ul << (n & 31);
+    // leading one to bit 63, from the lower word where the upper one is empty
+    const bool low = uh == 0;
+    uh = low ? ul : uh;
+    const int n5 = __clz((int)uh), n = low ? n5 + 32 : n5;
+    const uint32_t n1 = __funnelshift_l(low ? 0u : ul, uh, n5), n0 = low ? 0u : ul << (n5 & 31);
     const unsigned long long t = (unsigned long long)n1 * s.w0 + __umulhi(n0, s.w0);
     const unsigned long long v = (unsigned long long)n0 * s.w1 + (uint32_t)t;
     const unsigned long long p = (unsigned long long)n1 * s.w1 + (uint32_t)(t >> 32) + (uint32_t)(v >> 32);
@@ -66,12 +71,17 @@ __device__ __forceinline__ bool scaled_difference(double a, double b, const Grad
     asm("add.cc.u32 %0, %0, 0x200;\n\taddc.u32 %1, %1, 0;" : "+r"(pl), "+r"(ph));
     const int be = (em & 0x7FF) + s.we - 1022 - n + top;  // exponent field less one
     const uint32_t rl = __funnelshift_r(pl, ph, 10), rh = (ph >> 10) + ((uint32_t)be << 20);
-    g = __hiloint2double((int)(rh | ((ha ^ sg) & 0x80000000u)), (int)rl);
-    return (sa | sb) >= 0 && (unsigned)((em & 0x7FF) - 64) < 1983u && uh != 0 && (unsigned)be < 2045u;
+    const bool none = uh == 0;  // (rl is 0 then)
+    g = __hiloint2double(none ? 0 : (int)(rh | ((ha ^ sg) & 0x80000000u)), (int)rl);
+    return (sa | sb) >= 0 && (unsigned)((em & 0x7FF) - 64) < 1983u && (none || (unsigned)be < 2045u);
 }
 
-// (out of line: inlined, its instructions were issued for every cell and selected afterwards)
-__device__ __noinline__ double scaled_difference_f64(double a, double b, double w) { return (a - b) * w; }
+// The float64 form, out of line (inlined, its instructions were issued for every cell and selected
+// afterwards) and with loads of its own, so that nothing is kept for it.
+__device__ __noinline__ double scaled_difference_f64(const double *hi, const double *lo, const GradStencil *s)
+{
+    return (__ldg(hi) - __ldg(lo)) * s->w;
+}
 
 template <int V>
 __device__ __forceinline__ void load_cells(const double *p, double (&x)[V], bool stream)
@@ -95,10 +105,14 @@ __device__ __forceinline__ void store_cells(double *p, const double (&x)[V])
 }
 
 // V neighbouring azimuthal cells a thread: 2 where every row starts on a 16-byte boundary (half
-// the memory instructions, twice the loads in flight).  At 512 x 128 x 256, S and E: 381 us with
-// every operation on the float64 pipe; 294 with the differences on the integer pipe; 251 with
-// two cells a thread in blocks of 64 threads at 64 registers (260 in blocks of 128; 317 with
-// one cell; rows in a loop 296-301).  The float64 pipe's floor is now 163 us, HBM's 178.
+// the memory instructions, twice the loads in flight), in blocks of 64 threads (260 against 251 us in
+// blocks of 128, in the form of that time; rows in a loop 296).  An axis on which a cell of the warp
+// does not fit goes the float64 way by itself and loads its values again: kept for it, they cost
+// spills at the 64 registers that four blocks of 256 threads leave.  At 512 x 128 x 256, S and E: 381
+// us with every operation on the float64 pipe, 240 so, on any potential of one sign (with one test
+// for all three axes and differences below 33 bits left to the float64 form: 249, and 388 on
+// symmetric or flat ones, 310 on Phi of a split solve); 381 -> 287 with an odd number of azimuthal
+// cells (410 there).  Noise of both signs takes 388.  The float64 pipe's floor is 163 us, HBM's 178.
 template <int V>
 __global__ void __launch_bounds__(256, V == 2 ? 4 : 6) k_gravity(const double *__restrict__ phi, const double *__restrict__ rho,
                                                  const double *__restrict__ v, double *__restrict__ grad,
@@ -135,21 +149,22 @@ __global__ void __launch_bounds__(256, V == 2 ? 4 : 6) k_gravity(const double *_
             load_cells<V>(v + 2 * N + c, v2, true);
         }
         double g[3][V];
-        bool fits = true;
+        bool fits[3] = {true, true, true};
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-            fits &= scaled_difference(hi[0][e], lo[0][e], gr, g[0][e]);
-            fits &= scaled_difference(hi[1][e], lo[1][e], gt, g[1][e]);
-            fits &= scaled_difference(hi[2][e], lo[2][e], gp[e], g[2][e]);
+            fits[0] &= scaled_difference(hi[0][e], lo[0][e], gr, g[0][e]);
+            fits[1] &= scaled_difference(hi[1][e], lo[1][e], gt, g[1][e]);
+            fits[2] &= scaled_difference(hi[2][e], lo[2][e], gp[e], g[2][e]);
             nr[e] = -nr[e];
         }
-        if (!fits) {
 #pragma unroll
-            for (int e = 0; e < V; ++e) {
-                g[0][e] = scaled_difference_f64(hi[0][e], lo[0][e], gr.w);
-                g[1][e] = scaled_difference_f64(hi[1][e], lo[1][e], gt.w);
-                g[2][e] = scaled_difference_f64(hi[2][e], lo[2][e], gp[e].w);
-            }
+        for (int a = 0; a < 3; ++a) {
+            if (fits[a]) continue;
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+                g[a][e] = a == 0 ? scaled_difference_f64(p_rhi + k + e, p_rlo + k + e, st + i)
+                          : a == 1 ? scaled_difference_f64(p_thi + k + e, p_tlo + k + e, st + n_r + j)
+                                   : scaled_difference_f64(p_row + sp[k + e].hi, p_row + sp[k + e].lo, sp + k + e);
         }
         if (grad) {
 #pragma unroll

@@ -1,0 +1,77 @@
+"""The gravitational source terms on potentials with equal or nearly equal neighbours: the same
+values as the float64 expression, at the rate of any other potential."""
+import numpy as np
+import pytest
+
+from oracle import gravity as OG
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import __graft_entry__ as g
+    g.build()
+
+
+def _edges(shape):
+    return (np.linspace(0.5, 1.5, shape[0] + 1) ** 2, np.linspace(0.0, np.pi, shape[1] + 1),
+            np.linspace(0.0, 2.0 * np.pi, shape[2] + 1))
+
+
+@pytest.mark.parametrize("shape", [(5, 4, 33), (4, 3, 64), (3, 5, 66), (2, 2, 190), (6, 1, 70)])
+def test_differences_of_every_length(shape):
+    """Neighbours that differ from the 5th to the 53rd bit, or not at all, of either sign: within one
+    unit in the last place of (Phi[hi] - Phi[lo]) * w, and +0 where there is no difference."""
+    import torch
+    from paper_2602_02507_gb300 import multipole as mpl
+    rng = np.random.default_rng(8)
+    phi = 1.5 + 2.0 ** -rng.uniform(5, 54, shape) * rng.choice([-1.0, 0.0, 1.0], shape)
+    phi *= rng.choice([-1.0, 1.0]) * 1e19
+    r, th, ph = _edges(shape)
+    grad = torch.empty(3 * phi.size, dtype=torch.float64, device="cuda")
+    with mpl.Mesh(r, th, ph, 2, 1.0, precision="fp64") as mesh:
+        mesh.gravity_sources(phi=torch.from_numpy(phi).cuda().reshape(-1),
+                             rho=torch.ones(phi.size, dtype=torch.float64, device="cuda"), grad=grad)
+        mesh.synchronize()
+    got = grad.cpu().numpy().reshape((3,) + shape)
+    for a, (edges, wraps) in enumerate(((r, False), (th, False), (ph, True))):
+        lo, hi, dx = OG.stencil(edges, wraps)
+        w = np.where(dx != 0.0, 1.0 / np.where(dx != 0.0, dx, 1.0), 0.0)
+        want = (phi.take(hi, axis=a) - phi.take(lo, axis=a)) * w.reshape([-1 if d == a else 1 for d in range(3)])
+        assert np.all(np.abs(got[a] - want) <= 2.3e-16 * np.abs(want))
+        assert np.array_equal(np.signbit(got[a]), np.signbit(want))
+
+
+def test_symmetric_potentials_run_at_the_same_rate():
+    """Phi(r), Phi(r, theta), a flat one and a float32 one take at most 1.2 times a general one's
+    time (they took 1.56 times it while equal neighbours left the integer form)."""
+    import torch
+    from paper_2602_02507_gb300 import multipole as mpl
+    shape = (512, 128, 256)
+    r, th, ph = _edges(shape)
+    rc, tc, pc = (torch.from_numpy(0.5 * (e[1:] + e[:-1])).cuda() for e in (r, th, ph))
+    angular = torch.sin(tc)[:, None] * torch.cos(pc)[None, :]
+    radial = (-1e19 / (1.0 + rc * rc).sqrt())[:, None, None].expand(shape).contiguous()
+    kinds = {"general": radial * (1.0 + 1e-2 * angular), "spherical": radial,
+             "axisymmetric": radial * (1.0 + 1e-2 * torch.cos(tc)[None, :, None]),
+             "flat": radial * (1.0 + 1e-9 * angular), "float32": (radial * (1.0 + 1e-6 * angular)).float().double()}
+    rho, v = torch.rand(shape, dtype=torch.float64, device="cuda"), torch.randn((3,) + shape, dtype=torch.float64, device="cuda")
+    S, E = torch.empty_like(v), torch.empty_like(rho)
+    times = {}
+    with mpl.Mesh(r, th, ph, 2, 1.0, precision="fp64") as mesh:
+        for kind, phi in kinds.items():
+            phi, runs = phi.contiguous(), []
+            for _ in range(6):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                for _ in range(10):
+                    mesh.gravity_sources(phi=phi, rho=rho, v=v, S=S, E=E)
+                b.record()
+                torch.cuda.synchronize()
+                runs.append(a.elapsed_time(b))
+            times[kind] = min(runs)
+    assert max(times.values()) <= 1.2 * times["general"], times
