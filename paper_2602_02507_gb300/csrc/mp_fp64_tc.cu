@@ -332,7 +332,7 @@ __device__ __forceinline__ double tab_value(const TabParams &t, int set, int n, 
 // then [digit of A][octet][16 rows][8]}; expand tables are blocks of 32
 // columns, [block][K step][octet][7 x 32][8].  Cells past K are never written (the tables
 // start as zeros).
-__global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t, int n_sets)
+__global__ void __launch_bounds__(128) k64_digit_tables(const TabParams t)
 {
     const int set = blockIdx.y, lane = threadIdx.x & 31;
     const bool own0 = t.kind == TAB_PROJECT && t.m0 && set == 0;
@@ -1451,7 +1451,7 @@ cudaError_t launch_fp64_tc_tables(mp_mesh *m)
         TabParams t{m->d_Ith, m->d_Iph, m->d_Iphc, m->d_dmu, f.arena + tab, fp64_off(m, off),
                     reinterpret_cast<int *>(f.arena + et), kind, m->n_t, m->n_p, L, m->P, f.pass_cols, f.m0, et_ld,
                     reinterpret_cast<int *>(f.arena + f.o_bound) + kind};
-        k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t, n_sets);
+        k64_digit_tables<<<dim3((n_max + 3) / 4, n_sets), 128, 0, m->stream>>>(t);
     };
     if (f.on) build(TAB_EXPAND_TH, f.o_tab_x, 0, f.o_et_x, round_up(m->n_t, kNtX), m->n_t, L + 1);
     if (f.proj_on) build(TAB_PROJECT, f.o_tab_pc, 1, f.o_et_pc, kEtLd, f.pass_cols + f.m0, f.npass);

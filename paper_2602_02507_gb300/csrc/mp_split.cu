@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(kProjThreads, 1) k_proj_tc(const __grid_consta
 #pragma unroll
                     for (int pi = 0; pi < NPROD; ++pi) {
                         umma_warp(d_tmem, a_lo + (prod_a(pi) * A_TERM_BYTES + ks * 256) / 16, a_hi,
-                                       b_lo + (prod_b(pi) * b_term + ks * 256) / 16, b_hi, idesc,
-                                       (it >= nacc) || ((ks | pi) != 0), leader);
+                                  b_lo + (prod_b(pi) * b_term + ks * 256) / 16, b_hi, idesc,
+                                  (it >= nacc) || ((ks | pi) != 0), leader);
                     }
                 }
                 umma_commit_warp(smem_u32(&o_empty[ro.idx]), leader);
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(synth::THREADS, 1)
 #pragma unroll
                     for (int pi = 0; pi < NPROD; ++pi) {
                         umma_warp(d_tmem, a_lo + prod_a(pi) * (a_term_bytes / 16), a_hi,
-                                       b_lo + (uint32_t)(prod_b(pi) * NC * 2), b_hi, idesc, (kk | pi) != 0, leader);
+                                  b_lo + (uint32_t)(prod_b(pi) * NC * 2), b_hi, idesc, (kk | pi) != 0, leader);
                     }
                     if (!prm.b_resident) {
                         umma_commit_warp(smem_u32(&b_empty[rb.idx]), leader);

@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(thc::THREADS, 1) k_theta_tc(const __grid_const
 #pragma unroll
                     for (int pi = 0; pi < NPROD; ++pi) {
                         umma_warp(d_tmem, a_lo + (prod_a(pi) * A_TERM_BYTES + ks * 256) / 16, a_hi,
-                                       t_lo + (prod_b(pi) * b_term + ks * 256) / 16, t_hi, idesc,
-                                       (c >= nacc) || ((ks | pi) != 0), leader);
+                                  t_lo + (prod_b(pi) * b_term + ks * 256) / 16, t_hi, idesc,
+                                  (c >= nacc) || ((ks | pi) != 0), leader);
                     }
                 }
                 umma_commit_warp(smem_u32(&o_empty[ro.idx]), leader);
@@ -426,8 +426,8 @@ __global__ void __launch_bounds__(gsc::THREADS, 1) k_gsynth_tc(const GsynthTcPar
 #pragma unroll
                         for (int pi = 0; pi < NPROD; ++pi) {
                             umma_warp(d_tmem, t_lo + (prod_b(pi) * T_TERM_BYTES + ks * 256) / 16, d_hi,
-                                           c_lo + (prod_a(pi) * c_term + ks * 256) / 16, d_hi, idesc,
-                                           (kc | ks | pi) != 0, leader);
+                                      c_lo + (prod_a(pi) * c_term + ks * 256) / 16, d_hi, idesc,
+                                      (kc | ks | pi) != 0, leader);
                         }
                     }
                     umma_commit_warp(smem_u32(&s_empty[rs.idx]), leader);

@@ -174,7 +174,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // x 180, l_max = 21, bf16x6), 3410 -> 3352 us (2048 x 512 x 1024, l_max = 64); scan and projection before the m = 0 kernels 470 -> 458 us (1024 x 256 x
 // 512, l_max = 32).  The other way round, projection before k32_theta_pipe: 85.1 without,
 // 84.2 with (512 x 128 x 256, l_max = 16).  The float64 tensor-core kernels do not
-// trigger either: 225 -> 204 us at 512 x 128 x 256 with moments, 130 -> 117 at 353 x 96 x 192.
+// trigger either: 225 -> 204 us at 512 x 128 x 256 with moments, 130 -> 117 at 353 x 96 x 192 (with the
+// theta contraction among them).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
 // ---------------------------------------------------------------- TMA / bulk copies
@@ -267,11 +268,6 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, 
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 
-__device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void *src, uint32_t src_bytes)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 template <int N>
@@ -326,7 +322,7 @@ __device__ __forceinline__ uint32_t elect_one()
 // word): only the low words change from one MMA to the next, and a lone warp's instructions are
 // what bounds a stream of small MMAs.
 __device__ __forceinline__ void umma_warp(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
-                                              uint32_t idesc, uint32_t accumulate, uint32_t leader)
+                                          uint32_t idesc, uint32_t accumulate, uint32_t leader)
 {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
@@ -446,8 +442,6 @@ __device__ __forceinline__ float f64w_to_f32(uint32_t lo, uint32_t hi)
     bits = (e >= 255) ? 0x7F800000u : bits;
     return __uint_as_float(bits | sign);
 }
-
-__device__ __forceinline__ bool f64w_nonfinite(uint32_t hi) { return (hi & 0x7FF00000u) == 0x7FF00000u; }
 
 // Same conversion, cheaper, for values that are split into bf16 terms next
 // (which keep about 16 significant bits): the float32 exponent field is the low
