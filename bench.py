@@ -558,7 +558,7 @@ def batch_workload(args, stream, with_oracle, hbm_peak):
     return out
 
 
-def beside_solve(stream, hbm_peak, rates, steps):
+def beside_solve(stream, hbm_peak, steps):
     """Gravitational source terms (Sec. 3) of a presupernova solve's potential and the
     coarsening-block averaging on the paper's N_theta = 256 mesh: float64 kernels bound by
     the float64 pipe, timed beside (not inside) the solve."""
@@ -589,12 +589,9 @@ def beside_solve(stream, hbm_peak, rates, steps):
     e1.record(stream)
     torch.cuda.synchronize()
     g_us = e0.elapsed_time(e1) / kg * 1e3
-    fp64_instr_peak = rates["fp64_tflops"] * 1e12 / 2.0  # one FMA instruction = 2 flops
     gravity = {"kernel": "gravity_sources", "workload": WORKLOADS["presn"], "launches": kg, "avg_launch_us": g_us,
                "algorithmic_bytes_per_cell": 72, "hbm_gbs": 72 * cells / g_us / 1e3,
                "hbm_frac": 72 * cells / g_us / 1e3 / hbm_peak,
-               "fp64_instr_per_cell": 6, "fp64_instr_per_s": 6 * cells / (g_us * 1e-6),
-               "fp64_frac": 6 * cells / (g_us * 1e-6) / fp64_instr_peak, "bound": "issue",
                "note": "S [3] and E from Phi, rho, v [3]: 9 float64 reads + 4 writes per cell"}
     mesh.close()
     del gvel, gS, gE, rho
@@ -795,7 +792,7 @@ def run_ours(args):
             line_extra["other_workloads"][name] = side_workload(name, args, stream, with_oracle, hbm_peak)
         log("batch workload ...")
         line_extra["other_workloads"]["batch"] = batch_workload(args, stream, with_oracle, hbm_peak)
-        gravity, coarsen = beside_solve(stream, hbm_peak, rates, args.steps)
+        gravity, coarsen = beside_solve(stream, hbm_peak, args.steps)
         line_extra["gravity_sources"] = gravity
         line_extra["coarsen_blocks"] = coarsen
 
