@@ -66,7 +66,7 @@ SPLIT_PRECISION = "bf16x3"
 # those two counters alone (one pass, as on a 128-shell cut first): 8.60 GB of density read
 # and 0.49 GB of F written back (F, 545 MB, outgrows L2 at this size; on the cut it stays).
 NCU_TRAFFIC = {
-    ("large", "split_phi_project_tc"): (8.603e9 + 487.8e6, "mp_split.cu", "b39e7ee298fb1997bd290f7c46aadda95b9b1c26"),
+    ("large", "split_phi_project_tc"): (8.603e9 + 487.8e6, "mp_split.cu", "46fc7c4f9f40f91d705b8ee9eedc69ca621b5d49"),
 }
 KERNEL_HEADERS = ("ptx.cuh", "mp_internal.h", "mp_errors.h")
 

@@ -41,9 +41,9 @@
 // right, so a K step of 16 takes seven MMAs for its 28 products and reads A seven times
 // instead of 28 (with one MMA per pair the shared-memory reads of A would bound it).
 //
-// What bounds them: not the tensor core (35 % of the time in the long contraction, 49 % in the
-// long expansion at 1024 x 256 x 512 cells, l_max = 32) nor HBM (24 and 34 %), but the integer
-// instructions that split and rejoin the operands (half the rate of float32's: their pipe is 50 and
+// What bounds them: not the tensor core (33 % of the time in the long contraction, 49 % in the
+// long expansion at 1024 x 256 x 512 cells, l_max = 32) nor HBM (22 and 34 %), but the integer
+// instructions that split and rejoin the operands (half the rate of float32's: their pipe is 53 and
 // 58 % busy) and the hand-offs between the warps that issue them.  Measured there against float64
 // on CUDA cores: (a1) 29.5 ms -> 691 us, (d1) 2143 -> 66 us, (d2) 13.9 ms -> 427 us; at 512 x 128 x
 // 256, l_max = 16: 1918 -> 91, 200 -> 16, 891 -> 69 us.  (Rounding the operands instead of

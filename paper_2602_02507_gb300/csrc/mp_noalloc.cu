@@ -5,7 +5,7 @@
 // mid-run can fail or stall), or plug-ins embedded in a host application that
 // owns every device allocation and forbids them to call cudaMalloc.
 // mp_moments_noalloc serves them: it computes the angular moments of step (a) in
-// float64 into the caller's buffer with the float64 path's own kernels, and their
+// float64 into the caller's buffer with the float64 path's CUDA-core kernels, and their
 // one intermediate array -- the phi projection F[row][p] -- lives in a fixed
 // file-scope device array instead of memory obtained from cudaMalloc.  A
 // non-finite density sets the mesh's device error word, which the next
@@ -76,7 +76,7 @@ extern "C" MP_API mp_status mp_moments_noalloc(const mp_mesh *mesh, const double
     double *F = nullptr;
     mp_status st = scratch_address(mesh->device, &F);
     if (st == MP_OK) {
-        // the float64 path's own projection and theta contraction, with the fixed array as
+        // the float64 path's CUDA-core projection and theta contraction, with the fixed array as
         // their workspace
         const cudaError_t e = launch_fp64_moments_into(mesh, rho_dev, F, ang_dev);
         if (e != cudaSuccess) st = set_error(MP_ERR_CUDA, "mp_moments_noalloc launch: %s", cudaGetErrorString(e));
