@@ -113,7 +113,10 @@ __device__ __forceinline__ void store_cells(double *p, const double (&x)[V])
 // for all three axes and differences below 33 bits left to the float64 form: 249, and 388 on
 // symmetric or flat ones, 310 on Phi of a split solve); 381 -> 287 with an odd number of azimuthal
 // cells (410 there).  Noise of both signs takes 388.  The float64 pipe's floor is 163 us, HBM's 178.
-template <int V>
+// INT false: every difference on the float64 pipe, for gradients alone with one cell a thread (six
+// float64 operations a cell in all: 53 us against 58 at 512 x 128 x 40; two cells a thread are faster in
+// integers there too, 205 -> 191 at 512 x 128 x 256).
+template <int V, bool INT>
 __global__ void __launch_bounds__(256, V == 2 ? 4 : 6) k_gravity(const double *__restrict__ phi, const double *__restrict__ rho,
                                                  const double *__restrict__ v, double *__restrict__ grad,
                                                  double *__restrict__ S, double *__restrict__ E,
@@ -152,10 +155,16 @@ __global__ void __launch_bounds__(256, V == 2 ? 4 : 6) k_gravity(const double *_
         bool fits[3] = {true, true, true};
 #pragma unroll
         for (int e = 0; e < V; ++e) {
+            nr[e] = -nr[e];
+            if constexpr (!INT) {
+                g[0][e] = (hi[0][e] - lo[0][e]) * gr.w;
+                g[1][e] = (hi[1][e] - lo[1][e]) * gt.w;
+                g[2][e] = (hi[2][e] - lo[2][e]) * gp[e].w;
+                continue;
+            }
             fits[0] &= scaled_difference(hi[0][e], lo[0][e], gr, g[0][e]);
             fits[1] &= scaled_difference(hi[1][e], lo[1][e], gt, g[1][e]);
             fits[2] &= scaled_difference(hi[2][e], lo[2][e], gp[e], g[2][e]);
-            nr[e] = -nr[e];
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -298,7 +307,7 @@ cudaError_t launch_gravity(mp_mesh *m, const double *phi, const double *rho, con
                            ((bits(phi) | bits(rho) | bits(v) | bits(grad) | bits(S) | bits(E)) & 15) == 0;
         const int cells = pairs ? m->n_p / 2 : m->n_p;
         const int threads = std::min(pairs ? 64 : 256, 32 * ((cells + 31) / 32));
-        auto kern = pairs ? k_gravity<2> : k_gravity<1>;
+        auto kern = pairs ? k_gravity<2, true> : S || E ? k_gravity<1, true> : k_gravity<1, false>;
         kern<<<(unsigned)m->R, threads, 0, m->stream>>>(phi, rho, v, grad, S, E, m->d_gst, m->n_r, m->n_t, m->n_p, m->N);
     }
     prof_end(m, "gravity_sources", ev);

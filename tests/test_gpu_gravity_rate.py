@@ -75,3 +75,24 @@ def test_symmetric_potentials_run_at_the_same_rate():
                 runs.append(a.elapsed_time(b))
             times[kind] = min(runs)
     assert max(times.values()) <= 1.2 * times["general"], times
+
+
+@pytest.mark.parametrize("shape", [(6, 5, 33), (5, 7, 40), (4, 3, 141)])
+def test_gradients_alone_with_one_cell_a_thread_are_the_float64_expression(shape):
+    """Six float64 operations a cell leave nothing to gain from the integer form: odd or few
+    azimuthal cells take the expression itself, bit for bit."""
+    import torch
+    from paper_2602_02507_gb300 import multipole as mpl
+    phi = -1.0 - np.random.default_rng(9).random(shape)
+    r, th, ph = _edges(shape)
+    grad = torch.empty(3 * phi.size, dtype=torch.float64, device="cuda")
+    with mpl.Mesh(r, th, ph, 2, 1.0, precision="fp64") as mesh:
+        mesh.gravity_sources(phi=torch.from_numpy(phi).cuda().reshape(-1),
+                             rho=torch.ones(phi.size, dtype=torch.float64, device="cuda"), grad=grad)
+        mesh.synchronize()
+    got = grad.cpu().numpy().reshape((3,) + shape)
+    for a, (edges, wraps) in enumerate(((r, False), (th, False), (ph, True))):
+        lo, hi, dx = OG.stencil(edges, wraps)
+        w = np.where(dx != 0.0, 1.0 / np.where(dx != 0.0, dx, 1.0), 0.0)
+        want = (phi.take(hi, axis=a) - phi.take(lo, axis=a)) * w.reshape([-1 if d == a else 1 for d in range(3)])
+        assert np.array_equal(got[a], want)
