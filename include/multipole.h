@@ -83,9 +83,9 @@ typedef enum {
     MP_PREC_FP64 = 0,   /* float64 throughout, or its accuracy: the theta part of the       */
                         /* moments and the recurrences are float64 sums; the phi projection */
                         /* and the synthesis of Phi may (l_max <= 71) be exact sums of      */
-                        /* 55-bit fixed-point operands on the tensor cores, off by at most  */
-                        /* about K 2^-54 x (largest value of the row) x (largest of the     */
-                        /* table's column) for K terms                                      */
+                        /* 55-bit fixed-point operands on the tensor cores, off by about    */
+                        /* sqrt(K) 2^-55 (at most K 2^-51) x (largest value of the row) x   */
+                        /* (largest of the table's column) for K terms                      */
     MP_PREC_BF16X3 = 1, /* angular contractions as split-bf16 tensor-core GEMMs,     */
                         /* density deviations in 2 bf16 terms, tables in 3           */
     MP_PREC_BF16X6 = 2  /* as BF16X3 with 3 bf16 terms on both operands              */

@@ -17,9 +17,10 @@
 // instructions (ldexp, on the float64 pipe, for results outside the normal range).
 //
 // Accuracy.  The operands are fixed-point: a value 2^k below its row's (or table column's) maximum
-// keeps 55 - k bits.  A result of K terms is off by at most about K 2^-54 x (row maximum) x (column
-// maximum), whether or not the two maxima meet at one index, where a float64 sum is off by a
-// multiple of 2^-53 of the sum of its terms' magnitudes.  The steps below can afford that: the
+// keeps 55 - k bits.  A result of K terms is off by at most K 2^-51 x (row maximum) x (column
+// maximum), and since roundings and left-out digits have either sign by about sqrt(K) 2^-55 of it (K
+// 2^-56 where all small cells of a row are equal), whether or not the two maxima meet at one index.
+// A float64 sum is off by a multiple of 2^-53 of the sum of its terms' magnitudes.  The steps below can afford that: the
 // azimuthal tables are of one size along a row of cells (a factor of two in their widths is let in)
 // and themselves off by the rounding of m phi, 2^-53 m phi of their maximum; and the synthesis delivers Phi alone, whose sum over the
 // orders is of the size of the row maxima (errors stay at 2^-53 of the largest |Phi| of the
